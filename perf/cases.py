@@ -348,3 +348,89 @@ def tolerance(case):
         return {"rel": 1e-3, "max": 1e-2, "differ": 0.0} if case["temperature"] > 0 else {"rel": 1e-4, "max": 4e-4, "differ": 0.0}
     # keys and values of the last layer: 0.25 %, at most 1.2 % of the root mean square
     return {"rel": 0.01, "max": 0.05, "differ": 0.0}
+
+
+# ----------------------------------------------------------------------------- the same in 64 bits
+def _forward64(shape, w, ids, segments):
+    """The model over whole sequences in 64-bit floats: ids[b] [n], segments[b] [n] ascending; a row sees the rows of its own
+    and earlier segments.  Returns the residual streams after the last layer and the last layer's keys and values [heads, n, d_head]."""
+    f64 = torch.float64
+    dh, hq, hkv, half = shape.d_head, shape.n_q_heads, shape.n_kv_heads, shape.d_head // 2
+    cut = [len(i) for i in ids]
+    x = w["tok_emb"][torch.cat(ids).long()].to(f64)
+    inv = torch.tensor([float(shape.rope_theta) ** (-2.0 * k / dh) for k in range(half)], dtype=f64, device="cuda")
+    ang = torch.cat([torch.arange(n, dtype=f64, device="cuda") for n in cut])[:, None] * inv
+    cos, sin = ang.cos()[:, None], ang.sin()[:, None]
+
+    def normed(v):
+        return v * torch.rsqrt(v.pow(2).mean(1, keepdim=True) + shape.rms_eps)
+
+    def times(v, m):
+        return v @ m.to(f64).t()
+
+    def turned(v):
+        a, b = v[..., :half], v[..., half:]
+        return torch.cat([a * cos - b * sin, b * cos + a * sin], -1)
+
+    kv = None
+    for m in w["layers"]:
+        h = normed(x)
+        q = turned(times(h, m["wq"]).view(-1, hq, dh))
+        k = turned(times(h, m["wk"]).view(-1, hkv, dh))
+        v = times(h, m["wv"]).view(-1, hkv, dh)
+        kv = [(a.transpose(0, 1), b.transpose(0, 1)) for a, b in zip(k.split(cut), v.split(cut))]
+        o = []
+        for qb, (kb, vb), seg in zip(q.split(cut), kv, segments):
+            hidden = seg[None, :] > seg[:, None]
+            heads = []
+            for g in range(hkv):
+                per = hq // hkv
+                sc = qb[:, g * per:(g + 1) * per].transpose(0, 1) @ kb[g].t() / math.sqrt(dh)
+                heads.append(sc.masked_fill_(hidden, -math.inf).softmax(-1) @ vb[g])
+            o.append(torch.cat(heads).transpose(0, 1).reshape(len(seg), hq * dh))
+        x = x + times(torch.cat(o), m["wo"])
+        h = normed(x)
+        x = x + times(torch.nn.functional.silu(times(h, m["w_gate"])) * times(h, m["w_up"]), m["w_down"])
+    return normed(x).split(cut), kv
+
+
+def exact(case, seed):
+    """What `run` returns, in 64 bits: keys and values, confidences and entropies (the tokens are whole numbers)."""
+    if case["kind"] == "trajectory":
+        return None
+    shape, lens, bs, block = SHAPES[case["model"]], _lengths(case), case["bs"], case["block"]
+    gen = torch.Generator("cuda")
+    gen.manual_seed(seed + 1)
+    prompts = torch.randint(0, shape.vocab - 2, (bs, case["p_max"]), device="cuda", generator=gen, dtype=torch.int32)
+    ids = [prompts[b, :n] for b, n in enumerate(lens)]
+    segments = [torch.zeros(n, dtype=torch.int64, device="cuda") for n in lens]
+    w = _weights(shape, seed, case["jump"])
+    if case["kind"] == "step":
+        known = 1 + seed % case["jump"]
+        rows = torch.full((bs, block), shape.mask_id, dtype=torch.int32, device="cuda")
+        rows[:, :known] = torch.randint(0, shape.vocab - 2, (bs, known), device="cuda", generator=gen, dtype=torch.int32)
+        x, _ = _forward64(shape, w, [torch.cat([a, b]) for a, b in zip(ids, rows)], [torch.cat([s, torch.ones_like(s[:1]).expand(block)]) for s in segments])
+        head = w["lm_head"].to(torch.float64)
+        conf, entropy = [], []
+        for v in x:
+            logits = v[-block:] @ head.t()
+            logits[:, shape.mask_id] = -math.inf
+            p = logits.softmax(-1)
+            conf.append(p.max(-1).values)
+            entropy.append(torch.special.entr(p).sum(-1))
+        return None, None, None, None, None, (torch.cat(conf) if case["temperature"] == 0 else None), torch.cat(entropy)
+    if case["gen"]:
+        # the response copies the token `jump` positions back; a position sees the prompt, the blocks before its own and its own
+        # (a refresh makes one segment of what is stored by then)
+        joined = 0
+        if case["refresh"]:
+            joined = (case["gen"] // block - 1) // case["refresh"] * case["refresh"]
+        after = torch.arange(case["gen"], device="cuda") // block + 1
+        after[:joined * block] = 0
+        for b in range(bs):
+            last = ids[b][-case["jump"]:]
+            ids[b] = torch.cat([ids[b], last.repeat(-(-case["gen"] // case["jump"]))[:case["gen"]]])
+            segments[b] = torch.cat([segments[b], after])
+    _, kv = _forward64(shape, w, ids, segments)
+    stored = [torch.stack(pair) for pair in kv]
+    return stored if not case["gen"] else [None, None] + stored
