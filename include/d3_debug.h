@@ -51,6 +51,8 @@ typedef struct d3_tuning {
                                of a pair fit one 128-row tile, whatever the number of pairs */
   int32_t cta_pairs;        /* matmuls of more than 128 rows on tiled weights run 256 x 256 tiles on pairs of CTAs that share
                                one MMA (cta_group::2, gemm_pair_kernel): -1 = when the shape allows (default), 0 never */
+  int32_t k_cut_pairs;      /* matmuls of decode-sized forwards on resident CTA pairs with the tiles of an incomplete wave cut
+                               along K (gemm_sk_kernel): -1 = by row count (default), 0 never, 1 wherever the shape allows */
 } d3_tuning;
 void d3_tuning_defaults(d3_tuning *t);
 int d3_set_tuning(d3_ctx *ctx, const d3_tuning *t);

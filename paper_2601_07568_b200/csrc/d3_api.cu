@@ -23,6 +23,7 @@
 #include "gemm_simt.cuh"
 #include "gemm_tc.cuh"
 #include "gemm_pair.cuh"
+#include "gemm_sk.cuh"
 #include "gemm_xt.cuh"
 #include "small_kernels.cuh"
 
@@ -124,6 +125,10 @@ struct d3_ctx {
   int live_rps = 0, live_rows = 0;    // (padded prompts): the pair kernel passes over row tiles without a live row
   int tune_cta_pairs = -1;      // wide matmuls on CTA pairs (cta_group::2): -1 when the shape allows, 0 never
   int pair_clusters = 0;        // CTA pairs of gemm_pair_kernel resident at once (asked once)
+  int tune_sk = -1;             // decode matmuls with K-cut tiles on resident CTA pairs (gemm_sk.cuh): -1 by rule, 0 never, 1 wherever the shape allows
+  int sk_pairs = 0;             // CTA pairs of gemm_sk_kernel resident at once (asked once)
+  unsigned int* sk_sync = nullptr;  // counters of a forward's gemm_sk launches (arrivals per cut tile, borders)
+  size_t sk_sync_cap = 0, sk_sync_used = 0;
   int tune_xt = -1;             // 129..256-row matmuls with weights as the 128-row operand: -1 when the shape allows, 0 never
   unsigned int* chain_sync = nullptr;  // [operators of the program] border counters of a forward's chain launches
   void* chain_prog = nullptr;          // the forward's operators (tc::ChainOp) on the device
@@ -967,8 +972,116 @@ int run_linear_pair(d3_ctx* c, const void* X, const void* W, int M, int N, int K
   return fail(c, D3_ERR_INVALID_ARG, "unknown epilogue");
 }
 
+// ---- matmuls with K-cut tiles on resident CTA pairs (gemm_sk.cuh)
+constexpr int SK_MAX_BORDERS = tc::SK_MAX_OPS;
+constexpr int SK_OP_COUNTERS = 256;  // counters set aside per matmul: two per cut tile (fewer than the pairs, at most 74), borders
+
+bool sk_shape_ok(int N, int K) {
+  return N % 256 == 0 && K % 64 == 0 && static_cast<long long>(N / 128) * (K / 64) * 128 < (1ll << 31);
+}
+// Before the first launch of a forward: room for the counters of `n_ops` matmuls, all zero.
+int sk_begin(d3_ctx* c, int n_ops) {
+  const size_t need = static_cast<size_t>(n_ops) * SK_OP_COUNTERS;
+  if (need > c->sk_sync_cap) return fail(c, D3_ERR_SHAPE, "more matmuls in a forward than counters");
+  CUDA_TRY(c, cudaMemsetAsync(c->sk_sync, 0, need * sizeof(unsigned int), c->stream));
+  c->sk_sync_used = 0;
+  return D3_OK;
+}
+struct SkMatmul {
+  const void *x, *w;
+  int N, K, epi;
+  EpiParams ep;
+  const QkvExtra* qx;
+};
+// One launch over `n` matmuls that follow one another (n <= SK_MAX_OPS), all over the same M rows.
+int run_sk(d3_ctx* c, const SkMatmul* mm, int n, int M) {
+  tc::SkParams p{};
+  p.n_ops = n;
+  p.M = M;
+  p.tok_tiles = (M + 255) / 256;
+  p.tok_n = ((M + p.tok_tiles - 1) / p.tok_tiles + 31) / 32 * 32;
+  const size_t stage_bytes = tc::SK_W_BYTES + static_cast<size_t>(p.tok_n) * 64;
+  p.stages = static_cast<int>(static_cast<size_t>(204 * 1024) / stage_bytes);
+  p.stages = std::min(p.stages, 16);
+  const size_t smem = tc::gemm_sk_smem_bytes(p.tok_n, p.stages);
+  cudaLaunchConfig_t cfg{};
+  cfg.blockDim = dim3(tc::SK_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = c->stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (c->sk_pairs == 0) {
+    CUDA_TRY(c, cudaFuncSetAttribute(tc::gemm_sk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 222 * 1024));
+    cfg.gridDim = dim3(static_cast<unsigned>(c->n_sms & ~1));
+    cfg.dynamicSmemBytes = 222 * 1024;
+    int n_cl = 0;
+    CUDA_TRY(c, cudaOccupancyMaxActiveClusters(&n_cl, tc::gemm_sk_kernel, &cfg));
+    c->sk_pairs = std::max(1, std::min(n_cl, c->n_sms / 2));
+    cfg.dynamicSmemBytes = smem;
+  }
+  const int P = c->sk_pairs;
+  if (static_cast<size_t>(P) * 6 * p.tok_n * 128 > c->partial_slots * 128 * 128) return fail(c, D3_ERR_SHAPE, "partial tiles exceed the workspace");
+  p.partial = c->partial;
+  p.error_word = c->error_word;
+  p.skip_flag = c->skip_flag;
+  p.rope_cos = c->rope_cos; p.rope_sin = c->rope_sin;
+  p.n_q_heads = c->cfg.n_q_heads; p.n_kv_heads = c->cfg.n_kv_heads; p.max_seq = c->cfg.max_seq;
+  p.rows_per_seq = 1;
+  if (c->sk_sync_used + static_cast<size_t>(n) * SK_OP_COUNTERS > c->sk_sync_cap) return fail(c, D3_ERR_SHAPE, "more matmuls in a forward than counters");
+  unsigned int* counters = c->sk_sync + c->sk_sync_used;
+  c->sk_sync_used += static_cast<size_t>(n) * SK_OP_COUNTERS;
+  p.border = counters;  // the first n of the launch's counters
+  for (int j = 0; j < n; ++j) {
+    const SkMatmul& m = mm[j];
+    tc::SkOp& o = p.op[j];
+    if ((reinterpret_cast<uintptr_t>(m.w) & 15) != 0) return fail(c, D3_ERR_UNSUPPORTED, "tiled weights must be 16-byte aligned");
+    o.ep = m.ep;
+    o.epi = m.epi;
+    o.N = m.N;
+    o.k_chunks = m.K / 64;
+    o.n_tiles = m.N / 256;
+    o.tiles = o.n_tiles * p.tok_tiles;
+    // Whole waves of tiles are dealt round-robin; what is left over is cut along K when that saves more slabs per pair
+    // than the exchange of partials costs (about 12 slabs' time).
+    o.full_tiles = o.tiles / P * P;
+    const int rest = o.tiles - o.full_tiles;
+    const int gain = rest > 0 ? o.k_chunks - rest * o.k_chunks / P : 0;
+    if (rest * o.k_chunks < P || (c->tune_sk != 1 && gain <= 12)) o.full_tiles = o.tiles;
+    o.part_count = counters + SK_MAX_BORDERS + j * (SK_OP_COUNTERS - SK_MAX_BORDERS);
+    const CUtensorMap* t = nullptr;
+    TRY(get_tmap(c, m.x, M, m.K, p.tok_n / 2, &t));
+    p.x[j] = *t;
+    TRY(get_tmap(c, m.w, m.N / 128 * o.k_chunks * 128, 64, 128, &t, false));
+    p.w[j] = *t;
+    if (m.qx) {
+      p.rope_rows = 1;
+      p.pos_base = m.qx->rm.pos_base; p.n_valid = m.qx->rm.n_valid; p.rows_per_seq = m.qx->rm.rows_per_seq;
+      o.k_cache = static_cast<bf16*>(m.qx->k_cache); o.v_cache = static_cast<bf16*>(m.qx->v_cache);
+    }
+  }
+  cfg.gridDim = dim3(static_cast<unsigned>(2 * P));
+  if (c->pdl && !c->prof_on) {
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+  }
+  CUDA_TRY(c, cudaLaunchKernelEx(&cfg, tc::gemm_sk_kernel, p));
+  LAUNCHED(c, "gemm_sk_kernel");
+  return D3_OK;
+}
+
 int run_linear_tc(d3_ctx* c, const void* X, const void* W, int M, int N, int K, int epi, const EpiParams& ep,
                   int ctas_hint, const QkvExtra* qx, int w_tiled) {
+  if (ctas_hint == 0 && c->tune_sk == 1 && w_tiled && epi != EPI_STATS && M <= tc::SK_MAX_ROWS && sk_shape_ok(N, K) && (reinterpret_cast<uintptr_t>(ep.y) & 15) == 0) {  // asked for by name
+    const SkMatmul m{X, W, N, K, epi, ep, qx};
+    TRY(sk_begin(c, 1));
+    return run_sk(c, &m, 1, M);
+  }
   // `ctas_hint` 1..8 on a skinny matmul forces the cluster size; larger hints ask for the unit-range kernel
   // Few column tiles and a long K (O-proj, down): clusters that split K and reduce through
   // distributed shared memory beat the L2 reduction of the unit-range kernel (measured at 32 rows on
@@ -1312,6 +1425,24 @@ int run_stats_merge(d3_ctx* c, int M, int n_tiles, float* conf, float* ent, int*
   return D3_OK;
 }
 
+// Forwards whose matmuls run on gemm_sk_kernel (those that the chain does not take): up to 640 rows.  Measured, ms per
+// decode forward of sequences with 128..400 stored positions, one kernel per matmul against this: 8B shape 4.48 -> 4.07
+// at 128 rows, 6.40 -> 5.37 at 256, 9.80 -> 8.37 at 384, 10.46 -> 10.04 at 512, 12.57 -> 12.46 at 640, but 13.31 -> 13.55 at
+// 768 and 16.77 -> 17.76 at 1024 (tiles of an incomplete wave weigh less there, and whole tiles that go through L2 more);
+// 7B shape 6.18 -> 3.63 at 128, 5.91 -> 4.95 at 256, 9.54 -> 8.42 at 512, 11.73 -> 11.41 at 640.
+constexpr int SK_FORWARD_ROWS = 640;
+bool sk_forward_usable(const d3_ctx* c, int M) {
+  const d3_config& g = c->cfg;
+  if (c->tune_sk == 0 || !c->use_tc || !c->fuse_qkv || !c->fold_norm || !c->w_tiled) return false;
+  const int d = g.d_model, nq = g.n_q_heads * g.d_head, nkv = g.n_kv_heads * g.d_head, f = g.d_ffn;
+  if (!sk_shape_ok(nq + 2 * nkv, d) || !sk_shape_ok(d, nq) || !sk_shape_ok(2 * f, d) || !sk_shape_ok(d, f)) return false;
+  if (M > tc::SK_MAX_ROWS) return false;
+  if (c->tune_sk == 1) return true;
+  // a schedule asked for by name is another kernel's
+  if (c->tune_strip != 0 || c->tune_no_cluster || c->tune_xt == 0 || c->tune_cta_pairs == 0 || c->tune_wide_tiles >= 0 || c->tune_pair >= 0) return false;
+  return M <= SK_FORWARD_ROWS;
+}
+
 // The transformer stack over M rows laid out as bs x rows_per_seq (row map already on the device).
 //   head: 0 = none, 1 = fused statistics into ctx conf/ent/argmax, 2 = fp32 logits into `logits`.
 //   seg: rows per segment when a sequence's rows are consecutive blocks that must not see later ones (0: one segment).
@@ -1372,6 +1503,54 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
       TRY(run_chain(c, o_in, o_out, rm));
       CUDA_TRY(c, cudaMemcpyAsync(c->tap_out, c->x, sizeof(float) * M * d, cudaMemcpyDeviceToDevice, c->stream));
       if (o_out < n_ops) TRY(run_chain(c, o_out, n_ops, rm));
+    }
+  } else if (sk_forward_usable(c, M)) {
+    // Decode-sized forward: the matmuls between two attention kernels (O-proj, gate/up, down, the next layer's QKV) in
+    // one launch of resident CTA pairs.  The residual stream between two launches is a layer's output.
+    TRY(sk_begin(c, 4 * g.n_layers));
+    auto qkv = [&](int l, QkvExtra& qx) {
+      EpiParams ep;
+      ep.y = c->q; ep.ldy = nq;
+      after_norm(ep);
+      qx = QkvExtra{rm, k_plane(c, l), v_plane(c, l)};
+      return SkMatmul{c->xb, c->wqkv[l], nq + 2 * nkv, d, EPI_QKV, ep, &qx};
+    };
+    // (while classes are timed every matmul is a launch of its own)
+    auto launch = [&](const SkMatmul* mm, const int* cls, int n) {
+      if (!c->prof_on) return run_sk(c, mm, n, M);
+      for (int j = 0; j < n; ++j) {
+        ProfScope ps(c, cls[j]);
+        TRY(run_sk(c, mm + j, 1, M));
+      }
+      return static_cast<int>(D3_OK);
+    };
+    const int classes[4] = {D3_PROF_GEMM_O, D3_PROF_GEMM_GATE_UP, D3_PROF_GEMM_DOWN, D3_PROF_GEMM_QKV};
+    const bool tap = M <= c->tap_rows;
+    QkvExtra qx{};
+    {
+      const SkMatmul first = qkv(0, qx);
+      TRY(launch(&first, classes + 3, 1));
+    }
+    for (int l = 0; l < g.n_layers; ++l) {
+      if (l == c->tap_layer && tap)
+        CUDA_TRY(c, cudaMemcpyAsync(c->tap_in, c->x, sizeof(float) * M * d, cudaMemcpyDeviceToDevice, c->stream));
+      TRY(run_attention(c, c->q, l, c->o, rm));
+      EpiParams eo, eg, ed;
+      eo.y = c->x; eo.ldy = d;
+      updates_resid(eo);
+      eg.y = c->h; eg.ldy = f;
+      after_norm(eg);
+      ed.y = c->x; ed.ldy = d;
+      updates_resid(ed);
+      SkMatmul mm[4] = {{c->o, c->wo[l], d, nq, EPI_RESID, eo, nullptr},
+                        {c->xb, c->wgu[l], 2 * f, d, EPI_SWIGLU, eg, nullptr},
+                        {c->h, c->wd[l], d, f, EPI_RESID, ed, nullptr},
+                        {}};
+      const bool more = l + 1 < g.n_layers;
+      if (more) mm[3] = qkv(l + 1, qx);
+      TRY(launch(mm, classes, more ? 4 : 3));
+      if (l == c->tap_layer && tap)
+        CUDA_TRY(c, cudaMemcpyAsync(c->tap_out, c->x, sizeof(float) * M * d, cudaMemcpyDeviceToDevice, c->stream));
     }
   } else
   for (int l = 0; l < g.n_layers; ++l) {
@@ -1549,6 +1728,8 @@ extern "C" int d3_create(const d3_config* cfg, void* cuda_stream, d3_ctx** out) 
     A_(c->partial, c->partial_slots * 128 * 128 * sizeof(float));
     c->n_tile_count = 1 << 16;
     A_(c->tile_count, sizeof(int) * c->n_tile_count);
+    c->sk_sync_cap = static_cast<size_t>(4 * g.n_layers) * SK_OP_COUNTERS;
+    A_(c->sk_sync, sizeof(unsigned int) * c->sk_sync_cap);
   }
   if (c->use_tc && g.d_head == 128) {
     const long long kv_rows = static_cast<long long>(g.n_layers) * 2 * g.max_batch * g.n_kv_heads * g.max_seq;
@@ -2224,6 +2405,7 @@ extern "C" void d3_tuning_defaults(d3_tuning* t) {
   t->weights_as_rows = -1;
   t->attention_tmem = -1;
   t->cta_pairs = -1;
+  t->k_cut_pairs = -1;
 }
 extern "C" int d3_set_tuning(d3_ctx* c, const d3_tuning* t) {
   if (!c || !t) return D3_ERR_INVALID_ARG;
@@ -2233,7 +2415,7 @@ extern "C" int d3_set_tuning(d3_ctx* c, const d3_tuning* t) {
       (t->round_robin != 0 && t->round_robin != 1) || t->column_strips < 0 || t->column_strips > 3 || t->strip_stages < 0 ||
       t->strip_stages > 32 || t->chain < -1 || t->chain > 0 || t->chain_clusters < 0 || t->chain_l2_ahead < -1 || t->chain_l2_ahead > 256 || t->weights_as_rows < -1 || t->weights_as_rows > 0 ||
       ((t->attention_tmem < -1 || t->attention_tmem > 2) && t->attention_tmem != 64 && t->attention_tmem != 128) ||
-      t->cta_pairs < -1 || t->cta_pairs > 0)
+      t->cta_pairs < -1 || t->cta_pairs > 0 || t->k_cut_pairs < -1 || t->k_cut_pairs > 1)
     return fail(c, D3_ERR_INVALID_ARG, "d3_set_tuning: a field is outside its range");
   c->tune_ring_kb = t->ring_kb;
   c->tune_ctas_per_sm = t->ctas_per_sm;
@@ -2252,6 +2434,7 @@ extern "C" int d3_set_tuning(d3_ctx* c, const d3_tuning* t) {
   c->tune_attn_tmem = t->attention_tmem > 1 ? 1 : t->attention_tmem;
   c->tune_attn_shape = t->attention_tmem > 1 ? t->attention_tmem : 0;
   c->tune_cta_pairs = t->cta_pairs;
+  c->tune_sk = t->k_cut_pairs;
   return D3_OK;
 }
 extern "C" int d3_set_fused_finalize(d3_ctx* c, int on) {

@@ -5,6 +5,8 @@ within 3e-2 of max |logit|; committed ids bit-exact except where the oracle's |c
 or top-2 probability gap is below 1e-3 (or the forced commit is a near-tie between the two most
 confident masked positions); those are counted and reported.
 """
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -542,6 +544,45 @@ def test_small_bf16_ragged_batch_step_locked(d_head, hq, hkv, impl):
             r2 = free_running_p2(ctx, model, ids[b, :lens[b]], 64, 32, 0.9, noise)
             record_report(f"small_bf16_free_running_{d_head}_{hq}_{hkv}_impl{impl}_seq{b}", r2)
             assert r2["resyncs"] <= r2["blocks"] and max(r2["margins"], default=0.0) <= 1e-2, r2
+
+
+@pytest.mark.parametrize("lens,gen", [([45], 64), ([40, 7, 97, 64, 33], 64)])
+def test_small_bf16_batch_on_k_cut_pairs_step_locked(lens, gen):
+    """Forwards whose matmuls run as launches of resident CTA pairs (O-proj, gate/up, down and the next layer's QKV in
+    one launch), every tile of an incomplete wave cut along K: one 32-row block and 160 rows, prefill included (a
+    ragged batch with dead rows).  Step-locked against the oracle, and a tapped layer against the other schedules."""
+    # logit_scale 10: logits with the standard deviation 10 * 0.02 * sqrt(1024) = 6.4 of the d_model = 256 models (20 * 0.02 *
+    # sqrt(256)), for which the bound on the statistics was taken (a confidence moves by at most a logit's error)
+    shape = dataclasses.replace(si.scaled_shape(si.LLADA8B, name="small-k-cut", n_layers=3, d_model=1024, n_q_heads=8, n_kv_heads=4,
+                                                d_ffn=1280, vocab=1024, d_head=128), logit_scale=10.0)
+    W = si.gen_weights(shape)
+    wl, ids, lens = si.small_workload("small-k-cut", shape, len(lens), lens, gen, 32, 0.9, 79)
+    model = o.model_from_shape(shape, W, np.float32, mirror_bf16=True)
+    exact = o.model_from_shape(shape, W, np.float32)
+    bs = len(lens)
+    blk = np.full((bs, 32), shape.mask_id, dtype=np.int32)
+    with Ctx(shape, W, block=32, max_batch=bs, max_seq=wl.max_seq) as ctx:
+        def tapped():
+            ctx.prefill(ids, lens)
+            d3.d3_set_tap(ctx.ctx, 1)
+            lg = ctx.logits(blk)
+            t = [torch.zeros((bs * 32, shape.d_model), dtype=torch.float32, device="cuda") for _ in range(2)]
+            d3.d3_read_tap(ctx.ctx, t[0], t[1], bs * 32)
+            d3.d3_set_tap(ctx.ctx, -1)
+            return [lg] + [x.cpu().numpy() for x in t]
+        d3.d3_set_tuning(ctx.ctx, chain=0, k_cut_pairs=0)
+        base = tapped()
+        d3.d3_set_tuning(ctx.ctx, chain=0, k_cut_pairs=1)
+        n0 = d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel")
+        got = tapped()
+        assert d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel") == n0 + 2 * (shape.n_layers + 1) + 1  # prefill, block forward, logits
+        for a, b in zip(got, base):  # two schedules of one forward: the bound of the column-strip test
+            assert np.max(np.abs(a - b)) <= 1e-2 * np.max(np.abs(b))
+        rep, _ = step_locked(ctx, model, ids, lens, gen, 32, 0.9, logit_tol=3e-2, exact_model=exact)
+        record_report(f"small_bf16_step_locked_on_k_cut_pairs_{bs}", rep)
+        assert rep["max_logit_err"] <= 3e-2
+        assert_rounding_bounded(rep, BF16_STAT_ERR_BOUND)
+        assert ctx.error_word() == 0
 
 
 def test_small_bf16_batch_on_cta_pairs_step_locked():

@@ -141,6 +141,47 @@ def test_linear_bf16_weights_as_rows(ctx_bf16, m, n, k, cluster):
     assert ctx_bf16.error_word() == 0
 
 
+@pytest.mark.parametrize("m,n,k", [(1, 256, 64), (32, 512, 4096), (33, 3584, 3584), (96, 256, 8192), (128, 12288, 512), (129, 4096, 1024),
+                                   (200, 768, 2048), (256, 4096, 4096), (257, 1280, 1920), (501, 3584, 1024), (640, 19200, 256)])
+def test_linear_bf16_k_cut_pairs(ctx_bf16, m, n, k):
+    """Weights as the row operand of CTA pairs with the tiles of an incomplete wave cut along K: one tile and no cut,
+    one tile shared by all pairs, ranges that touch two tiles, a whole wave followed by cut tiles (640 x 19200), one
+    to three tiles of rows, row counts on both sides of a multiple of 16, 32 and 256; fp32, residual, bf16 and SwiGLU
+    epilogues against the fp64 product (bounds as in the other matmul tests), twice with the same bits."""
+    rng = np.random.default_rng(m + n + k)
+    xt, x = rand_bf16(rng, (m, k))
+    wt, w = rand_bf16(rng, (n, k), 0.05)
+    ref = x @ w.T
+    tol = 2e-5 * np.sqrt(k) * np.abs(ref).max() + 1e-6
+    xd, wd = xt.to(DEV), wt.to(DEV)
+    packed = torch.full((d3.d3_packed_weight_elems(n, k),), 3.0, dtype=torch.bfloat16, device=DEV)
+    d3.d3_pack_weight(ctx_bf16.ctx, wd, packed)
+    d3.d3_set_tuning(ctx_bf16.ctx, k_cut_pairs=1)
+    try:
+        n0 = d3.d3_launch_count_of(ctx_bf16.ctx, "gemm_sk_kernel")
+        y = torch.full((m, n), 7.0, dtype=torch.float32, device=DEV)
+        d3.d3_op_linear_packed(ctx_bf16.ctx, xd, packed, y, n, 0, 0)
+        assert np.max(np.abs(y.cpu().numpy() - ref)) <= tol
+        y2 = torch.full((m, n), 7.0, dtype=torch.float32, device=DEV)
+        d3.d3_op_linear_packed(ctx_bf16.ctx, xd, packed, y2, n, 0, 0)
+        assert torch.equal(y, y2)
+        y0 = rng.standard_normal((m, n)).astype(np.float32)
+        yr = torch.from_numpy(y0).to(DEV)
+        d3.d3_op_linear_packed(ctx_bf16.ctx, xd, packed, yr, n, 2, 0)
+        assert np.max(np.abs(yr.cpu().numpy() - (ref + y0))) <= tol + 1e-6
+        yb = torch.zeros((m, n), dtype=torch.bfloat16, device=DEV)
+        d3.d3_op_linear_packed(ctx_bf16.ctx, xd, packed, yb, n, 1, 0)
+        assert np.max(np.abs(yb.float().cpu().numpy() - ref)) <= tol + 2 ** -8 * np.abs(ref).max()
+        h = torch.zeros((m, n // 2), dtype=torch.bfloat16, device=DEV)
+        d3.d3_op_linear_packed(ctx_bf16.ctx, xd, packed, h, n, 3, 0)
+        want = swiglu_ref(ref, n)
+        assert np.max(np.abs(h.float().cpu().numpy() - want)) <= 2 ** -7 * np.abs(want).max() + tol
+        assert d3.d3_launch_count_of(ctx_bf16.ctx, "gemm_sk_kernel") == n0 + 5
+    finally:
+        d3.d3_set_tuning(ctx_bf16.ctx)
+    assert ctx_bf16.error_word() == 0
+
+
 @pytest.mark.parametrize("m,n,k", [(512, 256, 64), (1024, 512, 512), (640, 768, 1024), (1000, 256, 4096), (2048, 4096, 1024),
                                    (513, 12288, 256), (256, 19200, 128), (130, 19200, 64)])
 def test_linear_bf16_cta_pairs(ctx_bf16, m, n, k):
