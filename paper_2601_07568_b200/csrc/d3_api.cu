@@ -1415,12 +1415,12 @@ int run_rmsnorm(d3_ctx* c, const float* x, const float* gain, void* xn, int M) {
 int run_stats_merge(d3_ctx* c, int M, int n_tiles, float* conf, float* ent, int* argmax, bool sampled = false) {
   ProfScope ps(c, D3_PROF_OTHER);
   if (sampled) {
-    CUDA_TRY(c, launch_pdl(c, stats_merge_sample_kernel, dim3((M + 3) / 4), dim3(128), 0, static_cast<const float4*>(c->stat_part),
+    CUDA_TRY(c, launch_pdl(c, stats_merge_sample_kernel, dim3(M), dim3(MERGE_THREADS), 0, static_cast<const float4*>(c->stat_part),
                            static_cast<const float4*>(c->sample_part), n_tiles, M, conf, ent, argmax));
     LAUNCHED(c, "stats_merge_sample_kernel");
     return D3_OK;
   }
-  CUDA_TRY(c, launch_pdl(c, stats_merge_kernel, dim3((M + 3) / 4), dim3(128), 0, static_cast<const float4*>(c->stat_part), n_tiles, M, conf, ent, argmax));
+  CUDA_TRY(c, launch_pdl(c, stats_merge_kernel, dim3(M), dim3(MERGE_THREADS), 0, static_cast<const float4*>(c->stat_part), n_tiles, M, conf, ent, argmax));
   LAUNCHED(c, "stats_merge_kernel");
   return D3_OK;
 }
@@ -1466,12 +1466,13 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
 
   {
     ProfScope ps(c, D3_PROF_OTHER);
-    if (c->is_bf16) CUDA_TRY(c, launch_pdl(c, embed_kernel<bf16>, dim3(M), dim3(128), 0, ids, static_cast<const bf16*>(c->tok_emb), c->x, d, g.vocab, c->error_word));
-    else CUDA_TRY(c, launch_pdl(c, embed_kernel<float>, dim3(M), dim3(128), 0, ids, static_cast<const float*>(c->tok_emb), c->x, d, g.vocab, c->error_word));
-    LAUNCHED(c, "embed_kernel");
     if (c->fold_norm) {
-      CUDA_TRY(c, launch_pdl(c, row_prep_kernel, dim3(M), dim3(128), 0, static_cast<const float*>(c->x), static_cast<bf16*>(c->xb), c->ssq, d));
-      LAUNCHED(c, "row_prep_kernel");
+      CUDA_TRY(c, launch_pdl(c, embed_prep_kernel, dim3(M), dim3(256), 0, ids, static_cast<const bf16*>(c->tok_emb), c->x, static_cast<bf16*>(c->xb), c->ssq, d, g.vocab, c->error_word));
+      LAUNCHED(c, "embed_prep_kernel");
+    } else {
+      if (c->is_bf16) CUDA_TRY(c, launch_pdl(c, embed_kernel<bf16>, dim3(M), dim3(128), 0, ids, static_cast<const bf16*>(c->tok_emb), c->x, d, g.vocab, c->error_word));
+      else CUDA_TRY(c, launch_pdl(c, embed_kernel<float>, dim3(M), dim3(128), 0, ids, static_cast<const float*>(c->tok_emb), c->x, d, g.vocab, c->error_word));
+      LAUNCHED(c, "embed_kernel");
     }
   }
   // Folded RMSNorm: the matmuls after a norm read the bf16 copy of the residual stream and scale
@@ -2166,11 +2167,19 @@ extern "C" int d3_generate_multiblock(d3_ctx* c, int32_t gen_len, float threshol
   return check_device_error(c);
 }
 
+static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
 extern "C" int d3_trajectory_rank(d3_ctx* c, const int32_t* commit_step, int32_t bs, int32_t gen_len, int32_t* rank) {
   if (!c) return D3_ERR_INVALID_ARG;
   if (!commit_step || !rank || bs <= 0 || gen_len <= 0) return fail(c, D3_ERR_INVALID_ARG, "bad trajectory_rank arguments");
   if (gen_len % c->cfg.block != 0) return fail(c, D3_ERR_SHAPE, "gen_len not a multiple of the block size");
-  trajectory_rank_kernel<<<bs, 32, 0, c->stream>>>(commit_step, gen_len, c->cfg.block, rank);
+  const int B = c->cfg.block;
+  if (B >= 4 && B <= 128 && (B & (B - 1)) == 0 && aligned16(commit_step) && aligned16(rank)) {
+    trajectory_rank4_kernel<<<(bs + 7) / 8, 256, 0, c->stream>>>(commit_step, bs, gen_len, B, rank);
+    LAUNCHED(c, "trajectory_rank4_kernel");
+    return D3_OK;
+  }
+  trajectory_rank_kernel<<<bs, 32, 0, c->stream>>>(commit_step, gen_len, B, rank);
   LAUNCHED(c, "trajectory_rank_kernel");
   return D3_OK;
 }
@@ -2179,6 +2188,13 @@ extern "C" int d3_noisy_sequence(d3_ctx* c, const int32_t* y, const int32_t* ran
   if (!c) return D3_ERR_INVALID_ARG;
   if (!y || !rank || !s || !k || !m || !out || bs <= 0 || n <= 0) return fail(c, D3_ERR_INVALID_ARG, "bad noisy_sequence arguments");
   if (bs > 65535) return fail(c, D3_ERR_SHAPE, "more than 65535 sequences in one call");
+  if (n % 4 == 0 && aligned16(y) && aligned16(rank) && aligned16(out)) {
+    const long long quads = static_cast<long long>(bs) * (n / 4);
+    noisy_sequence4_kernel<<<static_cast<unsigned>((quads + 255) / 256), 256, 0, c->stream>>>(
+        reinterpret_cast<const int4*>(y), reinterpret_cast<const int4*>(rank), s, k, m, bs, n / 4, c->cfg.mask_id, reinterpret_cast<int4*>(out));
+    LAUNCHED(c, "noisy_sequence4_kernel");
+    return D3_OK;
+  }
   noisy_sequence_kernel<<<dim3((n + 255) / 256, bs), 256, 0, c->stream>>>(y, rank, s, k, m, n, c->cfg.mask_id, out);
   LAUNCHED(c, "noisy_sequence_kernel");
   return D3_OK;
@@ -2581,7 +2597,7 @@ int lm_head_stats_static(const void* x, const void* w, int m, int vocab, int k, 
     (void)cudaGetLastError();
     return D3_ERR_CUDA;
   }
-  stats_merge_kernel<<<(m + 3) / 4, 128, 0, stream>>>(part, n_tiles, m, conf, entropy, argmax);
+  stats_merge_kernel<<<m, MERGE_THREADS, 0, stream>>>(part, n_tiles, m, conf, entropy, argmax);
   if (cudaPeekAtLastError() != cudaSuccess) {
     (void)cudaGetLastError();
     return D3_ERR_CUDA;

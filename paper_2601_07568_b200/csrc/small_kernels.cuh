@@ -50,25 +50,45 @@ __global__ void embed_kernel(const int* __restrict__ ids, const T* __restrict__ 
 }
 
 // ----------------------------------------------------------------------------- folded RMSNorm helpers
-// What a residual epilogue leaves behind for the next matmul (see EpiParams), for rows that no matmul
-// has written yet (the embeddings): bf16 copy of x and the sum of squares of every 32-column chunk.
-// One block per row; thread t takes chunks t, t + blockDim.x, ...
-__global__ void row_prep_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ xb, float* __restrict__ ssq, int d) {
+// The embeddings of a forward on the tensor-core path: the rows themselves and what a residual epilogue leaves behind for
+// the next matmul (see EpiParams), bf16 copy and sum of squares of every 32-column chunk, from one read of the table.
+// One block per row, 8 columns a thread (d_model is a multiple of 8), four neighbouring lanes a chunk.  Bound by its
+// stores.  As two kernels, the second with 32 columns a thread: 22 us in front of a 32-row forward and 0.85 ms in front of
+// a 16384 x 4096 prefill; this one 5 us and 0.10 ms.
+__global__ void __launch_bounds__(256) embed_prep_kernel(const int* __restrict__ ids, const __nv_bfloat16* __restrict__ emb, float* __restrict__ x,
+                                                         __nv_bfloat16* __restrict__ xb, float* __restrict__ ssq, int d, int vocab, uint32_t* error_word) {
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
-  const int m = blockIdx.x;
-  const int n_chunks = (d + 31) / 32;
-  const float* row = x + static_cast<size_t>(m) * d;
-  __nv_bfloat16* out = xb + static_cast<size_t>(m) * d;
-  for (int ch = threadIdx.x; ch < n_chunks; ch += blockDim.x) {
+  const int m = blockIdx.x, n_chunks = (d + 31) / 32;
+  int id = ids[m];
+  if (id < 0 || id >= vocab) {
+    if (threadIdx.x == 0) atomicOr(error_word, ERRW_BAD_TOKEN_ID);
+    id = 0;
+  }
+  const uint4* src = reinterpret_cast<const uint4*>(emb + static_cast<size_t>(id) * d);
+  float4* row = reinterpret_cast<float4*>(x + static_cast<size_t>(m) * d);
+  uint4* copy = reinterpret_cast<uint4*>(xb + static_cast<size_t>(m) * d);
+  for (int i0 = 0; i0 < n_chunks * 4; i0 += blockDim.x) {  // (all lanes: the sums are exchanged)
+    const int i = i0 + threadIdx.x;
     float sq = 0.f;
-    const int e1 = min(d, ch * 32 + 32);
-    for (int e = ch * 32; e < e1; ++e) {  // same element order as the matmul epilogue's chunk sum
-      const float v = row[e];
-      sq += v * v;
-      out[e] = __float2bfloat16_rn(v);
+    if (i < d / 8) {
+      const uint4 v = src[i];
+      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+      float f[8];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        f[2 * q] = __uint_as_float(w[q] << 16);
+        f[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) sq += f[q] * f[q];
+      row[2 * i] = make_float4(f[0], f[1], f[2], f[3]);
+      row[2 * i + 1] = make_float4(f[4], f[5], f[6], f[7]);
+      copy[i] = v;
     }
-    ssq[static_cast<size_t>(m) * n_chunks + ch] = sq;
+    sq += __shfl_xor_sync(0xffffffffu, sq, 1);
+    sq += __shfl_xor_sync(0xffffffffu, sq, 2);
+    if ((threadIdx.x & 3) == 0 && i / 4 < n_chunks) ssq[static_cast<size_t>(m) * n_chunks + i / 4] = sq;
   }
 }
 
@@ -185,32 +205,57 @@ __global__ void rope_kv_kernel(const float* __restrict__ qkv, T* __restrict__ q_
 }
 
 // ----------------------------------------------------------------------------- statistics merge
-// One warp per row merges the per-tile partial statistics in ascending tile order (fixed tree) and
-// writes confidence = 1/Z, entropy = ln Z - S/Z (nats) and the arg max.
-__global__ void stats_merge_kernel(const float4* __restrict__ part, int n_tiles, int M, float* __restrict__ conf,
-                                   float* __restrict__ entropy, int* __restrict__ argmax) {
-  ptx::grid_dep_wait();
-  ptx::grid_dep_launch();
-  const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+// One 256-thread block per row: thread t merges tiles t, t + 256, ... in ascending order, all its loads in flight, then a
+// fixed tree over lanes and warps; confidence = 1/Z, entropy = ln Z - S/Z (nats) and the arg max.  (A warp per row walks
+// through 31 tiles a lane of a 126464-token vocabulary, a load and two exponentials each: 20 us behind the LM head, 5 here.)
+constexpr int MERGE_THREADS = 256;
+__device__ __forceinline__ SoftStat stat_shfl_xor(const SoftStat& st, int o) {
+  SoftStat other;
+  other.m = __shfl_xor_sync(0xffffffffu, st.m, o);
+  other.z = __shfl_xor_sync(0xffffffffu, st.z, o);
+  other.s = __shfl_xor_sync(0xffffffffu, st.s, o);
+  other.a = __shfl_xor_sync(0xffffffffu, st.a, o);
+  return other;
+}
+// The statistic of a row's partials, in every thread of warp 0.
+__device__ __forceinline__ SoftStat merge_row_stats(const float4* __restrict__ row, int n_tiles) {
+  __shared__ SoftStat warp_stat[MERGE_THREADS / 32];
   const int lane = threadIdx.x & 31;
-  if (m >= M) return;
   SoftStat st = stat_empty();
-  for (int t = lane; t < n_tiles; t += 32) {
-    float4 v = part[static_cast<size_t>(m) * n_tiles + t];
-    SoftStat o{v.x, v.y, v.z, __float_as_int(v.w)};
-    st = stat_merge(st, o);
+  for (int t0 = threadIdx.x; t0 < n_tiles; t0 += 4 * MERGE_THREADS) {
+    float4 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int t = t0 + q * MERGE_THREADS;
+      v[q] = t < n_tiles ? __ldcg(row + t) : make_float4(-INFINITY, 0.f, 0.f, __int_as_float(0x7fffffff));
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) st = stat_merge(st, SoftStat{v[q].x, v[q].y, v[q].z, __float_as_int(v[q].w)});
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    SoftStat other;
-    other.m = __shfl_xor_sync(0xffffffffu, st.m, o);
-    other.z = __shfl_xor_sync(0xffffffffu, st.z, o);
-    other.s = __shfl_xor_sync(0xffffffffu, st.s, o);
-    other.a = __shfl_xor_sync(0xffffffffu, st.a, o);
+    const SoftStat other = stat_shfl_xor(st, o);
     // keep the operand order fixed (lower lane first) so every lane computes the same bits
     st = (lane & o) ? stat_merge(other, st) : stat_merge(st, other);
   }
-  if (lane == 0) {
+  if (lane == 0) warp_stat[threadIdx.x >> 5] = st;
+  __syncthreads();
+  if (threadIdx.x >= 32) return st;
+  st = warp_stat[lane & (MERGE_THREADS / 32 - 1)];
+#pragma unroll
+  for (int o = MERGE_THREADS / 64; o > 0; o >>= 1) {
+    const SoftStat other = stat_shfl_xor(st, o);
+    st = (lane & o) ? stat_merge(other, st) : stat_merge(st, other);
+  }
+  return st;
+}
+__global__ void __launch_bounds__(MERGE_THREADS) stats_merge_kernel(const float4* __restrict__ part, int n_tiles, int M, float* __restrict__ conf,
+                                                                    float* __restrict__ entropy, int* __restrict__ argmax) {
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
+  const int m = blockIdx.x;
+  const SoftStat st = merge_row_stats(part + static_cast<size_t>(m) * n_tiles, n_tiles);
+  if (threadIdx.x == 0) {
     if (st.z > 0.f) {
       conf[m] = 1.0f / st.z;
       entropy[m] = fmaxf(logf(st.z) - st.s / st.z, 0.f);
@@ -226,35 +271,40 @@ __global__ void stats_merge_kernel(const float4* __restrict__ part, int n_tiles,
 // The same with temperature sampling: the token is the index of the largest perturbed logit over all
 // tiles (lowest index on ties) and the confidence its probability e^(l - m) / Z under the unperturbed
 // softmax; the entropy is unchanged.
-__global__ void stats_merge_sample_kernel(const float4* __restrict__ part, const float4* __restrict__ sample_part, int n_tiles,
-                                          int M, float* __restrict__ conf, float* __restrict__ entropy, int* __restrict__ argmax) {
+__global__ void __launch_bounds__(MERGE_THREADS) stats_merge_sample_kernel(const float4* __restrict__ part, const float4* __restrict__ sample_part,
+                                                                           int n_tiles, int M, float* __restrict__ conf,
+                                                                           float* __restrict__ entropy, int* __restrict__ argmax) {
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
-  const int m = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (m >= M) return;
-  SoftStat st = stat_empty();
+  __shared__ SampleStat warp_sample[MERGE_THREADS / 32];
+  const int m = blockIdx.x, lane = threadIdx.x & 31;
+  const float4* row = sample_part + static_cast<size_t>(m) * n_tiles;
   SampleStat sp = sample_empty();
-  for (int t = lane; t < n_tiles; t += 32) {
-    const float4 v = part[static_cast<size_t>(m) * n_tiles + t];
-    st = stat_merge(st, SoftStat{v.x, v.y, v.z, __float_as_int(v.w)});
-    const float4 w = sample_part[static_cast<size_t>(m) * n_tiles + t];
-    sp = sample_merge(sp, SampleStat{w.x, w.y, __float_as_int(w.z)});
-  }
+  for (int t0 = threadIdx.x; t0 < n_tiles; t0 += 4 * MERGE_THREADS) {
+    float4 w[4];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    SoftStat other;
-    other.m = __shfl_xor_sync(0xffffffffu, st.m, o);
-    other.z = __shfl_xor_sync(0xffffffffu, st.z, o);
-    other.s = __shfl_xor_sync(0xffffffffu, st.s, o);
-    other.a = __shfl_xor_sync(0xffffffffu, st.a, o);
-    st = (lane & o) ? stat_merge(other, st) : stat_merge(st, other);
-    SampleStat so;
-    so.pm = __shfl_xor_sync(0xffffffffu, sp.pm, o);
-    so.la = __shfl_xor_sync(0xffffffffu, sp.la, o);
-    so.pa = __shfl_xor_sync(0xffffffffu, sp.pa, o);
-    sp = sample_merge(sp, so);
+    for (int q = 0; q < 4; ++q) {
+      const int t = t0 + q * MERGE_THREADS;
+      w[q] = t < n_tiles ? __ldcg(row + t) : make_float4(-INFINITY, 0.f, __int_as_float(0x7fffffff), 0.f);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sp = sample_merge(sp, SampleStat{w[q].x, w[q].y, __float_as_int(w[q].z)});
   }
+  auto over_lanes = [&](int widest) {
+    for (int o = widest; o > 0; o >>= 1) {
+      SampleStat so;
+      so.pm = __shfl_xor_sync(0xffffffffu, sp.pm, o);
+      so.la = __shfl_xor_sync(0xffffffffu, sp.la, o);
+      so.pa = __shfl_xor_sync(0xffffffffu, sp.pa, o);
+      sp = sample_merge(sp, so);
+    }
+  };
+  over_lanes(16);
+  if (lane == 0) warp_sample[threadIdx.x >> 5] = sp;
+  const SoftStat st = merge_row_stats(part + static_cast<size_t>(m) * n_tiles, n_tiles);  // (its barrier also publishes warp_sample)
+  if (threadIdx.x >= 32) return;
+  sp = warp_sample[lane & (MERGE_THREADS / 32 - 1)];
+  over_lanes(MERGE_THREADS / 64);
   if (lane == 0) {
     if (st.z > 0.f && sp.pa != 0x7fffffff) {
       conf[m] = fminf(expf(sp.la - st.m) / st.z, 1.0f);
@@ -845,6 +895,43 @@ __global__ void trajectory_rank_kernel(const int* __restrict__ commit_step, int 
     done += mx;
   }
 }
+// The same with four positions a lane and all loads of 512 positions in flight: block sizes that are a power of two from 4
+// to 128, 16-byte aligned rows.  Bound by memory (8 bytes a position); a warp per 32-thread block that waits for every
+// decoding block's load in turn takes 22 us for 16384 x 256 positions, this one 8.
+__global__ void __launch_bounds__(256) trajectory_rank4_kernel(const int* __restrict__ commit_step, int bs, int gen_len, int B, int* __restrict__ rank) {
+  const int b = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (b >= bs) return;  // warp-uniform
+  const int4* cs = reinterpret_cast<const int4*>(commit_step + static_cast<size_t>(b) * gen_len);
+  int4* out = reinterpret_cast<int4*>(rank + static_cast<size_t>(b) * gen_len);
+  const int n4 = gen_len / 4, group = B / 4;  // lanes of a block
+  int done = 0;
+  for (int j0 = 0; j0 < n4; j0 += 128) {
+    int4 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = j0 + q * 32 + lane;
+      v[q] = j < n4 ? cs[j] : make_int4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (j0 + q * 32 >= n4) break;
+      int mx = max(max(max(v[q].x, v[q].y), max(v[q].z, v[q].w)), 0);
+      for (int o = 1; o < group; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      // steps of the blocks before this lane's: the sum over the earlier groups of the 32 lanes
+      const int one = lane % group == 0 ? mx : 0;
+      int sum = one;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int other = __shfl_up_sync(0xffffffffu, sum, o);
+        if (lane >= o) sum += other;
+      }
+      const int base = done + sum - mx;
+      const int j = j0 + q * 32 + lane;
+      if (j < n4) out[j] = make_int4(base + v[q].x, base + v[q].y, base + v[q].z, base + v[q].w);
+      done += __shfl_sync(0xffffffffu, sum, 31);
+    }
+  }
+}
 // The noisy sequence of Sec. 3.1 for a batch: with positions counted from 1, window start s, window
 // length k and m = ceil(k t), position i keeps y_i if i <= s, is the mask id if i > s + k, and in
 // between keeps y_i iff the trajectory had unmasked it by step s + m (rank <= s + m).
@@ -862,6 +949,28 @@ __global__ void noisy_sequence_kernel(const int* __restrict__ y, const int* __re
   if (i <= s) v = y[at];
   else if (i > s + k) v = mask_id;
   else v = rank[at] <= s + m ? y[at] : mask_id;
+  out[at] = v;
+}
+
+// The same with four positions a thread over the whole batch (n a multiple of 4, 16-byte aligned rows), loading only what
+// the result depends on: 16384 x 256 positions in 8 us, with one position a thread in 16.
+__global__ void __launch_bounds__(256) noisy_sequence4_kernel(const int4* __restrict__ y, const int4* __restrict__ rank, const int* __restrict__ s_arr,
+                                                              const int* __restrict__ k_arr, const int* __restrict__ m_arr, int bs, int n4, int mask_id,
+                                                              int4* __restrict__ out) {
+  const long long at = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (at >= static_cast<long long>(bs) * n4) return;
+  const int b = static_cast<int>(at / n4), i = 4 * static_cast<int>(at - static_cast<long long>(b) * n4) + 1;  // first position
+  const int s = s_arr[b], k = k_arr[b], m = m_arr[b];
+  int4 v = make_int4(mask_id, mask_id, mask_id, mask_id);
+  if (i <= s || i <= s + k) {
+    const int4 t = y[at];
+    const int4 r = i + 3 > s ? rank[at] : make_int4(0, 0, 0, 0);
+    const int last = s + m, end = s + k;
+    v.x = i <= s || (i <= end && r.x <= last) ? t.x : mask_id;
+    v.y = i + 1 <= s || (i + 1 <= end && r.y <= last) ? t.y : mask_id;
+    v.z = i + 2 <= s || (i + 2 <= end && r.z <= last) ? t.z : mask_id;
+    v.w = i + 3 <= s || (i + 3 <= end && r.w <= last) ? t.w : mask_id;
+  }
   out[at] = v;
 }
 

@@ -90,3 +90,31 @@ def test_rank_with_several_tokens_per_step_and_long_rows():
         for b in range(2):
             want = o.noisy_sequence(y[b], rank[b], int(s_arr[b]), int(k_arr[b]), int(m_arr[b]), shape.mask_id)
             assert np.array_equal(out[b].cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("block,n_blocks,bs,shift", [(4, 1, 1, 0), (8, 67, 3, 0), (16, 33, 9, 0), (32, 16, 8, 0), (32, 17, 17, 0),
+                                                     (64, 9, 5, 0), (128, 5, 2, 0), (24, 7, 3, 0), (32, 3, 2, 1)])
+def test_rank_and_builder_forms(block, n_blocks, bs, shift):
+    """Block sizes, row lengths on both sides of 128 and 512 positions and rows that are not 16-byte aligned
+    (``shift``): the forms with four positions a thread and the general ones against the oracle, bit for bit."""
+    n = block * n_blocks
+    rng = np.random.default_rng(n + bs)
+    cs = np.stack([np.concatenate([rng.integers(1, 2 + rng.integers(1, block + 1), size=block) for _ in range(n_blocks)]) for _ in range(bs)]).astype(np.int32)
+    y = rng.integers(0, 500, size=(bs, n)).astype(np.int32)
+    s_arr, k_arr, m_arr = (rng.integers(0, hi + 1, size=bs).astype(np.int32) for hi in (n, block, block))
+
+    def dev(a):  # a contiguous tensor that begins `shift` elements into its storage
+        t = torch.zeros(a.size + shift, dtype=torch.int32, device=DEV)[shift:].view(a.shape)
+        t.copy_(torch.from_numpy(a))
+        return t
+    ctx = d3.d3_create(d3.make_config(si.TINY, block=block, max_batch=1, max_seq=block))
+    try:
+        rank, out = dev(np.zeros_like(cs)), dev(np.zeros_like(cs))
+        d3.d3_trajectory_rank(ctx, dev(cs), rank)
+        d3.d3_noisy_sequence(ctx, dev(y), rank, _dev(s_arr), _dev(k_arr), _dev(m_arr), out)
+        torch.cuda.synchronize()
+        for b in range(bs):
+            assert np.array_equal(rank[b].cpu().numpy(), o.trajectory_rank(cs[b], block))
+            assert np.array_equal(out[b].cpu().numpy(), o.noisy_sequence(y[b], rank[b].cpu().numpy(), int(s_arr[b]), int(k_arr[b]), int(m_arr[b]), si.TINY.mask_id))
+    finally:
+        d3.d3_destroy(ctx)
