@@ -195,6 +195,7 @@ __global__ void __launch_bounds__(NW * KQ * 32, NW == 4 ? 1 : 2) attn_tc_kernel(
   const int kv_len = p.rm.kv_len[b];
   const int stable_keys = p.rm.pos_base[b];  // keys [0, pos_base) come from earlier forwards
   const int R = group * rps;
+  const size_t row0 = first_row(p.rm, b);
   bool work = !(qt * BM >= R || n_valid <= 0 || kv_len <= 0);  // rows of this tile that exist at all (uniform over the CTA)
   if (work) {  // a tile whose rows are all beyond n_valid has nothing to do (rows of one head are contiguous)
     bool any = false;
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(NW * KQ * 32, NW == 4 ? 1 : 2) attn_tc_kernel(
   auto row_ptr = [&](int pr, bool& ok) -> const __nv_bfloat16* {
     const int hg = pr / rps, r = pr % rps;
     ok = pr < R && r < n_valid;
-    return p.q + (static_cast<size_t>(b) * rps + r) * p.hq * 128 + (g * group + hg) * 128;
+    return p.q + (row0 + r) * p.hq * 128 + (g * group + hg) * 128;
   };
   bool ok_lo, ok_hi;
   const __nv_bfloat16* q_lo = row_ptr(pr_lo, ok_lo);
@@ -364,7 +365,7 @@ __global__ void __launch_bounds__(NW * KQ * 32, NW == 4 ? 1 : 2) attn_tc_kernel(
 
   auto out_ptr = [&](int pr) -> __nv_bfloat16* {
     const int hg = pr / rps, r = pr % rps;
-    return p.out + (static_cast<size_t>(b) * rps + r) * p.hq * 128 + (g * group + hg) * 128;
+    return p.out + (row0 + r) * p.hq * 128 + (g * group + hg) * 128;
   };
   float* red = reinterpret_cast<float*>(smem);  // [KQ][BM][PART_LD]: partial of every key part; part 0 becomes the CTA's
   if constexpr (KQ == 1) {

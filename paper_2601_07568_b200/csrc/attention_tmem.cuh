@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(TM_THREADS, KT == 64 ? 2 : 1) attn_tmem_kernel
   const int kv_len = p.rm.kv_len[b];
   const int stable_keys = p.rm.pos_base[b];
   const int R = group * rps;
+  const size_t row0 = first_row(p.rm, b);
   bool work = !(qt * BM >= R || n_valid <= 0 || kv_len <= 0);
   if (work) {
     bool any = false;
@@ -248,7 +249,7 @@ __global__ void __launch_bounds__(TM_THREADS, KT == 64 ? 2 : 1) attn_tmem_kernel
     const bool warp_rows = __any_sync(0xffffffffu, row_ok);  // a warp without rows only keeps the barriers going
     ptx::grid_dep_wait();  // Q comes from the kernel before this one
     {  // this thread's row of Q into its lane (128 bf16 = 64 columns) or its shared-memory row; a row that does not exist is zero
-      const uint4* src = reinterpret_cast<const uint4*>(p.q + (static_cast<size_t>(b) * rps + r_seq) * p.hq * 128 +
+      const uint4* src = reinterpret_cast<const uint4*>(p.q + (row0 + r_seq) * p.hq * 128 +
                                                         (g * group + pr / rps) * 128);
       if constexpr (L::Q_SMEM) {
         // rows of a warp without any stay as they are: nobody reads what comes of them; a CTA without tiles needs no
@@ -365,7 +366,7 @@ __global__ void __launch_bounds__(TM_THREADS, KT == 64 ? 2 : 1) attn_tmem_kernel
   // ------------------------------------------------------------------ output
   auto out_ptr = [&](int prow) -> __nv_bfloat16* {
     const int hg = prow / rps, r = prow % rps;
-    return p.out + (static_cast<size_t>(b) * rps + r) * p.hq * 128 + (g * group + hg) * 128;
+    return p.out + (row0 + r) * p.hq * 128 + (g * group + hg) * 128;
   };
   if (p.n_splits == 1) {
     if (alive && row_ok) {

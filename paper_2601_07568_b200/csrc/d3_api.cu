@@ -121,8 +121,10 @@ struct d3_ctx {
   int tune_chain_l2 = -1;       // weight slabs the chain's L2 prefetch runs ahead (-1: default, 0: off)
   int tune_attn_shape = 0;      // experiment: keys per tile of the tcgen05 attention (0 = by rule, 64, 128)
   int tune_attn_tmem = -1;      // tcgen05 attention: -1 where measured faster, 0 never, 1 wherever the shape allows
-  const int* live_n_valid = nullptr;  // set for the span of a forward whose sequences have rows_per_seq % 256 == 0 rows
-  int live_rps = 0, live_rows = 0;    // (padded prompts): the pair kernel passes over row tiles without a live row
+  int* row_off = nullptr;      // [max_batch + 1] first row of every sequence where prompts are laid out one after the other
+  int2* row_map = nullptr;     // [max_rows, rounded up to 256] (sequence, row of it) of such a row
+  bool packed = false;         // set for the span of such a forward, over packed_bs sequences
+  int packed_bs = 0;
   int tune_cta_pairs = -1;      // wide matmuls on CTA pairs (cta_group::2): -1 when the shape allows, 0 never
   int pair_clusters = 0;        // CTA pairs of gemm_pair_kernel resident at once (asked once)
   int tune_sk = -1;             // decode matmuls with K-cut tiles on resident CTA pairs (gemm_sk.cuh): -1 by rule, 0 never, 1 wherever the shape allows
@@ -947,9 +949,9 @@ int run_linear_pair(d3_ctx* c, const void* X, const void* W, int M, int N, int K
   p.w_packed = static_cast<const bf16*>(W);
   p.w_blocks = static_cast<long long>(N / 128) * p.k_chunks;
   p.ep = ep;
-  if (c->live_n_valid != nullptr && M == c->live_rows) {
-    p.live_n_valid = c->live_n_valid;
-    p.live_rps = c->live_rps;
+  if (c->packed) {
+    p.live_rows = c->row_off + c->packed_bs;
+    p.row_map = c->row_map;
   }
   if (qx) {
     p.rope_cos = c->rope_cos; p.rope_sin = c->rope_sin;
@@ -1340,8 +1342,9 @@ int run_attention_tc(d3_ctx* c, const void* q, int layer, void* out, const RowMa
   // is the faster one (measured: 60-70 against 84-110 us per layer at 64 rows x 4200-5100 keys, 27 against 33-37 at
   // 224 rows x 550-1000 keys, a third of the time on 4096-row prompts); at 32 rows the two are level on batches and
   // the mma.sync kernel, with its cheaper start, is ahead on a single sequence (15 against 19 us).
-  if (c->tune_attn_shape == 2 ? attn_stream_usable(c, rm)
-                              : (c->tune_attn_tmem < 0 && attn_stream_usable(c, rm) && rm.bs * g.n_kv_heads >= 2 * c->n_sms))
+  // (the persistent form finds its query rows by a tensor map over equal sequences)
+  if (c->tune_attn_shape == 2 && rm.row_off == nullptr ? attn_stream_usable(c, rm)
+                              : (rm.row_off == nullptr && c->tune_attn_tmem < 0 && attn_stream_usable(c, rm) && rm.bs * g.n_kv_heads >= 2 * c->n_sms))
     return run_attention_tmem_stream(c, q, layer, out, rm);
   if (c->tune_attn_tmem == 1 || (c->tune_attn_tmem < 0 && R >= 64)) return run_attention_tmem(c, q, layer, out, rm);
   const int nw = R <= 32 ? 2 : (R <= 64 ? 4 : 8);
@@ -1443,10 +1446,23 @@ bool sk_forward_usable(const d3_ctx* c, int M) {
   return M <= SK_FORWARD_ROWS;
 }
 
+// Can the rows of a ragged forward be laid out without padding?  Where all its matmuls run on CTA pairs, which take the
+// number of rows from the device (32 prompts of 128..512 tokens, 16384 padded rows of which 10240 are in use: 200.5 -> 137.6 ms).
+// (A tapped forward keeps the layout that d3_read_tap describes.)
+bool pack_usable(const d3_ctx* c, int bs, int M) {
+  const d3_config& g = c->cfg;
+  if (bs < 2 || M <= SK_FORWARD_ROWS || c->tap_layer >= 0 || !c->use_tc || !c->fuse_qkv || !c->fold_norm || !c->attn_tc || c->tune_sk == 1 || c->tune_wide_tiles >= 0)
+    return false;
+  const int d = g.d_model, nq = g.n_q_heads * g.d_head, nkv = g.n_kv_heads * g.d_head, f = g.d_ffn;
+  return pair_usable(c, M, nq + 2 * nkv, d, EPI_QKV, c->w_tiled) && pair_usable(c, M, d, nq, EPI_RESID, c->w_tiled) &&
+         pair_usable(c, M, 2 * f, d, EPI_SWIGLU, c->w_tiled) && pair_usable(c, M, d, f, EPI_RESID, c->w_tiled);
+}
+
 // The transformer stack over M rows laid out as bs x rows_per_seq (row map already on the device).
 //   head: 0 = none, 1 = fused statistics into ctx conf/ent/argmax, 2 = fp32 logits into `logits`.
+//   ragged: a prompt-style forward whose sequences use n_valid of their rows; nothing reads the others afterwards.
 //   seg: rows per segment when a sequence's rows are consecutive blocks that must not see later ones (0: one segment).
-int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float* logits, int seg = 0) {
+int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float* logits, int seg = 0, bool ragged = false) {
   const d3_config& g = c->cfg;
   const int M = bs * rows_per_seq;
   if (M == 0) return D3_OK;
@@ -1454,20 +1470,23 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   const int d = g.d_model, nq = g.n_q_heads * g.d_head, nkv = g.n_kv_heads * g.d_head, f = g.d_ffn;
   RowMap rm{c->pos_base, c->n_valid, c->kv_len, rows_per_seq, bs, seg};
   c->last_rows = M;
-  // Padded prompts: the matmuls on CTA pairs pass over 256-row tiles that hold no live row of their sequence (rows
-  // beyond n_valid are computed by nobody's reader: attention, the cache write and the decisions skip them already).
-  struct LiveRows {
+  // Prompts of different lengths: their rows are laid out one after the other, and the matmuls, which know the padded
+  // count only, stop at the last row in use.
+  const bool packed = ragged && pack_usable(c, bs, M);
+  struct Packed {
     d3_ctx* c;
-    LiveRows(d3_ctx* c_, const int* n_valid, int rps, int rows) : c(c_) {
-      if (rps % 256 == 0) { c->live_n_valid = n_valid; c->live_rps = rps; c->live_rows = rows; }
-    }
-    ~LiveRows() { c->live_n_valid = nullptr; c->live_rps = 0; c->live_rows = 0; }
-  } live_rows(c, c->n_valid, rows_per_seq, M);
-
+    Packed(d3_ctx* c_, bool on, int n) : c(c_) { c->packed = on; c->packed_bs = n; }
+    ~Packed() { c->packed = false; }
+  } packed_span(c, packed, bs);
+  if (packed) {
+    pack_rows_kernel<<<bs, 256, 0, c->stream>>>(c->n_valid, bs, c->row_off, c->row_map);
+    LAUNCHED(c, "pack_rows_kernel");
+    rm.row_off = c->row_off;
+  }
   {
     ProfScope ps(c, D3_PROF_OTHER);
     if (c->fold_norm) {
-      CUDA_TRY(c, launch_pdl(c, embed_prep_kernel, dim3(M), dim3(256), 0, ids, static_cast<const bf16*>(c->tok_emb), c->x, static_cast<bf16*>(c->xb), c->ssq, d, g.vocab, c->error_word));
+      CUDA_TRY(c, launch_pdl(c, embed_prep_kernel, dim3(M), dim3(256), 0, ids, static_cast<const bf16*>(c->tok_emb), c->x, static_cast<bf16*>(c->xb), c->ssq, d, g.vocab, c->error_word, rm.row_off, static_cast<const int*>(c->n_valid), rows_per_seq));
       LAUNCHED(c, "embed_prep_kernel");
     } else {
       if (c->is_bf16) CUDA_TRY(c, launch_pdl(c, embed_kernel<bf16>, dim3(M), dim3(128), 0, ids, static_cast<const bf16*>(c->tok_emb), c->x, d, g.vocab, c->error_word));
@@ -1723,6 +1742,8 @@ extern "C" int d3_create(const d3_config* cfg, void* cuda_stream, d3_ctx** out) 
   A_(c->pos_base, sizeof(int) * g.max_batch);
   A_(c->n_valid, sizeof(int) * g.max_batch);
   A_(c->kv_len, sizeof(int) * g.max_batch);
+  A_(c->row_off, sizeof(int) * (static_cast<size_t>(g.max_batch) + 1));
+  A_(c->row_map, sizeof(int2) * ((R + 255) / 256 * 256));
   A_(c->error_word, sizeof(uint32_t));
   if (c->use_tc) {
     c->partial_slots = 2048;
@@ -1963,7 +1984,7 @@ extern "C" int d3_prefill(d3_ctx* c, const int32_t* prompt_ids, const int32_t* p
     return fail(c, D3_ERR_SHAPE, "prefill larger than max_batch / max_seq / max_prefill_rows");
   prefill_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(prompt_lens, bs, p_max, c->prefix_len, c->pos_base, c->n_valid, c->kv_len);
   LAUNCHED(c, "prefill_rowmap_kernel");
-  TRY(forward(c, prompt_ids, bs, p_max, 0, nullptr));
+  TRY(forward(c, prompt_ids, bs, p_max, 0, nullptr, 0, true));
   if (p_max > 0) {
     hist_store_kernel<<<bs, 128, 0, c->stream>>>(prompt_ids, p_max, c->prefix_len, 0, nullptr, c->hist_ids, c->cfg.max_seq);
     LAUNCHED(c, "hist_store_kernel");
@@ -1987,7 +2008,7 @@ static int refresh_forward(d3_ctx* c, int bs, int* flags, const int* active, lon
   refresh_rowmap_kernel<<<bs, 128, 0, c->stream>>>(c->hist_ids, c->cfg.max_seq, c->prefix_len, flags, active, p_max, 0, c->refresh_ids,
                                                    c->pos_base, c->n_valid, c->kv_len, pending);
   LAUNCHED(c, "refresh_rowmap_kernel");
-  TRY(forward(c, c->refresh_ids, bs, p_max, 0, nullptr));
+  TRY(forward(c, c->refresh_ids, bs, p_max, 0, nullptr, 0, true));
   return D3_OK;
 }
 

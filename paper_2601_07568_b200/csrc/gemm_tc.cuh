@@ -57,10 +57,10 @@ struct GemmParams {
   long long w_blocks;             // number of 128 x 64 blocks in w_packed
   int w_tiled;           // 0: W row-major [N, K]; 1: W stored as contiguous [128 x 64] blocks, block (n_tile, kc) at
                          // row (n_tile * k_chunks + kc) * 128 of a [rows, 64] array (see pack_tiled_kernel)
-  // pair kernel, optional: rows are laid out as sequences of live_rps rows (a multiple of 256) of which the first
-  // live_n_valid[sequence] are in use; a 256-row tile without a live row is not computed
-  const int* live_n_valid;
-  int live_rps;
+  // pair kernel, optional (prompts of different lengths laid out one after the other): the rows in use, on the device, and
+  // where each row belongs as (sequence, row of it), sequence -1 for the rows behind the last one in its 256-row tile
+  const int* live_rows;
+  const int2* row_map;
   EpiParams ep;
   // EPI_QKV only
   const float* rope_cos;  // [max_seq][64]
@@ -321,10 +321,18 @@ __device__ __forceinline__ void run_epilogue(const Source& src, const GemmParams
     // v heads keep their order.  q heads first, then k heads, then v heads.
     int pos = 0, b = 0;
     if (live) {
-      b = m / p.rows_per_seq;
-      const int r = m % p.rows_per_seq;
+      int r;
+      if (p.row_map != nullptr) {
+        const int2 at = p.row_map[m];
+        live = at.x >= 0;
+        b = live ? at.x : 0;
+        r = at.y;
+      } else {
+        b = m / p.rows_per_seq;
+        r = m % p.rows_per_seq;
+      }
       pos = p.pos_base[b] + r;
-      if (r >= p.n_valid[b]) live = false;
+      if (!live || r >= p.n_valid[b]) live = false;
       else if (pos < 0 || pos >= p.max_seq) {
         atomicOr(p.error_word, ERRW_BAD_POSITION);
         live = false;

@@ -19,7 +19,12 @@ struct RowMap {
   int rows_per_seq;
   int bs;
   int seg;
+  const int* row_off = nullptr;  // rows of sequence b begin at row_off[b] (null: at b * rows_per_seq)
 };
+// First row of sequence b in the activation buffers.
+__device__ __forceinline__ size_t first_row(const RowMap& rm, int b) {
+  return rm.row_off != nullptr ? static_cast<size_t>(rm.row_off[b]) : static_cast<size_t>(b) * rm.rows_per_seq;
+}
 __device__ __forceinline__ int row_kv_limit(const RowMap& rm, int b, int r, int kv_len) {
   if (rm.seg <= 0) return kv_len;
   const int lim = rm.pos_base[b] + (r / rm.seg + 1) * rm.seg;
@@ -53,17 +58,25 @@ __global__ void embed_kernel(const int* __restrict__ ids, const T* __restrict__ 
 // The embeddings of a forward on the tensor-core path: the rows themselves and what a residual epilogue leaves behind for
 // the next matmul (see EpiParams), bf16 copy and sum of squares of every 32-column chunk, from one read of the table.
 // One block per row, 8 columns a thread (d_model is a multiple of 8), four neighbouring lanes a chunk.  Bound by its
-// stores.  As two kernels, the second with 32 columns a thread: 22 us in front of a 32-row forward and 0.85 ms in front of
+// stores.  `row_off` non-null: sequences of rows_per_seq ids of which the first n_valid[b] go to rows row_off[b]...; the ids
+// of the others are looked at all the same.  As two kernels, the second with 32 columns a thread: 22 us in front of a 32-row forward and 0.85 ms in front of
 // a 16384 x 4096 prefill; this one 5 us and 0.10 ms.
 __global__ void __launch_bounds__(256) embed_prep_kernel(const int* __restrict__ ids, const __nv_bfloat16* __restrict__ emb, float* __restrict__ x,
-                                                         __nv_bfloat16* __restrict__ xb, float* __restrict__ ssq, int d, int vocab, uint32_t* error_word) {
+                                                         __nv_bfloat16* __restrict__ xb, float* __restrict__ ssq, int d, int vocab, uint32_t* error_word, const int* __restrict__ row_off,
+                                                         const int* __restrict__ n_valid, int rows_per_seq) {
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
-  const int m = blockIdx.x, n_chunks = (d + 31) / 32;
+  int m = blockIdx.x;
+  const int n_chunks = (d + 31) / 32;
   int id = ids[m];
   if (id < 0 || id >= vocab) {
     if (threadIdx.x == 0) atomicOr(error_word, ERRW_BAD_TOKEN_ID);
     id = 0;
+  }
+  if (row_off != nullptr) {
+    const int b = m / rows_per_seq, r = m - b * rows_per_seq;
+    if (r >= n_valid[b]) return;
+    m = row_off[b] + r;
   }
   const uint4* src = reinterpret_cast<const uint4*>(emb + static_cast<size_t>(id) * d);
   float4* row = reinterpret_cast<float4*>(x + static_cast<size_t>(m) * d);
@@ -992,6 +1005,29 @@ __global__ void prefill_rowmap_kernel(const int* prompt_lens, int bs, int p_max,
   pos_base[b] = 0;
   n_valid[b] = len;
   kv_len[b] = len;
+}
+// Rows of sequences of different lengths laid out one after the other: row_off[b] = sum of n_valid before b, row_off[bs] =
+// all rows, row_map[row] = (sequence, row of it), (-1, 0) from the last row up to the next multiple of 256.  One block per sequence.
+__global__ void __launch_bounds__(256) pack_rows_kernel(const int* __restrict__ n_valid, int bs, int* __restrict__ row_off, int2* __restrict__ row_map) {
+  __shared__ int part[8];
+  const int b = blockIdx.x;
+  int sum = 0;
+  for (int i = threadIdx.x; i < b; i += blockDim.x) sum += n_valid[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  int off = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) off += part[w];
+  const int n = n_valid[b];
+  for (int r = threadIdx.x; r < n; r += blockDim.x) row_map[off + r] = make_int2(b, r);
+  if (threadIdx.x == 0) row_off[b] = off;
+  if (b == bs - 1) {
+    const int all = off + n, end = (all + 255) / 256 * 256;
+    if (threadIdx.x == 0) row_off[bs] = all;
+    for (int r = all + threadIdx.x; r < end; r += blockDim.x) row_map[r] = make_int2(-1, 0);
+  }
 }
 __global__ void add_prefix_kernel(int* prefix_len, int bs, int B) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;

@@ -585,6 +585,46 @@ def test_small_bf16_batch_on_k_cut_pairs_step_locked(lens, gen):
         assert ctx.error_word() == 0
 
 
+@pytest.mark.parametrize("hq,hkv,lens", [(4, 2, [0, 1, 255, 256, 130, 40]), (4, 4, [40, 3, 17, 39] * 5), (4, 4, [33, 96, 64] * 3),
+                                         (8, 2, [700, 1]), (4, 2, [512, 512, 512])])
+def test_ragged_prompts_without_padding(hq, hkv, lens):
+    """Prompts of different lengths enter the cache (and are refreshed) with their rows laid out one after the other:
+    every stored key and value has the bits of the padded layout (which a tapped context keeps), for empty and
+    one-token prompts, sequences that end on, before and behind a 256-row tile, few and many rows per kv head, and
+    equal lengths; a second prompt batch of other lengths leaves no trace of the first."""
+    shape = si.scaled_shape(si.LLADA8B, name="small-ragged", n_layers=2, d_model=256, n_q_heads=hq, n_kv_heads=hkv,
+                            d_ffn=640, vocab=1024, d_head=128)
+    W = si.gen_weights(shape)
+    bs, p_max = len(lens), max(lens)
+    assert bs * p_max > 640
+    rng = np.random.default_rng(bs + p_max)
+    with Ctx(shape, W, block=32, max_batch=bs, max_seq=p_max + 32) as ctx:
+        def stored(n_of):
+            out = []
+            for b, n in enumerate(n_of):
+                for layer in range(shape.n_layers if n else 0):
+                    kv = torch.zeros((2, hkv, n, 128), dtype=torch.float32, device=DEV)
+                    d3.d3_read_kv(ctx.ctx, layer, b, 0, n, kv[0], kv[1])
+                    out.append(kv)
+            return out
+        for n_of in (lens, lens[::-1]):
+            ids = rng.integers(0, shape.vocab - 2, size=(bs, p_max)).astype(np.int32)
+            n0 = d3.d3_launch_count_of(ctx.ctx, "pack_rows_kernel")
+            ctx.prefill(ids, np.array(n_of, dtype=np.int32))
+            got = stored(n_of)
+            d3.d3_refresh_cache(ctx.ctx, bs)
+            again = stored(n_of)
+            assert d3.d3_launch_count_of(ctx.ctx, "pack_rows_kernel") == n0 + 2
+            d3.d3_set_tap(ctx.ctx, 0)
+            ctx.prefill(ids, np.array(n_of, dtype=np.int32))
+            want = stored(n_of)
+            d3.d3_set_tap(ctx.ctx, -1)
+            assert d3.d3_launch_count_of(ctx.ctx, "pack_rows_kernel") == n0 + 2
+            for a, b, c in zip(got, again, want):
+                assert torch.equal(a, c) and torch.equal(b, c)  # (a refresh of the prompt alone is the prefill again)
+        assert ctx.error_word() == 0
+
+
 def test_small_bf16_batch_on_cta_pairs_step_locked():
     """Six sequences x 32 rows = 192 rows per decode forward, 768 padded rows in the prefill, and a vocabulary and
     widths that are multiples of 256: QKV (RoPE + cache write), gate/up (SwiGLU) and the LM head (fused statistics)
