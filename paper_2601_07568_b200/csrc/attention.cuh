@@ -17,6 +17,8 @@ template <typename T, int DH>
 __global__ void __launch_bounds__(THREADS) attn_simt_kernel(const T* __restrict__ q, const T* __restrict__ k_cache,
                                                             const T* __restrict__ v_cache, T* __restrict__ out,
                                                             RowMap rm, int hq, int hkv, int max_seq, float scale) {
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
   __shared__ float Ks[KC][DH + 1];
   __shared__ float Vs[KC][DH + 1];
   __shared__ float Qs[QT][DH];

@@ -1125,21 +1125,35 @@ int run_linear_tc(d3_ctx* c, const void* X, const void* W, int M, int N, int K, 
   return run_linear_tc_bn<128, 1>(c, X, W, M, N, K, epi, ep, ctas_hint, qx, w_tiled);
 }
 
+template <typename T, int EPI>
+int launch_simt(d3_ctx* c, const T* x, const T* w, int M, int N, int K, const EpiParams& ep) {
+  const dim3 grid((N + simt::BN - 1) / simt::BN, (M + simt::BM - 1) / simt::BM);
+  // Fewer 32 x 128 tiles than half the SMs: small tiles (same bits).  A statistic belongs to 128 columns.
+  const bool vec = K % 4 == 0 && reinterpret_cast<uintptr_t>(x) % (4 * sizeof(T)) == 0 && reinterpret_cast<uintptr_t>(w) % (4 * sizeof(T)) == 0;
+  if (vec && grid.x * grid.y * 2 <= static_cast<unsigned>(c->n_sms)) {
+    if constexpr (EPI == EPI_STATS)
+      CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<T, EPI, 4, 128, 64>, dim3(grid.x, (M + 3) / 4), dim3(simt::THREADS), 0, x, w, M, N, K, ep));
+    else
+      CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<T, EPI, 16, 16, 256>, dim3((N + 15) / 16, (M + 15) / 16), dim3(simt::THREADS), 0, x, w, M, N, K, ep));
+    LAUNCHED(c, "gemm_simt_small_kernel");
+    return D3_OK;
+  }
+  CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_kernel<T, EPI>, grid, dim3(simt::THREADS), 0, x, w, M, N, K, ep));
+  LAUNCHED(c, "gemm_simt_kernel");
+  return D3_OK;
+}
 template <typename T>
 int run_linear_simt(d3_ctx* c, const void* X, const void* W, int M, int N, int K, int epi, const EpiParams& ep) {
-  dim3 grid((N + simt::BN - 1) / simt::BN, (M + simt::BM - 1) / simt::BM);
   const T* x = static_cast<const T*>(X);
   const T* w = static_cast<const T*>(W);
   switch (epi) {
-    case EPI_F32: simt::gemm_simt_kernel<T, EPI_F32><<<grid, simt::THREADS, 0, c->stream>>>(x, w, M, N, K, ep); break;
-    case EPI_T: simt::gemm_simt_kernel<T, EPI_T><<<grid, simt::THREADS, 0, c->stream>>>(x, w, M, N, K, ep); break;
-    case EPI_RESID: simt::gemm_simt_kernel<T, EPI_RESID><<<grid, simt::THREADS, 0, c->stream>>>(x, w, M, N, K, ep); break;
-    case EPI_SWIGLU: simt::gemm_simt_kernel<T, EPI_SWIGLU><<<grid, simt::THREADS, 0, c->stream>>>(x, w, M, N, K, ep); break;
-    case EPI_STATS: simt::gemm_simt_kernel<T, EPI_STATS><<<grid, simt::THREADS, 0, c->stream>>>(x, w, M, N, K, ep); break;
-    default: return fail(c, D3_ERR_INVALID_ARG, "unknown epilogue");
+    case EPI_F32: return launch_simt<T, EPI_F32>(c, x, w, M, N, K, ep);
+    case EPI_T: return launch_simt<T, EPI_T>(c, x, w, M, N, K, ep);
+    case EPI_RESID: return launch_simt<T, EPI_RESID>(c, x, w, M, N, K, ep);
+    case EPI_SWIGLU: return launch_simt<T, EPI_SWIGLU>(c, x, w, M, N, K, ep);
+    case EPI_STATS: return launch_simt<T, EPI_STATS>(c, x, w, M, N, K, ep);
   }
-  LAUNCHED(c, "gemm_simt_kernel");
-  return D3_OK;
+  return fail(c, D3_ERR_INVALID_ARG, "unknown epilogue");
 }
 
 int run_linear(d3_ctx* c, const void* X, const void* W, int M, int N, int K, int epi, const EpiParams& ep,
@@ -1162,9 +1176,9 @@ int launch_attention(d3_ctx* c, const void* q, const void* kc, const void* vc, v
   const T* vv = static_cast<const T*>(vc);
   T* oo = static_cast<T*>(out);
   switch (g.d_head) {
-    case 32: attn::attn_simt_kernel<T, 32><<<grid, attn::THREADS, 0, c->stream>>>(qq, kk, vv, oo, rm, g.n_q_heads, g.n_kv_heads, g.max_seq, scale); break;
-    case 64: attn::attn_simt_kernel<T, 64><<<grid, attn::THREADS, 0, c->stream>>>(qq, kk, vv, oo, rm, g.n_q_heads, g.n_kv_heads, g.max_seq, scale); break;
-    case 128: attn::attn_simt_kernel<T, 128><<<grid, attn::THREADS, 0, c->stream>>>(qq, kk, vv, oo, rm, g.n_q_heads, g.n_kv_heads, g.max_seq, scale); break;
+    case 32: CUDA_TRY(c, launch_pdl(c, attn::attn_simt_kernel<T, 32>, grid, dim3(attn::THREADS), 0, qq, kk, vv, oo, rm, g.n_q_heads, g.n_kv_heads, g.max_seq, scale)); break;
+    case 64: CUDA_TRY(c, launch_pdl(c, attn::attn_simt_kernel<T, 64>, grid, dim3(attn::THREADS), 0, qq, kk, vv, oo, rm, g.n_q_heads, g.n_kv_heads, g.max_seq, scale)); break;
+    case 128: CUDA_TRY(c, launch_pdl(c, attn::attn_simt_kernel<T, 128>, grid, dim3(attn::THREADS), 0, qq, kk, vv, oo, rm, g.n_q_heads, g.n_kv_heads, g.max_seq, scale)); break;
     default: return fail(c, D3_ERR_UNSUPPORTED, "d_head must be 32, 64 or 128");
   }
   LAUNCHED(c, "attn_simt_kernel");
@@ -1590,9 +1604,9 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
       TRY(run_linear(c, normed, c->wqkv[l], M, nq + 2 * nkv, d, EPI_F32, ep, 0, nullptr, D3_PROF_GEMM_QKV, c->w_tiled));
       ProfScope ps(c, D3_PROF_OTHER);
       if (c->is_bf16)
-        rope_kv_kernel<bf16><<<M, 256, 0, c->stream>>>(c->qkv_f32, static_cast<bf16*>(c->q), static_cast<bf16*>(k_plane(c, l)), static_cast<bf16*>(v_plane(c, l)), c->rope_cos, c->rope_sin, rm, g.n_q_heads, g.n_kv_heads, g.d_head, g.max_seq, c->error_word);
+        CUDA_TRY(c, launch_pdl(c, rope_kv_kernel<bf16>, dim3(M), dim3(256), 0, c->qkv_f32, static_cast<bf16*>(c->q), static_cast<bf16*>(k_plane(c, l)), static_cast<bf16*>(v_plane(c, l)), c->rope_cos, c->rope_sin, rm, g.n_q_heads, g.n_kv_heads, g.d_head, g.max_seq, c->error_word));
       else
-        rope_kv_kernel<float><<<M, 256, 0, c->stream>>>(c->qkv_f32, static_cast<float*>(c->q), static_cast<float*>(k_plane(c, l)), static_cast<float*>(v_plane(c, l)), c->rope_cos, c->rope_sin, rm, g.n_q_heads, g.n_kv_heads, g.d_head, g.max_seq, c->error_word);
+        CUDA_TRY(c, launch_pdl(c, rope_kv_kernel<float>, dim3(M), dim3(256), 0, c->qkv_f32, static_cast<float*>(c->q), static_cast<float*>(k_plane(c, l)), static_cast<float*>(v_plane(c, l)), c->rope_cos, c->rope_sin, rm, g.n_q_heads, g.n_kv_heads, g.d_head, g.max_seq, c->error_word));
       LAUNCHED(c, "rope_kv_kernel");
     }
     TRY(run_attention(c, c->q, l, c->o, rm));

@@ -3,15 +3,92 @@
 // and a debugging cross-check for bf16.  Tile 32 x 128, K slabs of 32, 256 threads, 4 x 4 outputs each.
 #pragma once
 #include "common.cuh"
+#include "ptx_sm100.cuh"
 
 namespace d3 {
 namespace simt {
 
 constexpr int BM = 32, BN = 128, BK = 32, THREADS = 256;
 
+// Epilogue of a BM_ x BN_ tile of sums in shared memory whose first element is (m0, n0).  (EPI_STATS: BN_ is 128.)
+template <typename T, int EPI, int BM_, int BN_>
+__device__ __forceinline__ void simt_epilogue(const float (*Cs)[BN_ + 1], int m0, int n0, int M, int N, const EpiParams& ep) {
+  const int t = threadIdx.x;
+  if constexpr (EPI == EPI_F32 || EPI == EPI_RESID || EPI == EPI_T) {
+    for (int e = t; e < BM_ * BN_; e += THREADS) {
+      int r = e / BN_, c = e % BN_;
+      int m = m0 + r, n = n0 + c;
+      if (m < M && n < N) {
+        size_t o = static_cast<size_t>(m) * ep.ldy + n;
+        if constexpr (EPI == EPI_F32) static_cast<float*>(ep.y)[o] = Cs[r][c] * ep.scale;
+        else if constexpr (EPI == EPI_RESID) static_cast<float*>(ep.y)[o] += Cs[r][c];
+        else static_cast<T*>(ep.y)[o] = TypeOps<T>::from_f(Cs[r][c]);
+      }
+    }
+  } else if constexpr (EPI == EPI_SWIGLU) {
+    // packed rows of W: 2j = gate row of hidden unit j, 2j+1 = its up row
+    const int F = N / 2;
+    for (int e = t; e < BM_ * (BN_ / 2); e += THREADS) {
+      int r = e / (BN_ / 2), c = e % (BN_ / 2);
+      int m = m0 + r, h = n0 / 2 + c;
+      if (m < M && h < F)
+        static_cast<T*>(ep.y)[static_cast<size_t>(m) * ep.ldy + h] =
+            TypeOps<T>::from_f(silu_f(Cs[r][2 * c]) * Cs[r][2 * c + 1]);
+    }
+  } else if constexpr (EPI == EPI_STATS) {
+    // one warp per row (8 warps, 4 rows each): lanes stride the 128 columns, fixed shuffle tree
+    const int warp = t / 32, lane = t % 32;
+    for (int r = warp; r < BM_; r += THREADS / 32) {
+      int m = m0 + r;
+      SoftStat st = stat_empty();
+      for (int c = lane; c < BN_; c += 32) {
+        int n = n0 + c;
+        if (n < N && n != ep.mask_id) stat_add(st, Cs[r][c] * ep.scale, n);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        SoftStat other;
+        other.m = __shfl_xor_sync(0xffffffffu, st.m, o);
+        other.z = __shfl_xor_sync(0xffffffffu, st.z, o);
+        other.s = __shfl_xor_sync(0xffffffffu, st.s, o);
+        other.a = __shfl_xor_sync(0xffffffffu, st.a, o);
+        st = (lane & o) ? stat_merge(other, st) : stat_merge(st, other);
+      }
+      if (lane == 0 && m < M)
+        ep.stat_part[static_cast<size_t>(m) * ep.n_tiles + blockIdx.x] =
+            make_float4(st.m, st.z, st.s, __int_as_float(st.a));
+      if (ep.sample_part != nullptr && m < M) {  // temperature sampling: largest l + T * g of the tile
+        SampleStat sp = sample_empty();
+        const SampleRow sr = sample_row(ep, m);
+        for (int c = lane; c < BN_; c += 32) {
+          const int n = n0 + c;
+          if (n < N && n != ep.mask_id) {
+            const uint4 bits = philox4x32_10(make_uint4(static_cast<uint32_t>(n >> 2), sr.pos, sr.step, sr.seq), ep.seed_lo, ep.seed_hi);
+            const uint32_t w = (n & 3) == 0 ? bits.x : (n & 3) == 1 ? bits.y : (n & 3) == 2 ? bits.z : bits.w;
+            const float l = Cs[r][c] * ep.scale;
+            sample_add(sp, __fadd_rn(l, __fmul_rn(ep.temperature, gumbel_from_bits(w))), l, n);
+          }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          SampleStat other;
+          other.pm = __shfl_xor_sync(0xffffffffu, sp.pm, o);
+          other.la = __shfl_xor_sync(0xffffffffu, sp.la, o);
+          other.pa = __shfl_xor_sync(0xffffffffu, sp.pa, o);
+          sp = sample_merge(sp, other);
+        }
+        if (lane == 0)
+          ep.sample_part[static_cast<size_t>(m) * ep.n_tiles + blockIdx.x] = make_float4(sp.pm, sp.la, __int_as_float(sp.pa), 0.f);
+      }
+    }
+  }
+}
+
 template <typename T, int EPI>
 __global__ void __launch_bounds__(THREADS) gemm_simt_kernel(const T* __restrict__ X, const T* __restrict__ W, int M,
                                                             int N, int K, EpiParams ep) {
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
   __shared__ float Xs[BM][BK + 1];
   __shared__ float Ws[BN][BK + 1];
   __shared__ float Cs[BM][BN + 1];
@@ -55,74 +132,62 @@ __global__ void __launch_bounds__(THREADS) gemm_simt_kernel(const T* __restrict_
     for (int j = 0; j < 4; ++j) Cs[ty * 4 + i][tx + 32 * j] = acc[i][j];
   __syncthreads();
 
-  if constexpr (EPI == EPI_F32 || EPI == EPI_RESID || EPI == EPI_T) {
-    for (int e = t; e < BM * BN; e += THREADS) {
-      int r = e / BN, c = e % BN;
-      int m = m0 + r, n = n0 + c;
-      if (m < M && n < N) {
-        size_t o = static_cast<size_t>(m) * ep.ldy + n;
-        if constexpr (EPI == EPI_F32) static_cast<float*>(ep.y)[o] = Cs[r][c] * ep.scale;
-        else if constexpr (EPI == EPI_RESID) static_cast<float*>(ep.y)[o] += Cs[r][c];
-        else static_cast<T*>(ep.y)[o] = TypeOps<T>::from_f(Cs[r][c]);
-      }
-    }
-  } else if constexpr (EPI == EPI_SWIGLU) {
-    // packed rows of W: 2j = gate row of hidden unit j, 2j+1 = its up row
-    const int F = N / 2;
-    for (int e = t; e < BM * 64; e += THREADS) {
-      int r = e / 64, c = e % 64;
-      int m = m0 + r, h = n0 / 2 + c;
-      if (m < M && h < F)
-        static_cast<T*>(ep.y)[static_cast<size_t>(m) * ep.ldy + h] =
-            TypeOps<T>::from_f(silu_f(Cs[r][2 * c]) * Cs[r][2 * c + 1]);
-    }
-  } else if constexpr (EPI == EPI_STATS) {
-    // one warp per row (8 warps, 4 rows each): lanes stride the 128 columns, fixed shuffle tree
-    const int warp = t / 32, lane = t % 32;
-    for (int r = warp; r < BM; r += THREADS / 32) {
-      int m = m0 + r;
-      SoftStat st = stat_empty();
-      for (int c = lane; c < BN; c += 32) {
-        int n = n0 + c;
-        if (n < N && n != ep.mask_id) stat_add(st, Cs[r][c] * ep.scale, n);
-      }
+  simt_epilogue<T, EPI, BM, BN>(Cs, m0, n0, M, N, ep);
+}
+
+// The same sums, bit for bit (one chain of fused multiply-adds per output, ascending in k), for matmuls whose 32 x 128 tiles
+// would leave most SMs idle: BM_ x BN_ tiles, 256 threads, KC columns of X and W in shared memory at a time, read four at
+// a time.  What bounds it is the chain of K multiply-adds and, per KC columns, one trip to memory.  A 16 x 128 x 512
+// product took 50 us as one 32 x 128 tile on one SM; as 8 tiles of 16 x 16 it takes 6.  K % 4 == 0, rows aligned to 4 elements.
+template <typename T, int EPI, int BM_, int BN_, int KC>
+__global__ void __launch_bounds__(THREADS) gemm_simt_small_kernel(const T* __restrict__ X, const T* __restrict__ W, int M, int N, int K, EpiParams ep) {
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
+  constexpr int OUT = BM_ * BN_ / THREADS, ROWS = THREADS / BN_;
+  __shared__ __align__(16) float Xs[BM_][KC + 4];
+  __shared__ __align__(16) float Ws[BN_][KC + 4];
+  __shared__ float Cs[BM_][BN_ + 1];
+  const int m0 = blockIdx.y * BM_, n0 = blockIdx.x * BN_;
+  const int t = threadIdx.x, c = t % BN_, r0 = t / BN_;
+  float acc[OUT];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        SoftStat other;
-        other.m = __shfl_xor_sync(0xffffffffu, st.m, o);
-        other.z = __shfl_xor_sync(0xffffffffu, st.z, o);
-        other.s = __shfl_xor_sync(0xffffffffu, st.s, o);
-        other.a = __shfl_xor_sync(0xffffffffu, st.a, o);
-        st = (lane & o) ? stat_merge(other, st) : stat_merge(st, other);
+  for (int i = 0; i < OUT; ++i) acc[i] = 0.f;
+  for (int k0 = 0; k0 < K; k0 += KC) {
+    auto stage = [&](float* dst, const T* src, int row, int rows, int k) {
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (row < rows && k < K) {
+        if constexpr (sizeof(T) == 4) {
+          v = *reinterpret_cast<const float4*>(src + static_cast<size_t>(row) * K + k);
+        } else {
+          const uint2 w = *reinterpret_cast<const uint2*>(src + static_cast<size_t>(row) * K + k);
+          v = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+        }
       }
-      if (lane == 0 && m < M)
-        ep.stat_part[static_cast<size_t>(m) * ep.n_tiles + blockIdx.x] =
-            make_float4(st.m, st.z, st.s, __int_as_float(st.a));
-      if (ep.sample_part != nullptr && m < M) {  // temperature sampling: largest l + T * g of the tile
-        SampleStat sp = sample_empty();
-        const SampleRow sr = sample_row(ep, m);
-        for (int c = lane; c < BN; c += 32) {
-          const int n = n0 + c;
-          if (n < N && n != ep.mask_id) {
-            const uint4 bits = philox4x32_10(make_uint4(static_cast<uint32_t>(n >> 2), sr.pos, sr.step, sr.seq), ep.seed_lo, ep.seed_hi);
-            const uint32_t w = (n & 3) == 0 ? bits.x : (n & 3) == 1 ? bits.y : (n & 3) == 2 ? bits.z : bits.w;
-            const float l = Cs[r][c] * ep.scale;
-            sample_add(sp, __fadd_rn(l, __fmul_rn(ep.temperature, gumbel_from_bits(w))), l, n);
-          }
-        }
+      *reinterpret_cast<float4*>(dst) = v;
+    };
+#pragma unroll 4
+    for (int e = t; e < BM_ * (KC / 4); e += THREADS) stage(&Xs[e / (KC / 4)][e % (KC / 4) * 4], X, m0 + e / (KC / 4), M, k0 + e % (KC / 4) * 4);
+#pragma unroll 4
+    for (int e = t; e < BN_ * (KC / 4); e += THREADS) stage(&Ws[e / (KC / 4)][e % (KC / 4) * 4], W, n0 + e / (KC / 4), N, k0 + e % (KC / 4) * 4);
+    __syncthreads();
+#pragma unroll 8
+    for (int k = 0; k < KC; k += 4) {
+      const float4 w = *reinterpret_cast<const float4*>(&Ws[c][k]);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          SampleStat other;
-          other.pm = __shfl_xor_sync(0xffffffffu, sp.pm, o);
-          other.la = __shfl_xor_sync(0xffffffffu, sp.la, o);
-          other.pa = __shfl_xor_sync(0xffffffffu, sp.pa, o);
-          sp = sample_merge(sp, other);
-        }
-        if (lane == 0)
-          ep.sample_part[static_cast<size_t>(m) * ep.n_tiles + blockIdx.x] = make_float4(sp.pm, sp.la, __int_as_float(sp.pa), 0.f);
+      for (int i = 0; i < OUT; ++i) {
+        const float4 x = *reinterpret_cast<const float4*>(&Xs[r0 + i * ROWS][k]);
+        acc[i] = fmaf(x.x, w.x, acc[i]);
+        acc[i] = fmaf(x.y, w.y, acc[i]);
+        acc[i] = fmaf(x.z, w.z, acc[i]);
+        acc[i] = fmaf(x.w, w.w, acc[i]);
       }
     }
+    __syncthreads();
   }
+#pragma unroll
+  for (int i = 0; i < OUT; ++i) Cs[r0 + i * ROWS][c] = acc[i];
+  __syncthreads();
+  simt_epilogue<T, EPI, BM_, BN_>(Cs, m0, n0, M, N, ep);
 }
 
 }  // namespace simt

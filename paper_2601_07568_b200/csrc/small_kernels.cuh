@@ -180,6 +180,8 @@ __global__ void rope_kv_kernel(const float* __restrict__ qkv, T* __restrict__ q_
                                T* __restrict__ v_cache, const float* __restrict__ rope_cos,
                                const float* __restrict__ rope_sin, RowMap rm, int hq, int hkv, int dh, int max_seq,
                                uint32_t* error_word) {
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
   const int m = blockIdx.x;
   const int b = m / rm.rows_per_seq, r = m % rm.rows_per_seq;
   if (r >= rm.n_valid[b]) return;

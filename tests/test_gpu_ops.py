@@ -141,6 +141,29 @@ def test_linear_bf16_weights_as_rows(ctx_bf16, m, n, k, cluster):
     assert ctx_bf16.error_word() == 0
 
 
+@pytest.mark.parametrize("m,n,k", [(1, 16, 4), (16, 128, 512), (17, 130, 260), (33, 384, 128), (48, 200, 1028), (5, 514, 64)])
+@pytest.mark.parametrize("epi", [0, 2, 3])
+def test_linear_fp32_small_tiles_same_bits(ctx_f32, m, n, k, epi):
+    """fp32 matmuls of few tiles run on 16 x 16 tiles: against the fp64 product, and bit for bit what a matmul of many
+    rows (the 32 x 128 tiles) gives for the same rows, since a sum is one chain of multiply-adds in either."""
+    rng = np.random.default_rng(m + n + k + epi)
+    big = (74 * 32 // ((n + 127) // 128) + 32) // 32 * 32 + 32  # rows at which the tiles are more than half the SMs
+    x = rng.standard_normal((big, k)).astype(np.float32)
+    w = (rng.standard_normal((n, k)) * 0.05).astype(np.float32)
+    y0 = rng.standard_normal((big, n // 2 if epi == 3 else n)).astype(np.float32)
+    xd, wd = torch.from_numpy(x).to(DEV), torch.from_numpy(w).to(DEV)
+    few, many = torch.from_numpy(y0[:m]).to(DEV), torch.from_numpy(y0).to(DEV)
+    n0 = d3.d3_launch_count_of(ctx_f32.ctx, "gemm_simt_small_kernel")
+    d3.d3_op_linear(ctx_f32.ctx, xd[:m].contiguous(), wd, few, epi, 0)
+    assert d3.d3_launch_count_of(ctx_f32.ctx, "gemm_simt_small_kernel") == n0 + 1
+    d3.d3_op_linear(ctx_f32.ctx, xd, wd, many, epi, 0)
+    assert d3.d3_launch_count_of(ctx_f32.ctx, "gemm_simt_small_kernel") == n0 + 1
+    assert torch.equal(few, many[:m])
+    ref = x[:m].astype(np.float64) @ w.T.astype(np.float64)
+    want = ref + y0[:m] if epi == 2 else swiglu_ref(ref, n) if epi == 3 else ref
+    assert np.max(np.abs(few.cpu().numpy() - want)) <= 1e-6 * np.sqrt(k) * (np.abs(ref).max() ** (2 if epi == 3 else 1) + 1) + 1e-6
+
+
 @pytest.mark.parametrize("m,n,k", [(1, 256, 64), (32, 512, 4096), (33, 3584, 3584), (96, 256, 8192), (128, 12288, 512), (129, 4096, 1024),
                                    (200, 768, 2048), (256, 4096, 4096), (257, 1280, 1920), (501, 3584, 1024), (640, 19200, 256)])
 def test_linear_bf16_k_cut_pairs(ctx_bf16, m, n, k):
