@@ -1460,6 +1460,15 @@ bool sk_forward_usable(const d3_ctx* c, int M) {
   return M <= SK_FORWARD_ROWS;
 }
 
+// The LM head of a decode forward on gemm_sk_kernel.
+bool sk_head_usable(const d3_ctx* c, int M) {
+  if (c->tune_sk == 0 || !c->use_tc || !c->fold_norm || !c->w_tiled || M > tc::SK_MAX_ROWS || !sk_shape_ok(c->cfg.vocab, c->cfg.d_model)) return false;
+  if (c->tune_sk == 1) return true;
+  if (c->tune_strip != 0 || c->tune_no_cluster || c->tune_xt == 0 || c->tune_cta_pairs == 0 || c->tune_wide_tiles >= 0 || c->tune_pair >= 0 ||
+      c->tune_producers > 0 || c->tune_ring_kb > 0 || c->tune_ctas_per_sm > 0) return false;
+  return M <= SK_FORWARD_ROWS;
+}
+
 // Can the rows of a ragged forward be laid out without padding?  Where all its matmuls run on CTA pairs, which take the
 // number of rows from the device (32 prompts of 128..512 tokens, 16384 padded rows of which 10240 are in use: 200.5 -> 137.6 ms).
 // (A tapped forward keeps the layout that d3_read_tap describes.)
@@ -1521,10 +1530,32 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
     ep.yb = static_cast<bf16*>(c->xb); ep.ssq_out = c->ssq;
   };
 
+  // The LM head with its statistics: an operand of the same persistent launches where those run.
+  auto head_epi = [&]() {
+    EpiParams ep;
+    ep.scale = g.logit_scale; ep.mask_id = g.mask_id; ep.stat_part = c->stat_part; ep.n_tiles = (g.vocab + 127) / 128;
+    if (c->temperature > 0.f) {  // temperature sampling: Gumbel noise keyed by (seed; sequence, position, step)
+      ep.sample_part = c->sample_part;
+      ep.temperature = c->temperature;
+      ep.seed_lo = static_cast<uint32_t>(c->seed & 0xffffffffull);
+      ep.seed_hi = static_cast<uint32_t>(c->seed >> 32);
+      ep.pos_base = c->pos_base;
+      ep.rows_per_seq = rows_per_seq;
+      ep.draw_step = c->draw_step;
+      ep.draw_step_add = c->draw_step_add;
+    }
+    after_norm(ep);
+    return ep;
+  };
+  const bool head_sk = head == 1 && sk_head_usable(c, M);
+  bool head_done = false;
+  const SkMatmul head_mm{c->xb, c->lm_head, g.vocab, d, EPI_STATS, head == 1 ? head_epi() : EpiParams{}, nullptr};
+
   if (chain_usable(c, bs, rows_per_seq, seg)) {
     // Skinny decode forward: all layers in one persistent launch (chain.cuh); a tapped layer cuts it.
     if (!c->chain_prog_ready) TRY(chain_build_program(c));
     CUDA_TRY(c, cudaMemsetAsync(c->chain_sync, 0, sizeof(unsigned int) * static_cast<size_t>(c->chain_prog_ops), c->stream));
+    if (head_sk) TRY(sk_begin(c, 1));
     const int n_ops = c->chain_prog_ops;
     const bool tap = c->tap_layer >= 0 && c->tap_layer < g.n_layers && M <= c->tap_rows;
     if (!tap) {
@@ -1538,10 +1569,15 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
       CUDA_TRY(c, cudaMemcpyAsync(c->tap_out, c->x, sizeof(float) * M * d, cudaMemcpyDeviceToDevice, c->stream));
       if (o_out < n_ops) TRY(run_chain(c, o_out, n_ops, rm));
     }
+    if (head_sk) {
+      ProfScope ps(c, D3_PROF_GEMM_HEAD);
+      TRY(run_sk(c, &head_mm, 1, M));
+      head_done = true;
+    }
   } else if (sk_forward_usable(c, M)) {
     // Decode-sized forward: the matmuls between two attention kernels (O-proj, gate/up, down, the next layer's QKV) in
     // one launch of resident CTA pairs.  The residual stream between two launches is a layer's output.
-    TRY(sk_begin(c, 4 * g.n_layers));
+    TRY(sk_begin(c, 4 * g.n_layers + 1));
     auto qkv = [&](int l, QkvExtra& qx) {
       EpiParams ep;
       ep.y = c->q; ep.ldy = nq;
@@ -1558,7 +1594,7 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
       }
       return static_cast<int>(D3_OK);
     };
-    const int classes[4] = {D3_PROF_GEMM_O, D3_PROF_GEMM_GATE_UP, D3_PROF_GEMM_DOWN, D3_PROF_GEMM_QKV};
+    int classes[4] = {D3_PROF_GEMM_O, D3_PROF_GEMM_GATE_UP, D3_PROF_GEMM_DOWN, D3_PROF_GEMM_QKV};
     const bool tap = M <= c->tap_rows;
     QkvExtra qx{};
     {
@@ -1582,7 +1618,12 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
                         {}};
       const bool more = l + 1 < g.n_layers;
       if (more) mm[3] = qkv(l + 1, qx);
-      TRY(launch(mm, classes, more ? 4 : 3));
+      if (!more && head_sk) {
+        mm[3] = head_mm;
+        classes[3] = D3_PROF_GEMM_HEAD;
+        head_done = true;
+      }
+      TRY(launch(mm, classes, more || head_sk ? 4 : 3));
       if (l == c->tap_layer && tap)
         CUDA_TRY(c, cudaMemcpyAsync(c->tap_out, c->x, sizeof(float) * M * d, cudaMemcpyDeviceToDevice, c->stream));
     }
@@ -1635,23 +1676,13 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   if (head == 0) return D3_OK;
   if (!c->fold_norm) TRY(run_rmsnorm(c, c->x, c->final_norm, c->xn, M));
   if (head == 1) {
-    const int n_tiles = (g.vocab + 127) / 128;
-    EpiParams ep;
-    ep.scale = g.logit_scale; ep.mask_id = g.mask_id; ep.stat_part = c->stat_part; ep.n_tiles = n_tiles;
-    const bool sampled = c->temperature > 0.f;
-    if (sampled) {  // temperature sampling: Gumbel noise keyed by (seed; sequence, position, step)
-      ep.sample_part = c->sample_part;
-      ep.temperature = c->temperature;
-      ep.seed_lo = static_cast<uint32_t>(c->seed & 0xffffffffull);
-      ep.seed_hi = static_cast<uint32_t>(c->seed >> 32);
-      ep.pos_base = c->pos_base;
-      ep.rows_per_seq = rows_per_seq;
-      ep.draw_step = c->draw_step;
-      ep.draw_step_add = c->draw_step_add;
+    if (head_sk && !head_done) {
+      TRY(sk_begin(c, 1));
+      ProfScope ps(c, D3_PROF_GEMM_HEAD);
+      TRY(run_sk(c, &head_mm, 1, M));
     }
-    after_norm(ep);
-    TRY(run_linear(c, normed, c->lm_head, M, g.vocab, d, EPI_STATS, ep, 0, nullptr, D3_PROF_GEMM_HEAD, c->w_tiled));
-    TRY(run_stats_merge(c, M, n_tiles, c->conf, c->ent, c->argmax, sampled));
+    if (!head_sk) TRY(run_linear(c, normed, c->lm_head, M, g.vocab, d, EPI_STATS, head_epi(), 0, nullptr, D3_PROF_GEMM_HEAD, c->w_tiled));
+    TRY(run_stats_merge(c, M, (g.vocab + 127) / 128, c->conf, c->ent, c->argmax, c->temperature > 0.f));
   } else {
     EpiParams ep;
     ep.y = logits; ep.ldy = g.vocab; ep.scale = g.logit_scale;
@@ -1764,7 +1795,7 @@ extern "C" int d3_create(const d3_config* cfg, void* cuda_stream, d3_ctx** out) 
     A_(c->partial, c->partial_slots * 128 * 128 * sizeof(float));
     c->n_tile_count = 1 << 16;
     A_(c->tile_count, sizeof(int) * c->n_tile_count);
-    c->sk_sync_cap = static_cast<size_t>(4 * g.n_layers) * SK_OP_COUNTERS;
+    c->sk_sync_cap = static_cast<size_t>(4 * g.n_layers + 1) * SK_OP_COUNTERS;
     A_(c->sk_sync, sizeof(unsigned int) * c->sk_sync_cap);
   }
   if (c->use_tc && g.d_head == 128) {

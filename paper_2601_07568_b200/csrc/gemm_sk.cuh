@@ -216,6 +216,83 @@ __device__ __forceinline__ void sk_row_rstd16(const EpiParams& ep, int m0, int M
   if ((lane & 1) == 0) rs[lane >> 1] = rsqrtf(a[0] * ep.inv_k + ep.rms_eps);
 }
 
+// LM head: softmax statistics of ROWS rows over this CTA's 128 columns, and with a temperature the largest perturbed logit
+// (one Philox call covers a lane's four columns).  `l`: the logits.
+template <int ROWS>
+__device__ __forceinline__ void sk_stats(const SkParams& p, const SkOp& o, float4 (&l)[ROWS], const bool (&live)[ROWS], int m, int n, int lane) {
+  const int gone = o.ep.mask_id - n;  // which of the lane's columns is the mask token, if any
+  float mx[ROWS], z[ROWS], t[ROWS];
+  int a[ROWS];
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) {
+    float v[4] = {l[u].x, l[u].y, l[u].z, l[u].w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q == gone) v[q] = -INFINITY;
+    l[u] = make_float4(v[0], v[1], v[2], v[3]);
+    mx[u] = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));
+  }
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1)
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u) mx[u] = fmaxf(mx[u], __shfl_xor_sync(0xffffffffu, mx[u], d));
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u) {
+    const float v[4] = {l[u].x, l[u].y, l[u].z, l[u].w};
+    z[u] = t[u] = 0.f;
+    a[u] = 0x7fffffff;
+#pragma unroll
+    for (int q = 3; q >= 0; --q) {
+      if (q == gone) continue;
+      const float d = v[q] == INFINITY ? 0.f : v[q] - mx[u], e = __expf(d);
+      z[u] += e;
+      t[u] += e * d;
+      if (v[q] == mx[u]) a[u] = n + q;
+    }
+    a[u] = __reduce_min_sync(0xffffffffu, a[u]);
+  }
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1)
+#pragma unroll
+    for (int u = 0; u < ROWS; ++u) {
+      z[u] += __shfl_xor_sync(0xffffffffu, z[u], d);
+      t[u] += __shfl_xor_sync(0xffffffffu, t[u], d);
+    }
+  const int tile = n >> 7;
+#pragma unroll
+  for (int u = 0; u < ROWS; ++u)
+    if (live[u] && lane == 0)
+      o.ep.stat_part[static_cast<size_t>(m + u * SK_EPI_WARPS) * o.ep.n_tiles + tile] = make_float4(mx[u], z[u], t[u], __int_as_float(a[u]));
+  if (o.ep.sample_part == nullptr) return;
+#pragma unroll 1
+  for (int u = 0; u < ROWS; ++u) {
+    float4 lu = l[0];
+    bool alive = live[0];
+#pragma unroll
+    for (int q = 1; q < ROWS; ++q)
+      if (q == u) { lu = l[q]; alive = live[q]; }
+    if (!alive) continue;  // warp-uniform
+    const int row = m + u * SK_EPI_WARPS;
+    const SampleRow sr = sample_row(o.ep, row);
+    const uint4 bits = philox4x32_10(make_uint4(static_cast<uint32_t>(n >> 2), sr.pos, sr.step, sr.seq), o.ep.seed_lo, o.ep.seed_hi);
+    const uint32_t w[4] = {bits.x, bits.y, bits.z, bits.w};
+    const float v[4] = {lu.x, lu.y, lu.z, lu.w};
+    SampleStat sp = sample_empty();
+#pragma unroll
+    for (int q = 0; q < 4; ++q)  // product and sum rounded separately
+      if (q != gone) sample_add(sp, __fadd_rn(v[q], __fmul_rn(o.ep.temperature, gumbel_from_bits(w[q]))), v[q], n + q);
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) {
+      SampleStat other;
+      other.pm = __shfl_xor_sync(0xffffffffu, sp.pm, d);
+      other.la = __shfl_xor_sync(0xffffffffu, sp.la, d);
+      other.pa = __shfl_xor_sync(0xffffffffu, sp.pa, d);
+      sp = sample_merge(sp, other);
+    }
+    if (lane == 0) o.ep.sample_part[static_cast<size_t>(row) * o.ep.n_tiles + tile] = make_float4(sp.pm, sp.la, __int_as_float(sp.pa), 0.f);
+  }
+}
+
 // Warp w takes rows w, w + SK_EPI_WARPS, ..., ROWS at a time with up to BATCH partials of each in flight.  No branch on
 // a single row's state but around its stores: the rows' instructions interleave.
 template <int ROWS, int BATCH>
@@ -306,10 +383,13 @@ __device__ __forceinline__ void sk_finish(const SkParams& p, const SkOp& o, cons
     }
 #pragma unroll
     for (int u = 0; u < ROWS; ++u) {
-      const float rs = live[u] ? rs_tab[m + u * SK_EPI_WARPS] : 0.f;
+      float rs = live[u] ? rs_tab[m + u * SK_EPI_WARPS] : 0.f;
+      if (epi == EPI_STATS) rs *= o.ep.scale;  // (one factor, as in the other kernels' logits)
       acc[u] = make_float4(acc[u].x * rs, acc[u].y * rs, acc[u].z * rs, acc[u].w * rs);
     }
-    if (epi == EPI_SWIGLU) {
+    if (epi == EPI_STATS) {
+      sk_stats<ROWS>(p, o, acc, live, m, n, lane);
+    } else if (epi == EPI_SWIGLU) {
       // packed rows of W: 2j = gate row of hidden unit j, 2j + 1 = its up row
       __nv_bfloat16* y = static_cast<__nv_bfloat16*>(o.ep.y) + static_cast<size_t>(m) * ld + n / 2;
 #pragma unroll
