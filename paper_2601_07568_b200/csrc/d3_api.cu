@@ -55,7 +55,9 @@ struct d3_ctx {
   size_t kv_layer_elems = 0;  // elements of one K (or V) plane of one layer
   float *rope_cos = nullptr, *rope_sin = nullptr;
   // workspaces
-  int max_rows = 0;
+  int max_rows = 0;       // rows of a prompt or window forward
+  int ws_rows = 0;        // rows the workspaces hold: fused forwards of a batch may have more
+  int fuse_rows = 0;      // rows of the largest fused forward the workspaces were sized for
   float* x = nullptr;
   void* xn = nullptr;
   float* qkv_f32 = nullptr;
@@ -290,6 +292,10 @@ int get_tmap(d3_ctx* c, const void* ptr, int rows, int cols, int box_rows, const
 // Up to this many rows a decode forward is bound by weight streaming, so twice the rows cost the same:
 // d3_generate then fuses a block's finalize forward with the next block's first denoise step.
 constexpr long long FUSE_MAX_ROWS = 64;
+// Batches, where every sequence pays the doubled rows: a fused forward instead of two where the share f of sequences at
+// a border outweighs them, f c(R) > c(2R) - c(R) with c the forward's time (8B shape, ms: c(96) 4.0, c(128) 4.1, c(192)
+// 5.0, c(256) 5.4, c(512) 10.0): half of the live sequences up to 256 fused rows, all of them up to 512.
+constexpr long long FUSE_HALF_ROWS = 256, FUSE_ALL_ROWS = 512;
 
 // ---- matmul dispatch
 struct QkvExtra {
@@ -1489,7 +1495,7 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   const d3_config& g = c->cfg;
   const int M = bs * rows_per_seq;
   if (M == 0) return D3_OK;
-  if (M > c->max_rows) return fail(c, D3_ERR_SHAPE, "forward over more rows than the workspaces hold");
+  if (M > c->ws_rows) return fail(c, D3_ERR_SHAPE, "forward over more rows than the workspaces hold");
   const int d = g.d_model, nq = g.n_q_heads * g.d_head, nkv = g.n_kv_heads * g.d_head, f = g.d_ffn;
   RowMap rm{c->pos_base, c->n_valid, c->kv_len, rows_per_seq, bs, seg};
   c->last_rows = M;
@@ -1757,7 +1763,11 @@ extern "C" int d3_create(const d3_config* cfg, void* cuda_stream, d3_ctx** out) 
   // on the skinny kernels (128 rows)
   dec_rows = std::max<long long>(dec_rows, 128);
   c->max_rows = static_cast<int>(std::max(pre_rows, dec_rows));
-  const size_t R = c->max_rows;
+  // (a batch's fused forwards; what callers may ask for stays as above)
+  c->fuse_rows = static_cast<int>(std::min<long long>(2ll * g.max_batch * g.block, FUSE_ALL_ROWS));
+  const long long head_rows = c->use_tc ? std::max<long long>(dec_rows, c->fuse_rows) : dec_rows;
+  c->ws_rows = static_cast<int>(std::max<long long>(c->max_rows, head_rows));
+  const size_t R = c->ws_rows;
 #define A_(ptr, bytes)                                                         \
   do {                                                                         \
     int rc_ = dev_alloc(c, reinterpret_cast<void**>(&(ptr)), (bytes));         \
@@ -1778,11 +1788,11 @@ extern "C" int d3_create(const d3_config* cfg, void* cuda_stream, d3_ctx** out) 
   A_(c->o, c->esz * R * nq);
   A_(c->h, c->esz * R * f);
   const size_t n_tiles = (g.vocab + 127) / 128;
-  A_(c->stat_part, sizeof(float4) * static_cast<size_t>(dec_rows) * n_tiles);
-  A_(c->sample_part, sizeof(float4) * static_cast<size_t>(dec_rows) * n_tiles);
-  A_(c->conf, sizeof(float) * dec_rows);
-  A_(c->ent, sizeof(float) * dec_rows);
-  A_(c->argmax, sizeof(int) * dec_rows);
+  A_(c->stat_part, sizeof(float4) * static_cast<size_t>(head_rows) * n_tiles);
+  A_(c->sample_part, sizeof(float4) * static_cast<size_t>(head_rows) * n_tiles);
+  A_(c->conf, sizeof(float) * head_rows);
+  A_(c->ent, sizeof(float) * head_rows);
+  A_(c->argmax, sizeof(int) * head_rows);
   A_(c->prefix_len, sizeof(int) * g.max_batch);
   A_(c->pos_base, sizeof(int) * g.max_batch);
   A_(c->n_valid, sizeof(int) * g.max_batch);
@@ -2132,7 +2142,9 @@ extern "C" int d3_generate(d3_ctx* c, int32_t gen_len, float threshold, int32_t 
   LAUNCHED(c, "gen_init_kernel");
   const long long max_iter = static_cast<long long>(n_blocks) * (B + 1) + 1;
   // (a refresh falls between a block's finalize forward and the next block's first step: no fusing then)
-  const int fuse = (c->gen_fuse && c->refresh_every == 0 && 2ll * bs * B <= FUSE_MAX_ROWS && 2ll * c->cfg.max_batch * B <= FUSE_MAX_ROWS) ? 1 : 0;
+  const bool fuse_any = c->gen_fuse && c->refresh_every == 0 && 2ll * bs * B <= FUSE_MAX_ROWS && 2ll * c->cfg.max_batch * B <= FUSE_MAX_ROWS;
+  const bool fuse_many = c->gen_fuse && c->refresh_every == 0 && 2ll * bs * B <= c->fuse_rows && sk_forward_usable(c, 2 * bs * B);
+  const int fuse = fuse_any || fuse_many ? 1 : 0;
   long long steps = 0;
   c->last_refreshes = 0;
   c->draw_step = g.step;  // sampling noise: each sequence's step within its block (the counter is bumped after the forward)
@@ -2153,7 +2165,9 @@ extern "C" int d3_generate(d3_ctx* c, int32_t gen_len, float threshold, int32_t 
       c->last_refreshes += c->host_counters[7];
       TRY(refresh_forward(c, bs, g.refresh_flag, nullptr, g.counters + 7));
     }
-    R = c->host_counters[5] > 0 ? 2 * B : B;
+    const long long live = c->host_counters[4], at_border = c->host_counters[5];
+    const bool wide = at_border > 0 && (fuse_any || (2ll * bs * B <= FUSE_HALF_ROWS ? 2 * at_border >= live : at_border == live));
+    R = wide ? 2 * B : B;
   }
   c->last_early_stops = c->host_counters[6];
   if (host_stats) {

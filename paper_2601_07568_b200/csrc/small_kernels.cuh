@@ -450,7 +450,8 @@ __global__ void unmask_kernel(const float* __restrict__ conf, const float* __res
 // the first denoise step of the next block except that the latter reads the former's K/V, which the
 // same forward writes before its attention runs: with `fuse` the two run as one forward of 2B rows
 // (segment 0 = the finished block, segment 1 = the new, fully masked block; segment 0 never sees
-// segment 1).  The last block of a request, and every block when fuse is off, is finalized alone.
+// segment 1).  The last block of a request, and every block when fuse is off, is finalized alone; so is a block whose
+// next forward has B rows per sequence because too few sequences of the batch are at a border.
 enum : int { SEQ_DENOISE = 0, SEQ_FINALIZE = 1, SEQ_DONE = 2, SEQ_FUSED = 3 };
 struct GenState {
   int* mode;        // [bs] SEQ_*
@@ -477,7 +478,7 @@ constexpr int COMMIT_HIST_BINS = 129;  // a block has at most 128 positions
 __global__ void gen_rowmap_kernel(GenState g, int bs, int B, int R, int mask_id, int* pos_base, int* n_valid, int* kv_len) {
   const int b = blockIdx.x;
   const int mode = g.mode[b];
-  const int rows = mode == SEQ_DONE ? 0 : (mode == SEQ_FUSED ? 2 * B : B);
+  const int rows = mode == SEQ_DONE ? 0 : (mode == SEQ_FUSED ? R : B);
   if (threadIdx.x == 0) {
     pos_base[b] = g.prefix_len[b];
     n_valid[b] = rows;
@@ -544,7 +545,9 @@ __global__ void gen_advance_kernel(GenState g, const float* __restrict__ conf, c
       g.prefix_len[b] += B;
       atomicAdd(reinterpret_cast<unsigned long long*>(&g.counters[1]), 1ull);
       atomicAdd(reinterpret_cast<unsigned long long*>(&g.counters[5]), static_cast<unsigned long long>(-1ll));
+      if (R == B) g.mode[b] = SEQ_DENOISE;
     }
+    if (R == B) return;  // a finalize forward of its own: the next block's first step comes with the next forward
     stat_row0 += B;
   }
   const int step = g.step[b] + 1;

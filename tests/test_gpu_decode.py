@@ -625,6 +625,44 @@ def test_ragged_prompts_without_padding(hq, hkv, lens):
         assert ctx.error_word() == 0
 
 
+@pytest.mark.parametrize("lens,tau", [([40, 7, 97], 0.0), ([40, 7, 97, 64], 0.0), ([40, 7, 97, 64], 0.3), ([33] * 6, 0.3), ([33, 5] * 4, 0.0)])
+def test_fused_finalize_of_batches(lens, tau):
+    """Batches finalize a block together with the next block's first step where half of the sequences are at a border (up to
+    256 fused rows) or all of them (up to 512).  At threshold 0 every step decodes a block: all sequences cross the borders
+    together and the forwards are counted; at 0.3 they drift, and borders are crossed either way.  The stored keys and
+    values of layer 0 (a function of the stored tokens alone) are those of a prefill of the same tokens."""
+    shape = si.scaled_shape(si.LLADA8B, name="small-fused", n_layers=2, d_model=256, n_q_heads=4, n_kv_heads=2,
+                            d_ffn=640, vocab=1024, d_head=128)
+    W = si.gen_weights(shape)
+    bs, gen, n_blocks = len(lens), 128, 4
+    wl, ids, lens = si.small_workload("small-fused", shape, bs, lens, gen, 32, 0.9, 80)
+    with Ctx(shape, W, block=32, max_batch=bs, max_seq=wl.max_seq) as ctx:
+        def stored(b, n):
+            kv = torch.zeros((2, shape.n_kv_heads, n, 128), dtype=torch.float32, device=DEV)
+            d3.d3_read_kv(ctx.ctx, 0, b, 0, n, kv[0], kv[1])
+            return kv.cpu().numpy()
+        ctx.prefill(ids, lens)
+        tok, cs, st = ctx.generate(bs, gen, tau)
+        assert st.tokens_committed == bs * gen and st.finalize_forwards == bs * n_blocks
+        if tau == 0.0:
+            assert st.steps == n_blocks + 1 and st.denoise_forwards == bs * n_blocks
+        else:
+            assert st.steps < st.denoise_forwards + st.finalize_forwards
+        got = [stored(b, lens[b] + gen) for b in range(bs)]
+        full = np.full((bs, max(lens) + gen), shape.pad_id, dtype=np.int32)
+        for b in range(bs):
+            full[b, :lens[b] + gen] = np.concatenate([ids[b, :lens[b]], tok[b]])
+        ctx.prefill(full, np.array([n + gen for n in lens], dtype=np.int32))
+        for b in range(bs):
+            want = stored(b, lens[b] + gen)
+            assert np.max(np.abs(got[b] - want)) <= 2 ** -7 * np.max(np.abs(want))  # one bf16 rounding either side
+        d3.d3_set_fused_finalize(ctx.ctx, False)
+        ctx.prefill(ids, lens)
+        _, _, alone = ctx.generate(bs, gen, tau)
+        assert tau != 0.0 or alone.steps == 2 * n_blocks
+        assert ctx.error_word() == 0
+
+
 def test_small_bf16_batch_on_cta_pairs_step_locked():
     """Six sequences x 32 rows = 192 rows per decode forward, 768 padded rows in the prefill, and a vocabulary and
     widths that are multiples of 256: QKV (RoPE + cache write), gate/up (SwiGLU) and the LM head (fused statistics)

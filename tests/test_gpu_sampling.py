@@ -135,6 +135,21 @@ def test_sampling_epilogue_fp32_simt_against_its_own_logits():
         assert compared >= 3 * 16 * 5 and differing <= 2
 
 
+@pytest.mark.parametrize("d_model,bs", [(256, 3), (2048, 1), (2048, 5)])
+def test_sampling_epilogue_bf16_k_cut_pairs_against_its_own_logits(d_model, bs):
+    """The LM head as a matmul of the persistent decode launch, its vocabulary tiles whole (four slabs of K) and cut along
+    K (32 slabs): the statistics and the drawn tokens against the oracle's rule on the device's own logits."""
+    shape = si.scaled_shape(si.LLADA8B, name="sample-k-cut", n_layers=1, d_model=d_model, n_q_heads=4, n_kv_heads=2,
+                            d_ffn=640, vocab=1024, d_head=128)
+    W = si.gen_weights(shape)
+    wl, ids, lens = si.small_workload("sample-k-cut", shape, bs, [40, 7, 97, 64, 5][:bs], 64, 32, 0.9, 77)
+    with Ctx(shape, W, block=32, max_batch=bs, max_seq=wl.max_seq) as ctx:
+        d3.d3_set_tuning(ctx.ctx, chain=0, k_cut_pairs=1)
+        for T, seed in [(0.1, 3), (1.0, (7 << 32) + 9)]:
+            compared, differing = _check_step_against_own_logits(ctx, shape, ids, lens, 32, T, seed, 4, 1e-4)
+            assert compared >= bs * 32 * 3 and differing <= bs and ctx.error_word() == 0
+
+
 def test_sampling_epilogue_bf16_tensor_core_against_its_own_logits():
     """The tensor-core LM head (vocabulary of 1000: eight 128-column tiles with a ragged last one; 96
     rows = three sequences of 32) draws the oracle's tokens from its own logits."""
