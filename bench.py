@@ -533,7 +533,7 @@ def run_ours(args):
     # K/V read by the attention of one forward at mid-generation
     kv_mid = 2 * shape.n_layers * shape.n_kv_heads * shape.d_head * 2 * sum(int(l) + w.gen_len // 2 for l in lens_np)
     chain = prof.get("chain", {"ms": 0.0, "launches": 0})
-    if chain["launches"] > 0:
+    if chain["ms"] > sum(prof[k]["ms"] for k in gb):
         # the decode forward's layers run as one launch (chain_kernel): matmuls of all layers and attention
         dominant = "chain_kernel (all layers of a decode forward: QKV, attention, O-proj, gate/up, down)"
         per_launch_bytes = sum(gb[k] for k in layer_keys) * shape.n_layers + kv_mid
@@ -542,7 +542,7 @@ def run_ours(args):
         tot_ms, n_dom = chain["ms"], chain["launches"]
         traffic_kernel = "chain_kernel"
     else:
-        dominant = "gemm_strip_kernel, gemm_ck_kernel, gemm_xt_kernel, gemm_tc_kernel, gemm_pair_kernel (all matmul launches of the decode loop)"
+        dominant = "gemm_sk_kernel, gemm_pair_kernel, gemm_strip_kernel, gemm_ck_kernel, gemm_xt_kernel, gemm_tc_kernel (all matmul launches of the decode loop)"
         tot_bytes = sum(gb[k] * prof[k]["launches"] for k in gb)
         tot_flops = sum(gf[k] * prof[k]["launches"] for k in gf)
         tot_ms = sum(prof[k]["ms"] for k in gb)

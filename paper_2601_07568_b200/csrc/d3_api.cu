@@ -1557,7 +1557,12 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   bool head_done = false;
   const SkMatmul head_mm{c->xb, c->lm_head, g.vocab, d, EPI_STATS, head == 1 ? head_epi() : EpiParams{}, nullptr};
 
-  if (chain_usable(c, bs, rows_per_seq, seg)) {
+  // A block of up to 32 rows: with large layers the launches of resident pairs, all SMs instead of the 132 that clusters of
+  // four leave, make up for attention between them.  Measured, ms per forward, chain against this: 3.46 -> 3.37 at the 8B
+  // shape (436 MB a layer), 2.51 -> 2.40 at d_model 3072 (245 MB), but 1.84 -> 1.88 at 2048 (109 MB) and 1.38 -> 1.54 at 1024.
+  const bool large_layers = static_cast<double>(nq + 2 * nkv + nq + 3.0 * f) * d * c->esz >= 200e6;
+  const bool pairs_first = M <= 32 && large_layers && c->tune_chain < 0 && c->tune_chain_clusters == 0 && sk_forward_usable(c, M);
+  if (!pairs_first && chain_usable(c, bs, rows_per_seq, seg)) {
     // Skinny decode forward: all layers in one persistent launch (chain.cuh); a tapped layer cuts it.
     if (!c->chain_prog_ready) TRY(chain_build_program(c));
     CUDA_TRY(c, cudaMemsetAsync(c->chain_sync, 0, sizeof(unsigned int) * static_cast<size_t>(c->chain_prog_ops), c->stream));
