@@ -51,8 +51,6 @@ typedef struct d3_tuning {
                                of a pair fit one 128-row tile, whatever the number of pairs */
   int32_t cta_pairs;        /* matmuls of more than 128 rows on tiled weights run 256 x 256 tiles on pairs of CTAs that share
                                one MMA (cta_group::2, gemm_pair_kernel): -1 = when the shape allows (default), 0 never */
-  int32_t k_cut_pairs;      /* matmuls of decode-sized forwards on resident CTA pairs with the tiles of an incomplete wave cut
-                               along K (gemm_sk_kernel): -1 = by row count (default), 0 never, 1 wherever the shape allows */
 } d3_tuning;
 void d3_tuning_defaults(d3_tuning *t);
 int d3_set_tuning(d3_ctx *ctx, const d3_tuning *t);
@@ -61,6 +59,11 @@ int d3_set_tuning(d3_ctx *ctx, const d3_tuning *t);
  * block while the forward stays skinny (see d3_generate).  on = 0: every block is finalized in a
  * forward of its own; results are the same (bit for bit on the fp32 path). */
 int d3_set_fused_finalize(d3_ctx *ctx, int on);
+
+/* Matmuls of decode-sized forwards on resident CTA pairs, the tiles of an incomplete wave cut along K (gemm_sk_kernel, up
+ * to 1024 rows): mode -1 = by row count (default), 0 never, 1 wherever the shape allows, every cut that gives each pair
+ * work included, and for d3_op_linear_packed.  INVALID_ARG for other values. */
+int d3_set_k_cut_pairs(d3_ctx *ctx, int32_t mode);
 
 /* Give-up path of the bounded waits.  Every device-side wait of the kernels (mbarrier phases) ends
  * after a time limit, raises bit 0 of the device error word and lets its CTA leave in order (all

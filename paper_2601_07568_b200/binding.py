@@ -32,7 +32,7 @@ EXPORTS = [
     "d3_strerror", "d3_last_error", "d3_version",
 ]
 # measurement and test switches (include/d3_debug.h)
-DEBUG_EXPORTS = ["d3_tuning_defaults", "d3_set_tuning", "d3_set_fused_finalize", "d3_debug_stall_probe",
+DEBUG_EXPORTS = ["d3_tuning_defaults", "d3_set_tuning", "d3_set_fused_finalize", "d3_set_k_cut_pairs", "d3_debug_stall_probe",
                  "d3_clear_error_word", "d3_status_of_error_word"]
 
 
@@ -358,7 +358,7 @@ def d3_set_overlap(ctx, on: bool) -> None:
 class d3_tuning(C.Structure):
     _fields_ = [(n, C.c_int32) for n in ("ring_kb", "ctas_per_sm", "producers", "tile_columns", "attn_key_tiles",
                                           "cluster_k_split", "row_tile_pairs", "round_robin", "column_strips",
-                                          "strip_stages", "chain", "chain_clusters", "chain_l2_ahead", "weights_as_rows", "attention_tmem", "cta_pairs", "k_cut_pairs")]
+                                          "strip_stages", "chain", "chain_clusters", "chain_l2_ahead", "weights_as_rows", "attention_tmem", "cta_pairs")]
 
 
 def d3_tuning_defaults() -> d3_tuning:
@@ -379,6 +379,10 @@ def d3_set_tuning(ctx, tuning: Optional[d3_tuning] = None, **fields) -> None:
 
 def d3_set_fused_finalize(ctx, on: bool) -> None:
     _check(ctx, lib().d3_set_fused_finalize(ctx, C.c_int(1 if on else 0)))
+
+
+def d3_set_k_cut_pairs(ctx, mode: int) -> None:
+    _check(ctx, lib().d3_set_k_cut_pairs(ctx, C.c_int32(mode)))
 
 
 def d3_debug_stall_probe(ctx, limit_us: int) -> int:

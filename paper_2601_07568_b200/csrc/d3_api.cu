@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <tuple>
 #include <utility>
@@ -43,6 +44,8 @@ struct d3_ctx {
   bool w_tiled = false;  // model matrices stored as contiguous 128 x 64 blocks (tensor-core path)
   size_t esz = 4;
   int n_sms = 148;
+  int device = 0;
+  cudaEvent_t order_event = nullptr;  // see ordered_launch
   // weights (context dtype), repacked
   void* tok_emb = nullptr;
   void* lm_head = nullptr;
@@ -296,6 +299,44 @@ constexpr long long FUSE_MAX_ROWS = 64;
 // a border outweighs them, f c(R) > c(2R) - c(R) with c the forward's time (8B shape, ms: c(96) 4.0, c(128) 4.1, c(192)
 // 5.0, c(256) 5.4, c(512) 10.0): half of the live sequences up to 256 fused rows, all of them up to 512.
 constexpr long long FUSE_HALF_ROWS = 256, FUSE_ALL_ROWS = 512;
+
+// ---- launches whose CTAs wait for one another
+// The chain and the launches of resident CTA pairs need all their CTAs on the device at once.  Two of them on different
+// streams (contexts of two threads, say) could each get a part of the SMs and wait for the rest until their waits run
+// out, so such launches of a process are put in one order per device: a launch on another stream than the one before
+// waits for that stream's work so far.  One context, or several on one stream, never wait for anything here.
+// (A cooperative launch gives the same guarantee, but no longer overlaps its start with the kernel before: 4.6 us a launch.)
+struct LaunchOrder {
+  std::mutex lock;
+  std::map<int, std::pair<cudaStream_t, const d3_ctx*>> last;  // per device: stream and context of the latest such launch
+};
+LaunchOrder& launch_order() {
+  static LaunchOrder order;
+  return order;
+}
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+template <typename Launch>
+int ordered_launch(d3_ctx* c, Launch&& launch) {
+  LaunchOrder& order = launch_order();
+  std::lock_guard<std::mutex> hold(order.lock);
+  auto it = order.last.find(c->device);
+  // (what is captured runs when the graph does: its order is the graph launches')
+  if (it != order.last.end() && it->second.first != c->stream && !capturing(c->stream) && !capturing(it->second.first)) {
+    if (!c->order_event) CUDA_TRY(c, cudaEventCreateWithFlags(&c->order_event, cudaEventDisableTiming));
+    CUDA_TRY(c, cudaEventRecord(c->order_event, it->second.first));
+    CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->order_event, 0));
+  }
+  CUDA_TRY(c, launch());
+  order.last[c->device] = {c->stream, c};
+  return D3_OK;
+}
 
 // ---- matmul dispatch
 struct QkvExtra {
@@ -887,7 +928,7 @@ int run_chain(d3_ctx* c, int op_begin, int op_end, const RowMap& rm) {
   }
   cfg.attrs = at;
   cfg.numAttrs = na;
-  CUDA_TRY(c, cudaLaunchKernelEx(&cfg, tc::chain_kernel, *t_o, *t_xb, *t_h, c->kv_tmap32, p));
+  TRY(ordered_launch(c, [&] { return cudaLaunchKernelEx(&cfg, tc::chain_kernel, *t_o, *t_xb, *t_h, c->kv_tmap32, p); }));
   LAUNCHED(c, "chain_kernel");
   return D3_OK;
 }
@@ -1078,7 +1119,7 @@ int run_sk(d3_ctx* c, const SkMatmul* mm, int n, int M) {
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = 2;
   }
-  CUDA_TRY(c, cudaLaunchKernelEx(&cfg, tc::gemm_sk_kernel, p));
+  TRY(ordered_launch(c, [&] { return cudaLaunchKernelEx(&cfg, tc::gemm_sk_kernel, p); }));
   LAUNCHED(c, "gemm_sk_kernel");
   return D3_OK;
 }
@@ -1752,6 +1793,7 @@ extern "C" int d3_create(const d3_config* cfg, void* cuda_stream, d3_ctx** out) 
   };
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return bail(D3_ERR_CUDA);
+  c->device = dev;
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return bail(D3_ERR_CUDA);
   c->n_sms = prop.multiProcessorCount;
@@ -1887,6 +1929,13 @@ extern "C" int d3_create(const d3_config* cfg, void* cuda_stream, d3_ctx** out) 
 extern "C" void d3_destroy(d3_ctx* c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
+  {
+    LaunchOrder& order = launch_order();
+    std::lock_guard<std::mutex> hold(order.lock);
+    auto it = order.last.find(c->device);
+    if (it != order.last.end() && it->second.second == c) order.last.erase(it);  // its work is done, and its stream may go
+  }
+  if (c->order_event) cudaEventDestroy(c->order_event);
   for (auto& pp : c->prof_pool) {
     cudaEventDestroy(pp.a);
     cudaEventDestroy(pp.b);
@@ -2506,7 +2555,6 @@ extern "C" void d3_tuning_defaults(d3_tuning* t) {
   t->weights_as_rows = -1;
   t->attention_tmem = -1;
   t->cta_pairs = -1;
-  t->k_cut_pairs = -1;
 }
 extern "C" int d3_set_tuning(d3_ctx* c, const d3_tuning* t) {
   if (!c || !t) return D3_ERR_INVALID_ARG;
@@ -2516,7 +2564,7 @@ extern "C" int d3_set_tuning(d3_ctx* c, const d3_tuning* t) {
       (t->round_robin != 0 && t->round_robin != 1) || t->column_strips < 0 || t->column_strips > 3 || t->strip_stages < 0 ||
       t->strip_stages > 32 || t->chain < -1 || t->chain > 0 || t->chain_clusters < 0 || t->chain_l2_ahead < -1 || t->chain_l2_ahead > 256 || t->weights_as_rows < -1 || t->weights_as_rows > 0 ||
       ((t->attention_tmem < -1 || t->attention_tmem > 2) && t->attention_tmem != 64 && t->attention_tmem != 128) ||
-      t->cta_pairs < -1 || t->cta_pairs > 0 || t->k_cut_pairs < -1 || t->k_cut_pairs > 1)
+      t->cta_pairs < -1 || t->cta_pairs > 0)
     return fail(c, D3_ERR_INVALID_ARG, "d3_set_tuning: a field is outside its range");
   c->tune_ring_kb = t->ring_kb;
   c->tune_ctas_per_sm = t->ctas_per_sm;
@@ -2535,7 +2583,12 @@ extern "C" int d3_set_tuning(d3_ctx* c, const d3_tuning* t) {
   c->tune_attn_tmem = t->attention_tmem > 1 ? 1 : t->attention_tmem;
   c->tune_attn_shape = t->attention_tmem > 1 ? t->attention_tmem : 0;
   c->tune_cta_pairs = t->cta_pairs;
-  c->tune_sk = t->k_cut_pairs;
+  return D3_OK;
+}
+extern "C" int d3_set_k_cut_pairs(d3_ctx* c, int32_t mode) {
+  if (!c) return D3_ERR_INVALID_ARG;
+  if (mode < -1 || mode > 1) return fail(c, D3_ERR_INVALID_ARG, "k_cut_pairs mode is -1, 0 or 1");
+  c->tune_sk = mode;
   return D3_OK;
 }
 extern "C" int d3_set_fused_finalize(d3_ctx* c, int on) {

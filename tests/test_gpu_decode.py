@@ -570,9 +570,10 @@ def test_small_bf16_batch_on_k_cut_pairs_step_locked(lens, gen):
             d3.d3_read_tap(ctx.ctx, t[0], t[1], bs * 32)
             d3.d3_set_tap(ctx.ctx, -1)
             return [lg] + [x.cpu().numpy() for x in t]
-        d3.d3_set_tuning(ctx.ctx, chain=0, k_cut_pairs=0)
+        d3.d3_set_tuning(ctx.ctx, chain=0)
+        d3.d3_set_k_cut_pairs(ctx.ctx, 0)
         base = tapped()
-        d3.d3_set_tuning(ctx.ctx, chain=0, k_cut_pairs=1)
+        d3.d3_set_k_cut_pairs(ctx.ctx, 1)
         n0 = d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel")
         got = tapped()
         assert d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel") == n0 + 2 * (shape.n_layers + 1) + 1  # prefill, block forward, logits
@@ -623,6 +624,46 @@ def test_ragged_prompts_without_padding(hq, hkv, lens):
             for a, b, c in zip(got, again, want):
                 assert torch.equal(a, c) and torch.equal(b, c)  # (a refresh of the prompt alone is the prefill again)
         assert ctx.error_word() == 0
+
+
+def test_two_contexts_on_two_streams():
+    """Two contexts, each on its own stream and thread, decode at the same time: the launches whose CTAs wait for one
+    another (resident pairs at 96 rows, the chain at 32) are ordered between the streams, and both give the tokens
+    and steps that they give alone."""
+    import threading
+    shape = si.scaled_shape(si.LLADA8B, name="small-streams", n_layers=3, d_model=256, n_q_heads=4, n_kv_heads=2,
+                            d_ffn=640, vocab=1024, d_head=128)
+    W = si.gen_weights(shape)
+    jobs = []
+    for lens in ([40, 7, 97], [33]):
+        wl, ids, lens = si.small_workload("small-streams", shape, len(lens), lens, 64, 32, 0.5, 81)
+        with torch.cuda.stream(torch.cuda.Stream()):
+            jobs.append((torch.cuda.current_stream(), Ctx(shape, W, block=32, max_batch=len(lens), max_seq=wl.max_seq), ids, lens))
+    torch.cuda.synchronize()
+    got = [[], []]
+
+    def decode(i, times):
+        st, ctx, ids, lens = jobs[i]
+        torch.cuda.set_device(0)
+        with torch.cuda.stream(st):
+            for _ in range(times):
+                ctx.prefill(ids, lens)
+                tok, cs, _ = ctx.generate(len(lens), 64, 0.5)
+                got[i].append((tok.copy(), cs.copy()))
+    try:
+        for i in range(2):
+            decode(i, 1)
+        threads = [threading.Thread(target=decode, args=(i, 6)) for i in range(2)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        for i, (_, ctx, _, _) in enumerate(jobs):
+            assert len(got[i]) == 7 and ctx.error_word() == 0
+            assert all(np.array_equal(a, got[i][0][0]) and np.array_equal(b, got[i][0][1]) for a, b in got[i])
+    finally:
+        for _, ctx, _, _ in jobs:
+            ctx.close()
 
 
 @pytest.mark.parametrize("lens,tau", [([40, 7, 97], 0.0), ([40, 7, 97, 64], 0.0), ([40, 7, 97, 64], 0.3), ([33] * 6, 0.3), ([33, 5] * 4, 0.0)])

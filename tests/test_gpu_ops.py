@@ -179,7 +179,7 @@ def test_linear_bf16_k_cut_pairs(ctx_bf16, m, n, k):
     xd, wd = xt.to(DEV), wt.to(DEV)
     packed = torch.full((d3.d3_packed_weight_elems(n, k),), 3.0, dtype=torch.bfloat16, device=DEV)
     d3.d3_pack_weight(ctx_bf16.ctx, wd, packed)
-    d3.d3_set_tuning(ctx_bf16.ctx, k_cut_pairs=1)
+    d3.d3_set_k_cut_pairs(ctx_bf16.ctx, 1)
     try:
         n0 = d3.d3_launch_count_of(ctx_bf16.ctx, "gemm_sk_kernel")
         y = torch.full((m, n), 7.0, dtype=torch.float32, device=DEV)
@@ -201,7 +201,7 @@ def test_linear_bf16_k_cut_pairs(ctx_bf16, m, n, k):
         assert np.max(np.abs(h.float().cpu().numpy() - want)) <= 2 ** -7 * np.abs(want).max() + tol
         assert d3.d3_launch_count_of(ctx_bf16.ctx, "gemm_sk_kernel") == n0 + 5
     finally:
-        d3.d3_set_tuning(ctx_bf16.ctx)
+        d3.d3_set_k_cut_pairs(ctx_bf16.ctx, -1)
     assert ctx_bf16.error_word() == 0
 
 

@@ -144,7 +144,8 @@ def test_sampling_epilogue_bf16_k_cut_pairs_against_its_own_logits(d_model, bs):
     W = si.gen_weights(shape)
     wl, ids, lens = si.small_workload("sample-k-cut", shape, bs, [40, 7, 97, 64, 5][:bs], 64, 32, 0.9, 77)
     with Ctx(shape, W, block=32, max_batch=bs, max_seq=wl.max_seq) as ctx:
-        d3.d3_set_tuning(ctx.ctx, chain=0, k_cut_pairs=1)
+        d3.d3_set_tuning(ctx.ctx, chain=0)
+        d3.d3_set_k_cut_pairs(ctx.ctx, 1)
         for T, seed in [(0.1, 3), (1.0, (7 << 32) + 9)]:
             compared, differing = _check_step_against_own_logits(ctx, shape, ids, lens, 32, T, seed, 4, 1e-4)
             assert compared >= bs * 32 * 3 and differing <= bs and ctx.error_word() == 0
