@@ -1507,15 +1507,6 @@ bool sk_forward_usable(const d3_ctx* c, int M) {
   return M <= SK_FORWARD_ROWS;
 }
 
-// The LM head of a decode forward on gemm_sk_kernel.
-bool sk_head_usable(const d3_ctx* c, int M) {
-  if (c->tune_sk == 0 || !c->use_tc || !c->fold_norm || !c->w_tiled || M > tc::SK_MAX_ROWS || !sk_shape_ok(c->cfg.vocab, c->cfg.d_model)) return false;
-  if (c->tune_sk == 1) return true;
-  if (c->tune_strip != 0 || c->tune_no_cluster || c->tune_xt == 0 || c->tune_cta_pairs == 0 || c->tune_wide_tiles >= 0 || c->tune_pair >= 0 ||
-      c->tune_producers > 0 || c->tune_ring_kb > 0 || c->tune_ctas_per_sm > 0) return false;
-  return M <= SK_FORWARD_ROWS;
-}
-
 // Can the rows of a ragged forward be laid out without padding?  Where all its matmuls run on CTA pairs, which take the
 // number of rows from the device (32 prompts of 128..512 tokens, 16384 padded rows of which 10240 are in use: 200.5 -> 137.6 ms).
 // (A tapped forward keeps the layout that d3_read_tap describes.)
@@ -1577,7 +1568,6 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
     ep.yb = static_cast<bf16*>(c->xb); ep.ssq_out = c->ssq;
   };
 
-  // The LM head with its statistics: an operand of the same persistent launches where those run.
   auto head_epi = [&]() {
     EpiParams ep;
     ep.scale = g.logit_scale; ep.mask_id = g.mask_id; ep.stat_part = c->stat_part; ep.n_tiles = (g.vocab + 127) / 128;
@@ -1594,20 +1584,20 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
     after_norm(ep);
     return ep;
   };
-  const bool head_sk = head == 1 && sk_head_usable(c, M);
-  bool head_done = false;
-  const SkMatmul head_mm{c->xb, c->lm_head, g.vocab, d, EPI_STATS, head == 1 ? head_epi() : EpiParams{}, nullptr};
-
   // A block of up to 32 rows: with large layers the launches of resident pairs, all SMs instead of the 132 that clusters of
   // four leave, make up for attention between them.  Measured, ms per forward, chain against this: 3.46 -> 3.37 at the 8B
   // shape (436 MB a layer), 2.51 -> 2.40 at d_model 3072 (245 MB), but 1.84 -> 1.88 at 2048 (109 MB) and 1.38 -> 1.54 at 1024.
   const bool large_layers = static_cast<double>(nq + 2 * nkv + nq + 3.0 * f) * d * c->esz >= 200e6;
   const bool pairs_first = M <= 32 && large_layers && c->tune_chain < 0 && c->tune_chain_clusters == 0 && sk_forward_usable(c, M);
-  if (!pairs_first && chain_usable(c, bs, rows_per_seq, seg)) {
+  const bool chain = !pairs_first && chain_usable(c, bs, rows_per_seq, seg);
+  // The LM head is the last matmul of the last layer's launch.  (Behind the chain it stays a launch of its own on 128-row tiles,
+  // whose weights are on their way while the chain drains: 3.79 ms a 64-row forward against 3.83.)
+  const bool head_sk = head == 1 && !chain && sk_forward_usable(c, M) && sk_shape_ok(g.vocab, d);
+
+  if (chain) {
     // Skinny decode forward: all layers in one persistent launch (chain.cuh); a tapped layer cuts it.
     if (!c->chain_prog_ready) TRY(chain_build_program(c));
     CUDA_TRY(c, cudaMemsetAsync(c->chain_sync, 0, sizeof(unsigned int) * static_cast<size_t>(c->chain_prog_ops), c->stream));
-    if (head_sk) TRY(sk_begin(c, 1));
     const int n_ops = c->chain_prog_ops;
     const bool tap = c->tap_layer >= 0 && c->tap_layer < g.n_layers && M <= c->tap_rows;
     if (!tap) {
@@ -1620,11 +1610,6 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
       TRY(run_chain(c, o_in, o_out, rm));
       CUDA_TRY(c, cudaMemcpyAsync(c->tap_out, c->x, sizeof(float) * M * d, cudaMemcpyDeviceToDevice, c->stream));
       if (o_out < n_ops) TRY(run_chain(c, o_out, n_ops, rm));
-    }
-    if (head_sk) {
-      ProfScope ps(c, D3_PROF_GEMM_HEAD);
-      TRY(run_sk(c, &head_mm, 1, M));
-      head_done = true;
     }
   } else if (sk_forward_usable(c, M)) {
     // Decode-sized forward: the matmuls between two attention kernels (O-proj, gate/up, down, the next layer's QKV) in
@@ -1671,9 +1656,8 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
       const bool more = l + 1 < g.n_layers;
       if (more) mm[3] = qkv(l + 1, qx);
       if (!more && head_sk) {
-        mm[3] = head_mm;
+        mm[3] = SkMatmul{c->xb, c->lm_head, g.vocab, d, EPI_STATS, head_epi(), nullptr};
         classes[3] = D3_PROF_GEMM_HEAD;
-        head_done = true;
       }
       TRY(launch(mm, classes, more || head_sk ? 4 : 3));
       if (l == c->tap_layer && tap)
@@ -1728,11 +1712,6 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   if (head == 0) return D3_OK;
   if (!c->fold_norm) TRY(run_rmsnorm(c, c->x, c->final_norm, c->xn, M));
   if (head == 1) {
-    if (head_sk && !head_done) {
-      TRY(sk_begin(c, 1));
-      ProfScope ps(c, D3_PROF_GEMM_HEAD);
-      TRY(run_sk(c, &head_mm, 1, M));
-    }
     if (!head_sk) TRY(run_linear(c, normed, c->lm_head, M, g.vocab, d, EPI_STATS, head_epi(), 0, nullptr, D3_PROF_GEMM_HEAD, c->w_tiled));
     TRY(run_stats_merge(c, M, (g.vocab + 127) / 128, c->conf, c->ent, c->argmax, c->temperature > 0.f));
   } else {
