@@ -57,10 +57,12 @@ __global__ void embed_kernel(const int* __restrict__ ids, const T* __restrict__ 
 // ----------------------------------------------------------------------------- folded RMSNorm helpers
 // The embeddings of a forward on the tensor-core path: the rows themselves and what a residual epilogue leaves behind for
 // the next matmul (see EpiParams), bf16 copy and sum of squares of every 32-column chunk, from one read of the table.
-// One block per row, 8 columns a thread (d_model is a multiple of 8), four neighbouring lanes a chunk.  Bound by its
-// stores.  `row_off` non-null: sequences of rows_per_seq ids of which the first n_valid[b] go to rows row_off[b]...; the ids
-// of the others are looked at all the same.  As two kernels, the second with 32 columns a thread: 22 us in front of a 32-row forward and 0.85 ms in front of
-// a 16384 x 4096 prefill; this one 5 us and 0.10 ms.
+// One block per row, 8 columns a thread (d_model is a multiple of 8), four neighbouring lanes a chunk, whose squares are added
+// in column order as gemm_tc's and gemm_pair's residual epilogues do (the same bits: a layer that leaves a row as it was
+// leaves its row factor as it was).  Bound by its stores.  `row_off` non-null: sequences of rows_per_seq ids of which the
+// first n_valid[b] go to rows row_off[b]...; the ids of the others are looked at all the same.  As two kernels, the second
+// with 32 columns a thread: 22 us in front of a 32-row forward and 0.85 ms in front of a 16384 x 4096 prefill; this one
+// 5 us and 0.10 ms.
 __global__ void __launch_bounds__(256) embed_prep_kernel(const int* __restrict__ ids, const __nv_bfloat16* __restrict__ emb, float* __restrict__ x,
                                                          __nv_bfloat16* __restrict__ xb, float* __restrict__ ssq, int d, int vocab, uint32_t* error_word, const int* __restrict__ row_off,
                                                          const int* __restrict__ n_valid, int rows_per_seq) {
@@ -83,24 +85,27 @@ __global__ void __launch_bounds__(256) embed_prep_kernel(const int* __restrict__
   uint4* copy = reinterpret_cast<uint4*>(xb + static_cast<size_t>(m) * d);
   for (int i0 = 0; i0 < n_chunks * 4; i0 += blockDim.x) {  // (all lanes: the sums are exchanged)
     const int i = i0 + threadIdx.x;
-    float sq = 0.f;
+    float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (i < d / 8) {
       const uint4 v = src[i];
       const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-      float f[8];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         f[2 * q] = __uint_as_float(w[q] << 16);
         f[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
       }
-#pragma unroll
-      for (int q = 0; q < 8; ++q) sq += f[q] * f[q];
       row[2 * i] = make_float4(f[0], f[1], f[2], f[3]);
       row[2 * i + 1] = make_float4(f[4], f[5], f[6], f[7]);
       copy[i] = v;
     }
-    sq += __shfl_xor_sync(0xffffffffu, sq, 1);
-    sq += __shfl_xor_sync(0xffffffffu, sq, 2);
+    float sq = 0.f;  // of the chunk's columns so far
+#pragma unroll
+    for (int turn = 0; turn < 4; ++turn) {
+      float mine = sq;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) mine += f[q] * f[q];
+      sq = __shfl_sync(0xffffffffu, mine, turn, 4);
+    }
     if ((threadIdx.x & 3) == 0 && i / 4 < n_chunks) ssq[static_cast<size_t>(m) * n_chunks + i / 4] = sq;
   }
 }

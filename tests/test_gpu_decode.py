@@ -626,6 +626,27 @@ def test_ragged_prompts_without_padding(hq, hkv, lens):
         assert ctx.error_word() == 0
 
 
+def test_chunk_sums_of_the_embeddings_are_the_residual_epilogue_s():
+    """A layer whose output projections are zero leaves the residual stream as it was, and with it the row factors of the
+    next layer: two layers with the same q, k, v matrices store the same keys and values, bit for bit."""
+    shape = si.scaled_shape(si.LLADA8B, name="small-sums", n_layers=2, d_model=520, n_q_heads=8, n_kv_heads=8,
+                            d_ffn=640, vocab=4096, d_head=128)
+    for shape, rows in ((shape, 200), (dataclasses.replace(shape, d_model=512), 700)):
+        W = si.gen_weights(shape)
+        W["layers"][1] = W["layers"][0]
+        for name in ("wo", "w_down"):
+            W["layers"][0][name] = np.zeros_like(W["layers"][0][name])
+        ids = np.random.default_rng(3).integers(0, shape.vocab - 2, size=(1, rows)).astype(np.int32)
+        with Ctx(shape, W, block=32, max_batch=1, max_seq=rows + 32) as ctx:
+            d3.d3_set_tuning(ctx.ctx, chain=0, weights_as_rows=0, cluster_k_split=0)
+            ctx.prefill(ids, np.array([rows], dtype=np.int32))
+            kv = torch.zeros((2, 2, 8, rows, 128), dtype=torch.float32, device=DEV)
+            for layer in range(2):
+                d3.d3_read_kv(ctx.ctx, layer, 0, 0, rows, kv[layer, 0], kv[layer, 1])
+            assert kv[0].abs().max() > 0 and torch.equal(kv[0], kv[1])
+            assert ctx.error_word() == 0
+
+
 def test_two_contexts_on_two_streams():
     """Two contexts, each on its own stream and thread, decode at the same time: the launches whose CTAs wait for one
     another (resident pairs at 96 rows, the chain at 32) are ordered between the streams, and both give the tokens
