@@ -1407,7 +1407,8 @@ int run_attention_tc(d3_ctx* c, const void* q, int layer, void* out, const RowMa
   if (c->tune_attn_shape == 2 && rm.row_off == nullptr ? attn_stream_usable(c, rm)
                               : (rm.row_off == nullptr && c->tune_attn_tmem < 0 && attn_stream_usable(c, rm) && rm.bs * g.n_kv_heads >= 2 * c->n_sms))
     return run_attention_tmem_stream(c, q, layer, out, rm);
-  if (c->tune_attn_tmem == 1 || (c->tune_attn_tmem < 0 && R >= 64)) return run_attention_tmem(c, q, layer, out, rm);
+  // (the mma.sync kernel has one key limit for 16 rows: segments that are not multiples of 16 rows are never its business)
+  if (c->tune_attn_tmem == 1 || (c->tune_attn_tmem < 0 && R >= 64) || rm.seg % 16 != 0) return run_attention_tmem(c, q, layer, out, rm);
   const int nw = R <= 32 ? 2 : (R <= 64 ? 4 : 8);
   const int q_tiles = (R + nw * 16 - 1) / (nw * 16);
   const int pairs = rm.bs * g.n_kv_heads;

@@ -626,6 +626,57 @@ def test_ragged_prompts_without_padding(hq, hkv, lens):
         assert ctx.error_word() == 0
 
 
+@pytest.mark.parametrize("block,n_win,bs,hq,hkv", [(8, 2, 1, 2, 2), (8, 3, 3, 4, 2), (24, 2, 2, 2, 2), (40, 3, 1, 1, 1), (8, 2, 10, 2, 2), (12, 2, 6, 2, 2)])
+def test_windows_of_blocks_that_are_no_multiple_of_16_rows(block, n_win, bs, hq, hkv):
+    """Every row of a window sees its own block and the earlier ones, whatever the block size: keys and values of the second
+    layer (which depend on what the first layer's attention saw) against those of the plain bf16 kernels."""
+    shape = si.scaled_shape(si.LLADA8B, name="odd-block", n_layers=2, d_model=256, n_q_heads=hq, n_kv_heads=hkv,
+                            d_ffn=640, vocab=1024, d_head=128)
+    W = si.gen_weights(shape)
+    rng = np.random.default_rng(block + bs)
+    lens = np.array([20 + 3 * b for b in range(bs)], dtype=np.int32)
+    ids = rng.integers(0, shape.vocab - 2, size=(bs, int(lens.max()))).astype(np.int32)
+    n = n_win * block
+    win = torch.from_numpy(rng.integers(0, shape.vocab - 2, size=(bs, n)).astype(np.int32)).to(DEV)
+    kv = torch.zeros((2, bs, 2, hkv, n, 128), dtype=torch.float32, device=DEV)
+    for impl in (0, 1):
+        with Ctx(shape, W, block=block, max_batch=bs * n_win, max_seq=200, gemm_impl=impl) as ctx:
+            ctx.prefill(ids, lens)
+            st = [torch.zeros(bs * n, dtype=dt, device=DEV) for dt in (torch.float32, torch.float32, torch.int32)]
+            d3.d3_denoise_window(ctx.ctx, win, n_win, *st)
+            for b in range(bs):
+                d3.d3_read_kv(ctx.ctx, 1, b, int(lens[b]), n, kv[impl, b, 0], kv[impl, b, 1])
+            assert ctx.error_word() == 0
+    # bf16 rounding of either side at the storage points of one layer (0.6 % measured); a wrong key limit moves them by 40 %
+    assert (kv[0] - kv[1]).abs().max() <= 2e-2 * kv[1].abs().max()
+
+
+@pytest.mark.parametrize("block,bs", [(8, 10), (8, 1), (24, 3), (32, 3)])
+def test_first_steps_of_fused_forwards(block, bs):
+    """At threshold 0 every block is decoded by its first step, which rides along with the finalize forward of the block
+    before: the tokens are those of a step of its own over the same stored blocks (near-ties of the two orders of
+    summation aside: 5 % of the positions)."""
+    shape = si.scaled_shape(si.LLADA8B, name="odd-fused", n_layers=2, d_model=256, n_q_heads=2, n_kv_heads=2,
+                            d_ffn=640, vocab=1024, d_head=128)
+    W = si.gen_weights(shape)
+    lens = np.array([20 + 3 * b for b in range(bs)], dtype=np.int32)
+    ids = np.random.default_rng(block).integers(0, shape.vocab - 2, size=(bs, int(lens.max()))).astype(np.int32)
+    gen = 4 * block
+    with Ctx(shape, W, block=block, max_batch=bs, max_seq=int(lens.max()) + gen) as ctx:
+        ctx.prefill(ids, lens)
+        tok, _, st = ctx.generate(bs, gen, 0.0)
+        assert st.steps == 5  # four blocks: every border fused
+        ctx.prefill(ids, lens)
+        same = []
+        for j in range(4):
+            own = tok[:, j * block:(j + 1) * block]
+            step = ctx.step(np.full((bs, block), shape.mask_id, dtype=np.int32), np.ones((bs, block)), 0.0)
+            same.append(step["ids"] == own)
+            ctx.commit(own)
+        assert np.mean(same) >= 0.95, [float(np.mean(s)) for s in same]
+        assert ctx.error_word() == 0
+
+
 def test_chunk_sums_of_the_embeddings_are_the_residual_epilogue_s():
     """A layer whose output projections are zero leaves the residual stream as it was, and with it the row factors of the
     next layer: two layers with the same q, k, v matrices store the same keys and values, bit for bit."""
