@@ -881,7 +881,7 @@ __global__ void refresh_rowmap_kernel(const int* __restrict__ hist, int max_seq,
   const int b = blockIdx.x;
   const bool take = (flag == nullptr || flag[b] != 0) && (active == nullptr || active[b] > 0);
   int len = take ? prefix_len[b] : 0;
-  len = len > p_max ? p_max : len;
+  len = len < 0 ? 0 : (len > p_max ? p_max : len);  // (a negative prefix holds no rows, and no negative count enters the row layout)
   __syncthreads();
   if (threadIdx.x == 0) {
     pos_base[b] = 0;

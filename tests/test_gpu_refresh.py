@@ -7,7 +7,7 @@ import torch
 from oracle import d3_oracle as o
 from paper_2601_07568_b200 import binding as d3
 from paper_2601_07568_b200 import synth_inputs as si
-from gpu_utils import Ctx, assert_rounding_bounded, record_report
+from gpu_utils import DEV, Ctx, assert_rounding_bounded, record_report
 from test_gpu_decode import BF16_STAT_ERR_BOUND, step_locked
 
 pytestmark = pytest.mark.gpu
@@ -150,3 +150,31 @@ def test_refresh_bf16_tensor_core():
         assert d3.d3_refresh_count(ctx.ctx) == 3 and stt.tokens_committed == 128 and ctx.error_word() == 0
         assert not np.any(tok == shape.mask_id)
         print("free-running equal to the oracle:", np.array_equal(tok[0], traces[0]["tokens"]))
+
+
+def test_refresh_passes_over_a_negative_prefix():
+    """d3_set_state takes any value.  A sequence whose prefix is negative has no rows in a refresh: the others get the keys
+    and values that they get without it, and its own stay."""
+    shape = si.scaled_shape(si.LLADA8B, name="refresh-negative", n_layers=2, d_model=256, n_q_heads=4, n_kv_heads=2,
+                            d_ffn=640, vocab=1024, d_head=128)
+    W = si.gen_weights(shape)
+    lens = np.array([30, 700, 9], dtype=np.int32)
+    ids = np.random.default_rng(5).integers(0, shape.vocab - 2, size=(3, 700)).astype(np.int32)
+
+    def stored(ctx):
+        out = []
+        for b, n in enumerate(lens):
+            for layer in range(shape.n_layers):
+                kv = torch.zeros((2, shape.n_kv_heads, int(n), 128), dtype=torch.float32, device=DEV)
+                d3.d3_read_kv(ctx.ctx, layer, b, 0, int(n), kv[0], kv[1])
+                out.append(kv)
+        return out
+    with Ctx(shape, W, block=32, max_batch=3, max_seq=732) as ctx:
+        ctx.prefill(ids, lens)
+        want = stored(ctx)
+        for prefixes in ((0, 700, 9), (-1, 700, 9), (-700, 700, 9), (30, 700, -5)):
+            ctx.set_prefix(prefixes)
+            d3.d3_refresh_cache(ctx.ctx, 3)
+            for a, b in zip(stored(ctx), want):
+                assert torch.equal(a, b)
+        assert ctx.error_word() == 0
