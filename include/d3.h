@@ -146,7 +146,7 @@ int d3_commit_block(d3_ctx *ctx, const int32_t *block_ids, int32_t bs);
  * while others still denoise).  out_ids [device][bs, gen_len]; commit_step (may be NULL)
  * [device][bs, gen_len]: 1-based step within its block at which each position was committed;
  * host_stats [host] may be NULL.  Waits for the stream.  Errors: SHAPE when gen_len is not a
- * multiple of B or prefix + gen_len > max_seq.
+ * multiple of B or prefix + gen_len > max_seq; INVALID_ARG when a prefix is negative.
  * While 2 * bs * B <= 64 rows (and the context was created with 2 * max_batch * B <= 64), the finalize
  * forward of a block and the first denoise step of the next block run as one forward of 2B rows per
  * sequence, the finished block unable to see the new one: same results as separate forwards (bit for
@@ -264,7 +264,8 @@ int d3_read_tap(d3_ctx *ctx, float *resid_in, float *resid_out, int32_t rows);
 int d3_read_kv(d3_ctx *ctx, int32_t layer, int32_t seq, int32_t pos0, int32_t n, float *k_out, float *v_out);
 
 /* Per-sequence prefix lengths ([device][bs]).  Setting them rewinds or advances the cache
- * cursor; cache contents are untouched. */
+ * cursor; cache contents are untouched.  The values are not looked at here: a later forward reports rows that
+ * would fall outside [0, max_seq) in the error word (bit 2) and neither writes nor reads there. */
 int d3_get_state(d3_ctx *ctx, int32_t *prefix_len, int32_t bs);
 int d3_set_state(d3_ctx *ctx, const int32_t *prefix_len, int32_t bs);
 

@@ -2126,7 +2126,7 @@ extern "C" int d3_denoise_step(d3_ctx* c, int32_t* block_ids, uint8_t* mask, flo
   if (!c->prefilled) return fail(c, D3_ERR_STATE, "d3_denoise_step before d3_prefill");
   if (bs > c->cfg.max_batch) return fail(c, D3_ERR_SHAPE, "bs > max_batch");
   const int B = c->cfg.block;
-  decode_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(c->prefix_len, bs, B, c->pos_base, c->n_valid, c->kv_len);
+  decode_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(c->prefix_len, bs, B, c->cfg.max_seq, c->pos_base, c->n_valid, c->kv_len);
   LAUNCHED(c, "decode_rowmap_kernel");
   c->draw_step = nullptr;  // sampling noise of the explicit calls: steps counted since the last prefill / commit
   c->draw_step_add = ++c->explicit_step;
@@ -2142,7 +2142,7 @@ extern "C" int d3_commit_block(d3_ctx* c, const int32_t* block_ids, int32_t bs) 
   if (!c->prefilled) return fail(c, D3_ERR_STATE, "d3_commit_block before d3_prefill");
   if (bs > c->cfg.max_batch) return fail(c, D3_ERR_SHAPE, "bs > max_batch");
   const int B = c->cfg.block;
-  decode_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(c->prefix_len, bs, B, c->pos_base, c->n_valid, c->kv_len);
+  decode_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(c->prefix_len, bs, B, c->cfg.max_seq, c->pos_base, c->n_valid, c->kv_len);
   LAUNCHED(c, "decode_rowmap_kernel");
   TRY(forward(c, block_ids, bs, B, 0, nullptr));
   hist_store_kernel<<<bs, 128, 0, c->stream>>>(block_ids, B, nullptr, B, c->prefix_len, c->hist_ids, c->cfg.max_seq);
@@ -2164,8 +2164,10 @@ extern "C" int d3_generate(d3_ctx* c, int32_t gen_len, float threshold, int32_t 
     std::vector<int> pl(bs);
     CUDA_TRY(c, cudaMemcpyAsync(pl.data(), c->prefix_len, sizeof(int) * bs, cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    for (int b = 0; b < bs; ++b)
-      if (pl[b] + gen_len > c->cfg.max_seq) return fail(c, D3_ERR_SHAPE, "prefix + gen_len exceeds max_seq");
+    for (int b = 0; b < bs; ++b) {
+      if (pl[b] < 0) return fail(c, D3_ERR_INVALID_ARG, "negative prefix length");
+      if (static_cast<long long>(pl[b]) + gen_len > c->cfg.max_seq) return fail(c, D3_ERR_SHAPE, "prefix + gen_len exceeds max_seq");
+    }
   }
   const int n_blocks = gen_len / B;
   const int64_t launches0 = c->launches;
@@ -2231,8 +2233,10 @@ extern "C" int d3_generate_multiblock(d3_ctx* c, int32_t gen_len, float threshol
     std::vector<int> pl(bs);
     CUDA_TRY(c, cudaMemcpyAsync(pl.data(), c->prefix_len, sizeof(int) * bs, cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    for (int b = 0; b < bs; ++b)
-      if (pl[b] + gen_len > c->cfg.max_seq) return fail(c, D3_ERR_SHAPE, "prefix + gen_len exceeds max_seq");
+    for (int b = 0; b < bs; ++b) {
+      if (pl[b] < 0) return fail(c, D3_ERR_INVALID_ARG, "negative prefix length");
+      if (static_cast<long long>(pl[b]) + gen_len > c->cfg.max_seq) return fail(c, D3_ERR_SHAPE, "prefix + gen_len exceeds max_seq");
+    }
   }
   const int n_blocks = gen_len / B;
   const int W = MB_MAX_WINDOW;
@@ -2345,7 +2349,7 @@ extern "C" int d3_forward_logits(d3_ctx* c, const int32_t* block_ids, int32_t bs
   if (!c->prefilled) return fail(c, D3_ERR_STATE, "d3_forward_logits before d3_prefill");
   if (bs > c->cfg.max_batch) return fail(c, D3_ERR_SHAPE, "bs > max_batch");
   const int B = c->cfg.block;
-  decode_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(c->prefix_len, bs, B, c->pos_base, c->n_valid, c->kv_len);
+  decode_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(c->prefix_len, bs, B, c->cfg.max_seq, c->pos_base, c->n_valid, c->kv_len);
   LAUNCHED(c, "decode_rowmap_kernel");
   return forward(c, block_ids, bs, B, 2, logits);
 }
@@ -2359,7 +2363,7 @@ extern "C" int d3_denoise_window(d3_ctx* c, const int32_t* window_ids, int32_t b
   const long long rows = static_cast<long long>(bs) * n_win * B;
   if (bs > c->cfg.max_batch || rows > std::min<long long>(c->stat_rows, c->max_rows))
     return fail(c, D3_ERR_SHAPE, "bs * n_win * block rows exceed the workspaces (raise max_batch at d3_create)");
-  decode_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(c->prefix_len, bs, n_win * B, c->pos_base, c->n_valid, c->kv_len);
+  decode_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(c->prefix_len, bs, n_win * B, c->cfg.max_seq, c->pos_base, c->n_valid, c->kv_len);
   LAUNCHED(c, "decode_rowmap_kernel");
   c->draw_step = nullptr;
   c->draw_step_add = ++c->explicit_step;
@@ -2479,7 +2483,7 @@ extern "C" int d3_op_attention(d3_ctx* c, const void* q, int32_t layer, int32_t 
   if (!q || !out || !kv_len || layer < 0 || layer >= c->cfg.n_layers || bs <= 0 || bs > c->cfg.max_batch || rows <= 0)
     return fail(c, D3_ERR_INVALID_ARG, "bad op_attention arguments");
   // all rows live, positions irrelevant here
-  decode_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(kv_len, bs, rows, c->pos_base, c->n_valid, c->kv_len);
+  decode_rowmap_kernel<<<(bs + 63) / 64, 64, 0, c->stream>>>(kv_len, bs, rows, c->cfg.max_seq, c->pos_base, c->n_valid, c->kv_len);
   LAUNCHED(c, "decode_rowmap_kernel");
   RowMap rm{c->pos_base, c->n_valid, kv_len, rows, bs, 0};
   return run_attention(c, q, layer, out, rm);

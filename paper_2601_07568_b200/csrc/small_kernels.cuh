@@ -868,8 +868,9 @@ __global__ void hist_store_kernel(const int* __restrict__ src, int src_stride, c
   const int b = blockIdx.x;
   int n = count ? count[b] : fixed_count;
   const int o = off ? off[b] : 0;
+  if (o < 0 || o >= max_seq) return;
   n = n < 0 ? 0 : (n > src_stride ? src_stride : n);
-  if (o + n > max_seq) n = max_seq - o;
+  if (n > max_seq - o) n = max_seq - o;
   for (int r = threadIdx.x; r < n; r += blockDim.x) hist[static_cast<size_t>(b) * max_seq + o + r] = src[static_cast<size_t>(b) * src_stride + r];
 }
 // Row map and input ids of a KV-refresh forward over the stored prefixes: rows_per_seq = p_max, rows
@@ -997,13 +998,15 @@ __global__ void __launch_bounds__(256) noisy_sequence4_kernel(const int4* __rest
   out[at] = v;
 }
 
-// Row maps for the explicit API.
-__global__ void decode_rowmap_kernel(const int* prefix_len, int bs, int B, int* pos_base, int* n_valid, int* kv_len) {
+// Row maps for the explicit API.  (A prefix can have been set to anything: rows outside the cache are reported where they
+// would be written, and attention reads no further than the cache.)
+__global__ void decode_rowmap_kernel(const int* prefix_len, int bs, int B, int max_seq, int* pos_base, int* n_valid, int* kv_len) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= bs) return;
+  const long long end = static_cast<long long>(prefix_len[b]) + B;
   pos_base[b] = prefix_len[b];
   n_valid[b] = B;
-  kv_len[b] = prefix_len[b] + B;
+  kv_len[b] = static_cast<int>(end < 0 ? 0 : (end > max_seq ? max_seq : end));
 }
 __global__ void prefill_rowmap_kernel(const int* prompt_lens, int bs, int p_max, int* prefix_len, int* pos_base,
                                       int* n_valid, int* kv_len) {

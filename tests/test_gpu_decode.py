@@ -943,6 +943,41 @@ def test_empty_prompt_and_state_errors():
         assert ctx.error_word() & 2  # token id outside the vocabulary is reported, not dereferenced
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("prefix", [-1, -40, 2 ** 31 - 8, 90])
+def test_prefixes_outside_the_cache(dtype, prefix):
+    """A prefix set to a value at which a block does not fit: steps and commits report the position, nothing outside the
+    cache is read or written, the other sequences are decoded as ever, and the generate loops refuse the call."""
+    shape = si.TINY if dtype == "f32" else small_bf16(128, 4, 2, "outside")
+    B, max_seq = 16, 96
+    lens = np.array([20, 33, 7], dtype=np.int32)
+    ids = np.random.default_rng(6).integers(0, shape.vocab - 2, size=(3, 33)).astype(np.int32)
+    blk = np.full((3, B), shape.mask_id, dtype=np.int32)
+    with Ctx(shape, si.gen_weights(shape), block=B, max_batch=3, max_seq=max_seq) as ctx:
+        ctx.prefill(ids, lens)
+        want = ctx.logits(blk)
+        assert ctx.error_word() == 0
+        for at in range(3):
+            prefixes = [int(n) for n in lens]
+            prefixes[at] = prefix
+            ctx.set_prefix(prefixes)
+            got = ctx.logits(blk)
+            for b in range(3):
+                assert b == at or np.array_equal(got[b], want[b])
+            assert ctx.error_word() == 4
+            d3.d3_clear_error_word(ctx.ctx)
+            ctx.commit(blk)
+            assert ctx.error_word() == 4
+            d3.d3_clear_error_word(ctx.ctx)
+            ctx.set_prefix(prefixes)
+            for run in (lambda: ctx.generate(3, 2 * B, 0.5), lambda: ctx.generate_multiblock(3, 2 * B, 0.5, 1)):
+                with pytest.raises(d3.D3Error) as ei:
+                    run()
+                assert ei.value.code == (d3.D3_ERR_INVALID_ARG if prefix < 0 else d3.D3_ERR_SHAPE)
+            ctx.prefill(ids, lens)
+            assert np.array_equal(ctx.logits(blk), want) and ctx.error_word() == 0
+
+
 @pytest.mark.parametrize("hq,hkv,bs,plens", [(4, 4, 1, [45]), (4, 2, 1, [45]), (4, 4, 2, [33, 7]), (2, 1, 2, [20, 64])])
 def test_chain_launch_small_models(hq, hkv, bs, plens):
     """Decode forwards of up to 64 rows run all layers as one chain launch (QKV, attention, O-proj, gate/up
