@@ -25,7 +25,10 @@
  *   - Calls enqueue work on the stream given to d3_create() and return
  *     without waiting, except where stated (d3_generate, d3_load_weights,
  *     d3_get_error_word).
- *   - One context per host thread.  No global state.
+ *   - One context per host thread.  Global state: the tensor-core contexts alive on each device and their streams are
+ *     counted (under a lock).  While they are on more than one stream, on cudaStreamPerThread, and in captures, launches
+ *     whose CTAs wait for one another are made as cooperative launches, so that contexts need no ordering between them.
+ *     The stream has to outlive the context.
  *   - Matrices are row-major [out_features, in_features]; activations are
  *     row-major [rows, features].  Token ids are int32.  Element type is
  *     float (D3_DTYPE_F32) or bfloat16 (D3_DTYPE_BF16) as the config says.
@@ -365,7 +368,8 @@ int d3_profile_read(d3_ctx *ctx, double *ms, int64_t *launches);
 int d3_get_error_word(d3_ctx *ctx, uint32_t *word);
 /* Number of this library's kernels launched on the context since creation. */
 int64_t d3_launch_count(d3_ctx *ctx);
-/* The same for one kernel, by its name in the source (e.g. "gemm_strip_kernel"); 0 for unknown names. */
+/* The same for one kernel, by its name in the source (e.g. "gemm_strip_kernel"); 0 for unknown names.  "cooperative": the
+ * cooperative launches among all of them. */
 int64_t d3_launch_count_of(d3_ctx *ctx, const char *kernel);
 /* Bytes of device memory the context holds. */
 int64_t d3_device_bytes(d3_ctx *ctx);

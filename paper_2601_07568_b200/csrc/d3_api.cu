@@ -45,7 +45,7 @@ struct d3_ctx {
   size_t esz = 4;
   int n_sms = 148;
   int device = 0;
-  cudaEvent_t order_event = nullptr;  // see ordered_launch
+  bool counted = false;  // see stream_use_add
   // weights (context dtype), repacked
   void* tok_emb = nullptr;
   void* lm_head = nullptr;
@@ -301,19 +301,26 @@ constexpr long long FUSE_MAX_ROWS = 64;
 constexpr long long FUSE_HALF_ROWS = 256, FUSE_ALL_ROWS = 512;
 
 // ---- launches whose CTAs wait for one another
-// The chain and the launches of resident CTA pairs need all their CTAs on the device at once.  Two of them on different
-// streams (contexts of two threads, say) could each get a part of the SMs and wait for the rest until their waits run
-// out, so such launches of a process are put in one order per device: a launch on another stream than the one before
-// waits for that stream's work so far.  One context, or several on one stream, never wait for anything here.
-// (A cooperative launch gives the same guarantee, but no longer overlaps its start with the kernel before: 4.6 us a launch.)
-struct LaunchOrder {
+// The chain and the launches of resident CTA pairs need all their CTAs on the device at once.  A stream runs such launches
+// one after the other; those of two streams could each get a part of the SMs and wait for the rest until their waits run
+// out.  So they are cooperative launches, whose CTAs the device takes all together or not yet, wherever more than one stream
+// can bring them: when tensor-core contexts on different streams share the device, on the per-thread default stream (one
+// handle, a stream for every thread), and in captures (a graph runs on whatever stream it is launched into).  Otherwise they
+// are ordinary dependent launches: a cooperative one does not overlap its start with the kernel before, 4.6 us a launch.
+// (An event wait between the streams instead holds a launch back behind everything that is queued on the other one.)
+struct StreamUse {
   std::mutex lock;
-  std::map<int, std::pair<cudaStream_t, const d3_ctx*>> last;  // per device: stream and context of the latest such launch
+  std::map<int, std::map<cudaStream_t, int>> contexts;  // per device and stream: tensor-core contexts alive
+  bool shared(int device) const {
+    auto it = contexts.find(device);
+    return it != contexts.end() && (it->second.size() > 1 || it->second.count(cudaStreamPerThread) != 0);
+  }
 };
-LaunchOrder& launch_order() {
-  static LaunchOrder order;
-  return order;
+StreamUse& stream_use() {
+  static StreamUse* use = new StreamUse();  // (never destroyed: contexts may go after the library's static objects)
+  return *use;
 }
+cudaStream_t stream_key(cudaStream_t s) { return s == cudaStreamLegacy ? nullptr : s; }
 bool capturing(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
@@ -322,19 +329,40 @@ bool capturing(cudaStream_t s) {
   }
   return st != cudaStreamCaptureStatusNone;
 }
+// A new context.  Where it is the first on a second stream, the ordinary launches that the other stream still has queued
+// are waited for: from here on all are cooperative.
+void stream_use_add(d3_ctx* c) {
+  StreamUse& use = stream_use();
+  std::lock_guard<std::mutex> hold(use.lock);
+  auto& of = use.contexts[c->device];
+  const bool was = use.shared(c->device);
+  ++of[stream_key(c->stream)];
+  c->counted = true;
+  if (was || !use.shared(c->device)) return;
+  for (const auto& other : of)
+    if (other.first != stream_key(c->stream) && other.first != cudaStreamPerThread && !capturing(other.first)) cudaStreamSynchronize(other.first);
+}
+void stream_use_remove(d3_ctx* c) {
+  if (!c->counted) return;
+  StreamUse& use = stream_use();
+  std::lock_guard<std::mutex> hold(use.lock);
+  auto& of = use.contexts[c->device];
+  if (--of[stream_key(c->stream)] == 0) of.erase(stream_key(c->stream));
+}
+// `at` is the attribute array of `cfg`, with room for one more.
 template <typename Launch>
-int ordered_launch(d3_ctx* c, Launch&& launch) {
-  LaunchOrder& order = launch_order();
-  std::lock_guard<std::mutex> hold(order.lock);
-  auto it = order.last.find(c->device);
-  // (what is captured runs when the graph does: its order is the graph launches')
-  if (it != order.last.end() && it->second.first != c->stream && !capturing(c->stream) && !capturing(it->second.first)) {
-    if (!c->order_event) CUDA_TRY(c, cudaEventCreateWithFlags(&c->order_event, cudaEventDisableTiming));
-    CUDA_TRY(c, cudaEventRecord(c->order_event, it->second.first));
-    CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->order_event, 0));
+int launch_resident(d3_ctx* c, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, Launch&& launch) {
+  StreamUse& use = stream_use();
+  std::lock_guard<std::mutex> hold(use.lock);
+  if (use.shared(c->device) || capturing(c->stream)) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeCooperative;
+    at[cfg.numAttrs++].val.cooperative = 1;
+    c->launches_by_kernel["cooperative"]++;
+  } else if (c->pdl && !c->prof_on) {
+    at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
   }
   CUDA_TRY(c, launch());
-  order.last[c->device] = {c->stream, c};
   return D3_OK;
 }
 
@@ -921,14 +949,9 @@ int run_chain(d3_ctx* c, int op_begin, int op_end, const RowMap& rm) {
   at[na].val.clusterDim.y = 1;
   at[na].val.clusterDim.z = 1;
   ++na;
-  if (c->pdl && !c->prof_on) {
-    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
-  }
   cfg.attrs = at;
   cfg.numAttrs = na;
-  TRY(ordered_launch(c, [&] { return cudaLaunchKernelEx(&cfg, tc::chain_kernel, *t_o, *t_xb, *t_h, c->kv_tmap32, p); }));
+  TRY(launch_resident(c, cfg, at, [&] { return cudaLaunchKernelEx(&cfg, tc::chain_kernel, *t_o, *t_xb, *t_h, c->kv_tmap32, p); }));
   LAUNCHED(c, "chain_kernel");
   return D3_OK;
 }
@@ -1114,12 +1137,7 @@ int run_sk(d3_ctx* c, const SkMatmul* mm, int n, int M) {
     }
   }
   cfg.gridDim = dim3(static_cast<unsigned>(2 * P));
-  if (c->pdl && !c->prof_on) {
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 2;
-  }
-  TRY(ordered_launch(c, [&] { return cudaLaunchKernelEx(&cfg, tc::gemm_sk_kernel, p); }));
+  TRY(launch_resident(c, cfg, at, [&] { return cudaLaunchKernelEx(&cfg, tc::gemm_sk_kernel, p); }));
   LAUNCHED(c, "gemm_sk_kernel");
   return D3_OK;
 }
@@ -1902,6 +1920,7 @@ extern "C" int d3_create(const d3_config* cfg, void* cuda_stream, d3_ctx** out) 
         cudaStreamSynchronize(c->stream) != cudaSuccess)
       return bail(D3_ERR_CUDA);
   }
+  if (c->use_tc) stream_use_add(c);
   *out = c;
   return D3_OK;
 }
@@ -1909,13 +1928,7 @@ extern "C" int d3_create(const d3_config* cfg, void* cuda_stream, d3_ctx** out) 
 extern "C" void d3_destroy(d3_ctx* c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
-  {
-    LaunchOrder& order = launch_order();
-    std::lock_guard<std::mutex> hold(order.lock);
-    auto it = order.last.find(c->device);
-    if (it != order.last.end() && it->second.second == c) order.last.erase(it);  // its work is done, and its stream may go
-  }
-  if (c->order_event) cudaEventDestroy(c->order_event);
+  stream_use_remove(c);
   for (auto& pp : c->prof_pool) {
     cudaEventDestroy(pp.a);
     cudaEventDestroy(pp.b);

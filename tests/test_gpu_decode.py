@@ -738,6 +738,60 @@ def test_two_contexts_on_two_streams():
             ctx.close()
 
 
+def test_launches_that_wait_are_cooperative_between_streams():
+    """A context alone on its device makes its waiting launches (resident pairs, the chain) as ordinary ones; with a second
+    context on another stream, on the per-thread default stream and in a capture they are cooperative, with the same bits;
+    a context on the same stream, and an fp32 one anywhere, change nothing."""
+    shape = si.scaled_shape(si.LLADA8B, name="small-coop", n_layers=2, d_model=256, n_q_heads=4, n_kv_heads=2,
+                            d_ffn=640, vocab=1024, d_head=128)
+    W = si.gen_weights(shape)
+    tiny = d3.make_config(si.TINY, block=16, max_batch=1, max_seq=64)
+    names = ("gemm_sk_kernel", "chain_kernel", "cooperative")
+    for bs, kernel in ((3, 0), (1, 1)):
+        ids = np.random.default_rng(4).integers(0, shape.vocab - 2, size=(bs, 40)).astype(np.int32)
+        lens, blk = np.full(bs, 40, dtype=np.int32), torch.full((bs, 32), shape.mask_id, dtype=torch.int32, device=DEV)
+        lg = torch.zeros((bs * 32, shape.vocab), dtype=torch.float32, device=DEV)
+
+        def forward(ctx):
+            n0 = [d3.d3_launch_count_of(ctx.ctx, k) for k in names]
+            lg.zero_()
+            d3.d3_forward_logits(ctx.ctx, blk, lg)
+            torch.cuda.synchronize()
+            n = [d3.d3_launch_count_of(ctx.ctx, k) - m for k, m in zip(names, n0)]
+            assert n[kernel] > 0 and n[1 - kernel] == 0 and ctx.error_word() == 0
+            return n[2] == n[kernel] if n[2] else None, lg.clone()
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            with Ctx(shape, W, block=32, max_batch=bs, max_seq=128) as ctx:
+                ctx.prefill(ids, lens)
+                alone, want = forward(ctx)
+                assert alone is None
+                same_stream, other = d3.d3_create(d3.make_config(shape, block=32, max_batch=1, max_seq=64)), d3.d3_create(tiny, torch.cuda.Stream())
+                assert forward(ctx)[0] is None
+                second = d3.d3_create(d3.make_config(shape, block=32, max_batch=1, max_seq=64), torch.cuda.Stream())
+                together, got = forward(ctx)
+                assert together and torch.equal(got, want)
+                for c in (second, same_stream, other):
+                    d3.d3_destroy(c)
+                assert forward(ctx)[0] is None
+                n0 = d3.d3_launch_count_of(ctx.ctx, "cooperative")
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph, stream=stream):
+                    d3.d3_forward_logits(ctx.ctx, blk, lg)
+                assert d3.d3_launch_count_of(ctx.ctx, "cooperative") > n0
+                for _ in range(3):
+                    lg.zero_()
+                    graph.replay()
+                    torch.cuda.synchronize()
+                    assert torch.equal(lg, want)
+                del graph
+        with torch.cuda.stream(torch.cuda.ExternalStream(2)):  # cudaStreamPerThread
+            with Ctx(shape, W, block=32, max_batch=bs, max_seq=128) as ctx:
+                ctx.prefill(ids, lens)
+                together, got = forward(ctx)
+                assert together and torch.equal(got, want)
+
+
 @pytest.mark.parametrize("lens,tau", [([40, 7, 97], 0.0), ([40, 7, 97, 64], 0.0), ([40, 7, 97, 64], 0.3), ([33] * 6, 0.3), ([33, 5] * 4, 0.0)])
 def test_fused_finalize_of_batches(lens, tau):
     """Batches finalize a block together with the next block's first step where half of the sequences are at a border (up to
