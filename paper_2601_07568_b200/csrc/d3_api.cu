@@ -811,6 +811,36 @@ int chain_max_clusters(d3_ctx* c, size_t smem) {
 
 constexpr int CHAIN_OPS_PER_LAYER = 5;  // QKV, attention, O-proj, gate/up, down
 
+// Shape of a chain launch.  Returns why there is none, or null.
+struct ChainPlan {
+  int n_clusters, a_rows, max_strip, stages;
+  size_t recv, smem;
+};
+const char* chain_plan(d3_ctx* c, int bs, int M, ChainPlan& p) {
+  const d3_config& g = c->cfg;
+  const int d = g.d_model, nq = g.n_q_heads * g.d_head, nkv = g.n_kv_heads * g.d_head, f = g.d_ffn;
+  // the grid: as many clusters as are resident at once (every CTA waits for every other at the borders)
+  if (c->chain_clusters < 0) c->chain_clusters = std::min(chain_max_clusters(c, 224 * 1024), c->n_sms / tc::CHAIN_C);
+  p.n_clusters = c->tune_chain_clusters > 0 ? std::min(c->chain_clusters, c->tune_chain_clusters) : c->chain_clusters;
+  if (p.n_clusters < 8 || p.n_clusters < bs * g.n_kv_heads) return "the chain kernel needs a resident cluster per (sequence, kv head) pair";
+  p.a_rows = M <= 32 ? 32 : 64;
+  auto strip_cols = [&](int N, int unit, int groups) { return ((N / unit + groups - 1) / groups) * unit; };
+  const int qkv_cols = strip_cols(nq + 2 * nkv, 32, p.n_clusters * (tc::CHAIN_C / c->chain_qkv_ks));
+  const int o_cols = strip_cols(d, 32, p.n_clusters);
+  const int gu_cols = strip_cols(2 * f, 16, p.n_clusters * tc::CHAIN_C);
+  p.max_strip = std::max(std::max(qkv_cols, o_cols), gu_cols);
+  if (p.max_strip > 256) return "a chain strip would be wider than 256 columns";
+  p.recv = std::max(std::max<size_t>(tc::chain_recv_bytes(p.a_rows, std::max(qkv_cols, o_cols)), sizeof(float) * tc::CHAIN_ARECV_FLOATS),
+                    static_cast<size_t>(tc::CHAIN_ASTAGES) * tc::CHAIN_ASTAGE_BYTES);
+  const size_t budget = (c->tune_ring_kb > 0 ? c->tune_ring_kb : 222) * 1024;  // whole CTA
+  const size_t stage_bytes = static_cast<size_t>(p.a_rows + p.max_strip) * 128;
+  const size_t fixed = tc::chain_fixed_smem_bytes(p.recv, 16);
+  p.stages = std::max(2, std::min(static_cast<int>((budget > fixed ? budget - fixed : 0) / stage_bytes), 16));
+  p.smem = tc::chain_smem_bytes(p.a_rows, static_cast<uint32_t>(p.max_strip) * 128u, p.stages, p.recv);
+  if (p.smem > 224 * 1024) return "the chain kernel's shared memory does not fit";
+  return nullptr;
+}
+
 // Can a forward of bs x rows_per_seq rows run as a chain?  (bf16 tensor-core context with the fused QKV
 // epilogue and folded norms; every (sequence, kv head) pair gets a cluster; all CTAs resident at once.)
 bool chain_usable(d3_ctx* c, int bs, int rows_per_seq, int seg) {
@@ -824,7 +854,8 @@ bool chain_usable(d3_ctx* c, int bs, int rows_per_seq, int seg) {
   if ((g.n_q_heads / g.n_kv_heads) * rows_per_seq > 64) return false;  // packed rows of a kv head: one attention tile
   if (seg > 0 && seg % 16 != 0) return false;                         // a 16-row group lies in one segment
   if (rows_per_seq % 16 != 0 && (g.n_q_heads / g.n_kv_heads) > 1) return false;
-  return true;
+  ChainPlan plan;
+  return c->tune_chain_clusters > 0 || chain_plan(c, bs, M, plan) == nullptr;  // (a number of clusters asked for by name is used or refused)
 }
 
 // The program of a forward: QKV, attention, O-proj, gate/up, down per layer.  Built once (all
@@ -883,40 +914,19 @@ int run_chain(d3_ctx* c, int op_begin, int op_end, const RowMap& rm) {
   ProfScope ps(c, D3_PROF_CHAIN);
   const d3_config& g = c->cfg;
   const int M = rm.bs * rm.rows_per_seq;
-  const int a_rows = M <= 32 ? 32 : 64;
-  const int d = g.d_model, nq = g.n_q_heads * g.d_head, nkv = g.n_kv_heads * g.d_head, f = g.d_ffn;
-  // the grid: as many clusters as are resident at once (every CTA waits for every other at the borders)
-  int n_clusters = c->chain_clusters;
-  if (n_clusters < 0) {
-    n_clusters = std::min(chain_max_clusters(c, 224 * 1024), c->n_sms / tc::CHAIN_C);
-    c->chain_clusters = n_clusters;
-  }
-  if (c->tune_chain_clusters > 0) n_clusters = std::min(n_clusters, c->tune_chain_clusters);
-  if (n_clusters < 8 || n_clusters < rm.bs * g.n_kv_heads)
-    return fail(c, D3_ERR_UNSUPPORTED, "the chain kernel needs a resident cluster per (sequence, kv head) pair");
-  const int n_cta = n_clusters * tc::CHAIN_C;
-  auto strip_cols = [&](int N, int unit, int groups) { return ((N / unit + groups - 1) / groups) * unit; };
-  const int qkv_cols = strip_cols(nq + 2 * nkv, 32, n_clusters * (tc::CHAIN_C / c->chain_qkv_ks));
-  const int o_cols = strip_cols(d, 32, n_clusters);
-  const int gu_cols = strip_cols(2 * f, 16, n_cta);
-  const int max_strip = std::max(std::max(qkv_cols, o_cols), gu_cols);
-  if (max_strip > 256) return fail(c, D3_ERR_UNSUPPORTED, "a chain strip would be wider than 256 columns");
+  const int d = g.d_model, nq = g.n_q_heads * g.d_head, f = g.d_ffn;
+  ChainPlan plan;
+  if (const char* why = chain_plan(c, rm.bs, M, plan)) return fail(c, D3_ERR_UNSUPPORTED, why);
+  const int a_rows = plan.a_rows;
   tc::ChainParams p{};
   p.prog = static_cast<const tc::ChainOp*>(c->chain_prog);
   p.op_begin = op_begin; p.op_end = op_end;
   p.M = M;
   p.a_rows = a_rows;
-  p.w_stage_bytes = static_cast<uint32_t>(max_strip) * 128u;
-  const size_t recv = std::max(std::max<size_t>(tc::chain_recv_bytes(a_rows, std::max(qkv_cols, o_cols)), sizeof(float) * tc::CHAIN_ARECV_FLOATS),
-                               static_cast<size_t>(tc::CHAIN_ASTAGES) * tc::CHAIN_ASTAGE_BYTES);
-  p.recv_bytes = static_cast<int>(recv);
+  p.w_stage_bytes = static_cast<uint32_t>(plan.max_strip) * 128u;
+  p.recv_bytes = static_cast<int>(plan.recv);
   p.l2_ahead = c->tune_chain_l2 >= 0 ? c->tune_chain_l2 : 0;  // off by default: measured neutral at 12 slabs, slower beyond
-  const size_t budget = (c->tune_ring_kb > 0 ? c->tune_ring_kb : 222) * 1024;  // whole CTA
-  const size_t stage_bytes = static_cast<size_t>(a_rows) * 128 + p.w_stage_bytes;
-  const size_t fixed = tc::chain_fixed_smem_bytes(recv, 16);
-  int stages = static_cast<int>((budget > fixed ? budget - fixed : 0) / stage_bytes);
-  stages = std::max(2, std::min(stages, 16));
-  p.stages = stages;
+  p.stages = plan.stages;
   p.sync = c->chain_sync;
   p.error_word = c->error_word;
   p.skip_flag = c->skip_flag;
@@ -930,17 +940,15 @@ int run_chain(d3_ctx* c, int op_begin, int op_end, const RowMap& rm) {
   TRY(get_tmap(c, c->o, M, nq, a_rows, &t_o));
   TRY(get_tmap(c, c->xb, M, d, a_rows, &t_xb));
   TRY(get_tmap(c, c->h, M, f, a_rows, &t_h));
-  const size_t smem = tc::chain_smem_bytes(a_rows, p.w_stage_bytes, stages, recv);
-  if (smem > 224 * 1024) return fail(c, D3_ERR_UNSUPPORTED, "the chain kernel's shared memory does not fit");
   static bool attr_set = false;
   if (!attr_set) {
     CUDA_TRY(c, cudaFuncSetAttribute(tc::chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024));
     attr_set = true;
   }
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned>(n_cta));
+  cfg.gridDim = dim3(static_cast<unsigned>(plan.n_clusters * tc::CHAIN_C));
   cfg.blockDim = dim3(tc::CHAIN_THREADS);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = plan.smem;
   cfg.stream = c->stream;
   cudaLaunchAttribute at[2];
   int na = 0;

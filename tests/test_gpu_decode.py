@@ -1079,3 +1079,33 @@ def test_chain_launch_small_models(hq, hkv, bs, plens):
             record_report(f"chain_free_running_{hq}_{hkv}", r2)
             assert r2["resyncs"] <= r2["blocks"] and max(r2["margins"], default=0.0) <= 1e-2, r2
             assert d3.d3_launch_count_of(ctx.ctx, "chain_kernel") > 0 and ctx.error_word() == 0
+
+
+@pytest.mark.parametrize("block,bs", [(32, 2), (16, 2), (16, 4)])
+def test_more_pairs_than_the_chain_has_clusters(block, bs):
+    """Two sequences of 32 kv heads are 64 (sequence, kv head) pairs, more than clusters of four CTAs fit the device: such
+    forwards of up to 64 rows run on the other launches.  A step, both generate loops (with fused forwards of 64 rows) and
+    a short prompt batch, against the plain bf16 kernels."""
+    shape = si.scaled_shape(si.LLADA8B, name="many-heads", n_layers=2, d_model=256, n_q_heads=32, n_kv_heads=32,
+                            d_ffn=512, vocab=1024, d_head=128)
+    W = si.gen_weights(shape)
+    lens = np.array([20, 11, 16, 5][:bs], dtype=np.int32)
+    ids = np.random.default_rng(8).integers(0, shape.vocab - 2, size=(bs, 20)).astype(np.int32)
+    blk = np.full((bs, block), shape.mask_id, dtype=np.int32)
+    blk[:, ::3] = 7
+    lg = []
+    for impl in (0, 1):
+        with Ctx(shape, W, block=block, max_batch=2 * bs, max_seq=160, gemm_impl=impl) as ctx:
+            ctx.prefill(ids, lens)
+            lg.append(ctx.logits(blk))
+            if impl == 0:
+                assert d3.d3_launch_count_of(ctx.ctx, "chain_kernel") == 0
+                step = ctx.step(blk, blk == shape.mask_id, 0.5)
+                assert (step["count"] >= 1).all()
+                for run in (lambda: ctx.generate(bs, 2 * block, 0.3), lambda: ctx.generate_multiblock(bs, 2 * block, 0.3, 2)):
+                    ctx.prefill(ids, lens)
+                    tok, _, st = run()
+                    assert st.tokens_committed == bs * 2 * block and (tok != shape.mask_id).all()
+                assert d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel") > 0
+            assert ctx.error_word() == 0
+    assert np.max(np.abs(lg[0] - lg[1])) <= 3e-2 * np.max(np.abs(lg[1]))
