@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -212,6 +213,20 @@ int check_launch(d3_ctx* c, const char* what) {
     if (rc_ != D3_OK) return rc_;  \
   } while (0)
 
+// Dynamic shared memory beyond 48 KB has to be allowed for a kernel on every device, before its first launch there.
+// (Contexts of several threads and devices come here: a kernel's flags are atomic, a bit per device.)
+struct OncePerDevice {
+  std::atomic<unsigned long long> done{0};
+};
+template <typename Kernel>
+int allow_smem(d3_ctx* c, OncePerDevice& allowed, Kernel kern, size_t bytes) {
+  const unsigned long long bit = c->device < 64 ? 1ull << c->device : 0ull;
+  if (allowed.done.load(std::memory_order_acquire) & bit) return D3_OK;
+  CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes)));
+  allowed.done.fetch_or(bit, std::memory_order_release);
+  return D3_OK;
+}
+
 // ---- optional per-class timing: an event pair around every launch of the class
 void prof_flush(d3_ctx* c) {
   if (c->prof_used == 0) return;
@@ -253,7 +268,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn get_encode_fn() {
-  static EncodeTiledFn fn = nullptr;
+  static std::atomic<EncodeTiledFn> fn{nullptr};
   if (!fn) {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -395,11 +410,8 @@ template <int EPI, int BLOCK_N, int MT>
 int launch_tc(d3_ctx* c, const CUtensorMap* tx, const CUtensorMap* tw, const tc::GemmParams& p, int n_ctas,
               size_t smem) {
   auto kern = tc::gemm_tc_kernel<EPI, BLOCK_N, MT>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    attr_set = true;
-  }
+  static OncePerDevice allowed;
+  TRY(allow_smem(c, allowed, kern, 220 * 1024));
   CUDA_TRY(c, launch_pdl(c, kern, dim3(n_ctas), dim3(tc::NUM_THREADS), smem, *tx, *tw, p));
   LAUNCHED(c, "gemm_tc_kernel");
   return D3_OK;
@@ -490,11 +502,8 @@ template <int EPI>
 int launch_ck(d3_ctx* c, const CUtensorMap* tx, const CUtensorMap* tw, const tc::GemmParams& p, const tc::ClusterSplit& cs,
               size_t smem) {
   auto kern = tc::gemm_ck_kernel<EPI>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    attr_set = true;
-  }
+  static OncePerDevice allowed;
+  TRY(allow_smem(c, allowed, kern, 220 * 1024));
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(cs.n_clusters * cs.C));
   cfg.blockDim = dim3(tc::NUM_THREADS);
@@ -602,11 +611,8 @@ int run_linear_ck(d3_ctx* c, const void* X, const void* W, int M, int N, int K, 
 template <int EPI>
 int launch_xt(d3_ctx* c, const CUtensorMap* tx, const tc::GemmParams& p, const tc::XtSplit& xs, int n_ctas, size_t smem) {
   auto kern = tc::gemm_xt_kernel<EPI>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    attr_set = true;
-  }
+  static OncePerDevice allowed;
+  TRY(allow_smem(c, allowed, kern, 220 * 1024));
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(n_ctas));
   cfg.blockDim = dim3(tc::XT_THREADS);
@@ -710,14 +716,11 @@ int strip_width(const d3_ctx* c, int M, int N, int w_tiled) {
 
 template <int EPI>
 int launch_strip(d3_ctx* c, const CUtensorMap* tx, const tc::GemmParams& p, int S, int n_ctas, size_t smem) {
-  static bool attr_set[2] = {false, false};
+  static OncePerDevice allowed[2];
   // tensor memory: one accumulator of S columns per pipeline, the second one half way up
   const int wide = S * p.n_producers > 128 ? 1 : 0;
   auto kern = wide ? tc::gemm_strip_kernel<EPI, 256> : tc::gemm_strip_kernel<EPI, 128>;
-  if (!attr_set[wide]) {
-    CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    attr_set[wide] = true;
-  }
+  TRY(allow_smem(c, allowed[wide], kern, 220 * 1024));
   CUDA_TRY(c, launch_pdl(c, kern, dim3(n_ctas), dim3(tc::STRIP_THREADS), smem, *tx, p, S));
   LAUNCHED(c, "gemm_strip_kernel");
   return D3_OK;
@@ -780,11 +783,8 @@ int run_linear_strip(d3_ctx* c, const void* X, const void* W, int M, int N, int 
 }
 
 // ---- the decode forward as a chain (chain.cuh)
-// Clusters of the chain kernel that can be resident at once with `smem` bytes per CTA (asked once per size).
+// Clusters of the chain kernel that can be resident at once with `smem` bytes per CTA (a context asks once).
 int chain_max_clusters(d3_ctx* c, size_t smem) {
-  static std::map<size_t, int> cache;
-  auto it = cache.find(smem);
-  if (it != cache.end()) return it->second;
   if (cudaFuncSetAttribute(tc::chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024) != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;
@@ -805,7 +805,6 @@ int chain_max_clusters(d3_ctx* c, size_t smem) {
     (void)cudaGetLastError();
     n = 0;
   }
-  cache[smem] = n;
   return n;
 }
 
@@ -940,11 +939,8 @@ int run_chain(d3_ctx* c, int op_begin, int op_end, const RowMap& rm) {
   TRY(get_tmap(c, c->o, M, nq, a_rows, &t_o));
   TRY(get_tmap(c, c->xb, M, d, a_rows, &t_xb));
   TRY(get_tmap(c, c->h, M, f, a_rows, &t_h));
-  static bool attr_set = false;
-  if (!attr_set) {
-    CUDA_TRY(c, cudaFuncSetAttribute(tc::chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024));
-    attr_set = true;
-  }
+  static OncePerDevice allowed;
+  TRY(allow_smem(c, allowed, tc::chain_kernel, 224 * 1024));
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(plan.n_clusters * tc::CHAIN_C));
   cfg.blockDim = dim3(tc::CHAIN_THREADS);
@@ -971,11 +967,8 @@ template <int EPI>
 int launch_pair(d3_ctx* c, const CUtensorMap* tx, const CUtensorMap* tw, const tc::GemmParams& p, int tiles) {
   auto kern = tc::gemm_pair_kernel<EPI>;
   const size_t smem = tc::gemm_pair_smem_bytes();
-  static bool attr_set = false;
-  if (!attr_set) {
-    CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    attr_set = true;
-  }
+  static OncePerDevice allowed;
+  TRY(allow_smem(c, allowed, kern, smem));
   cudaLaunchConfig_t cfg{};
   cfg.blockDim = dim3(tc::PAIR_THREADS);
   cfg.dynamicSmemBytes = smem;
@@ -1263,11 +1256,8 @@ int launch_attention(d3_ctx* c, const void* q, const void* kc, const void* vc, v
 template <int NW, int KQ>
 int launch_attn_tc(d3_ctx* c, const attn::AttnTcParams& p, dim3 grid) {
   auto kern = attn::attn_tc_kernel<NW, KQ>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(attn::attn_tc_smem_bytes())));
-    attr_set = true;
-  }
+  static OncePerDevice allowed;
+  TRY(allow_smem(c, allowed, kern, attn::attn_tc_smem_bytes()));
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(NW * KQ * 32);
@@ -1297,7 +1287,7 @@ int launch_attn_tc(d3_ctx* c, const attn::AttnTcParams& p, dim3 grid) {
 // CTAs of one attention instantiation that fit an SM (registers and shared memory), asked once.
 template <int NW, int KQ>
 int attn_ctas_per_sm() {
-  static int cached = 0;
+  static std::atomic<int> cached{0};
   if (cached == 0) {
     auto kern = attn::attn_tc_kernel<NW, KQ>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(attn::attn_tc_smem_bytes()));
@@ -1314,11 +1304,8 @@ template <int KT, int SBUF>
 int launch_attn_tmem(d3_ctx* c, const attn::AttnTcParams& p, dim3 grid) {
   auto kern = attn::attn_tmem_kernel<KT, SBUF>;
   const size_t smem = attn::TmLayout<KT, SBUF>::smem_bytes();
-  static bool attr_set = false;
-  if (!attr_set) {
-    CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-    attr_set = true;
-  }
+  static OncePerDevice allowed;
+  TRY(allow_smem(c, allowed, kern, smem));
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(attn::TM_THREADS);
@@ -1356,11 +1343,8 @@ int run_attention_tmem_stream(d3_ctx* c, const void* q, int layer, void* out, co
   const d3_config& g = c->cfg;
   auto kern = attn::attn_tmem_stream_kernel;
   const size_t smem = attn::TmStream::smem_bytes((g.n_q_heads / g.n_kv_heads) * rm.rows_per_seq);
-  static bool attr_set = false;
-  if (!attr_set) {
-    CUDA_TRY(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(attn::TmStream::smem_bytes(64))));
-    attr_set = true;
-  }
+  static OncePerDevice allowed;
+  TRY(allow_smem(c, allowed, kern, attn::TmStream::smem_bytes(64)));
   attn::AttnTcParams p{};
   p.q = static_cast<const bf16*>(q);
   p.out = static_cast<bf16*>(out);

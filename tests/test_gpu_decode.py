@@ -738,6 +738,42 @@ def test_two_contexts_on_two_streams():
             ctx.close()
 
 
+def test_first_launches_from_several_threads():
+    """Contexts created and used for the first time by four threads at once, in a process in which no kernel has run."""
+    import os
+    import subprocess
+    import sys
+    code = """
+import threading
+import numpy as np
+import torch
+from gpu_utils import Ctx
+from paper_2601_07568_b200 import synth_inputs as si
+shape = si.scaled_shape(si.LLADA8B, name="cold", n_layers=2, d_model=256, n_q_heads=4, n_kv_heads=2, d_ffn=640, vocab=1024, d_head=128)
+W, got, gate = si.gen_weights(shape), {}, threading.Barrier(4)
+torch.cuda.init()
+def work(i):
+    torch.cuda.set_device(0)
+    bs = (1, 3, 8, 3)[i]
+    ids = np.random.default_rng(bs).integers(0, 1000, size=(bs, 100)).astype(np.int32)
+    with torch.cuda.stream(torch.cuda.Stream()):
+        gate.wait()
+        with Ctx(shape, W, block=32, max_batch=bs, max_seq=200) as ctx:
+            ctx.prefill(ids, np.full(bs, 100, dtype=np.int32))
+            got[i] = ctx.generate(bs, 64, 0.5)[0]
+            assert ctx.error_word() == 0
+threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+[t.start() for t in threads]
+[t.join() for t in threads]
+assert len(got) == 4 and np.array_equal(got[1], got[3])
+print("cold ok")
+"""
+    here = os.path.dirname(os.path.abspath(__file__))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([os.path.dirname(here), here, os.environ.get("PYTHONPATH", "")]))
+    r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "cold ok" in r.stdout, r.stderr[-2000:]
+
+
 def test_launches_that_wait_are_cooperative_between_streams():
     """A context alone on its device makes its waiting launches (resident pairs, the chain) as ordinary ones; with a second
     context on another stream, on the per-thread default stream and in a capture they are cooperative, with the same bits;
