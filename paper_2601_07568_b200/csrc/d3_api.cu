@@ -84,6 +84,7 @@ struct d3_ctx {
   GenState gen{};
   MbState mb{};           // multi-block decoding state (d3_generate_multiblock)
   int stat_rows = 0;      // rows the statistics buffers hold
+  bool stat_fused = false;  // the latest statistics are of a generate loop's fused forward: rows from gen.stat_row on
   long long* host_counters = nullptr;  // pinned
   // taps
   int tap_layer = -1;
@@ -1723,6 +1724,7 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   if (head == 0) return D3_OK;
   if (!c->fold_norm) TRY(run_rmsnorm(c, c->x, c->final_norm, c->xn, M));
   if (head == 1) {
+    c->stat_fused = false;
     if (!head_sk) TRY(run_linear(c, normed, c->lm_head, M, g.vocab, d, EPI_STATS, head_epi(), 0, nullptr, D3_PROF_GEMM_HEAD, c->w_tiled));
     TRY(run_stats_merge(c, M, (g.vocab + 127) / 128, c->conf, c->ent, c->argmax, c->temperature > 0.f));
   } else {
@@ -1886,6 +1888,7 @@ extern "C" int d3_create(const d3_config* cfg, void* cuda_stream, d3_ctx** out) 
   A_(c->hist_ids, sizeof(int) * static_cast<size_t>(g.max_batch) * g.max_seq);
   A_(c->refresh_ids, sizeof(int) * R);
   A_(c->gen.refresh_flag, sizeof(int) * g.max_batch);
+  A_(c->gen.stat_row, sizeof(int) * g.max_batch);
   A_(c->mb.stab, sizeof(int) * static_cast<size_t>(g.max_batch) * MB_MAX_WINDOW);
   c->gen.hist = c->hist_ids;
   c->mb.hist = c->hist_ids;
@@ -2195,6 +2198,7 @@ extern "C" int d3_generate(d3_ctx* c, int32_t gen_len, float threshold, int32_t 
     gen_rowmap_kernel<<<bs, 64, 0, c->stream>>>(g, bs, B, R, c->cfg.mask_id, c->pos_base, c->n_valid, c->kv_len);
     LAUNCHED(c, "gen_rowmap_kernel");
     TRY(forward(c, g.fwd_ids, bs, R, 1, nullptr, R > B ? B : 0));
+    c->stat_fused = R > B;
     gen_advance_kernel<<<bs, 32, 0, c->stream>>>(g, c->conf, c->ent, c->argmax, bs, B, R, n_blocks, gen_len, threshold, c->cfg.decide_mode, c->cfg.mask_id, fuse, c->eos_id,
                                                  c->cfg.max_seq, c->refresh_every);
     LAUNCHED(c, "gen_advance_kernel");
@@ -2341,6 +2345,11 @@ extern "C" int64_t d3_early_stops(d3_ctx* c) { return c ? c->last_early_stops : 
 
 extern "C" int d3_get_step_stats(d3_ctx* c, float* conf, float* entropy, int32_t* argmax, int32_t bs) {
   if (!c || bs <= 0 || bs > c->cfg.max_batch) return D3_ERR_INVALID_ARG;
+  if (c->stat_fused) {  // (two blocks of rows per sequence, and not all of them decided on the second)
+    step_stats_kernel<<<bs, 128, 0, c->stream>>>(c->conf, c->ent, c->argmax, c->gen.stat_row, c->cfg.block, conf, entropy, argmax);
+    LAUNCHED(c, "step_stats_kernel");
+    return D3_OK;
+  }
   const size_t n = static_cast<size_t>(bs) * c->cfg.block;
   if (conf) CUDA_TRY(c, cudaMemcpyAsync(conf, c->conf, n * 4, cudaMemcpyDeviceToDevice, c->stream));
   if (entropy) CUDA_TRY(c, cudaMemcpyAsync(entropy, c->ent, n * 4, cudaMemcpyDeviceToDevice, c->stream));

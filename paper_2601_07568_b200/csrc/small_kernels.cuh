@@ -472,6 +472,7 @@ struct GenState {
   long long* counters;  // [0] denoise fwd, [1] finalize fwd, [2] tokens, [3] forced, [4] seqs not done, [5] seqs in SEQ_FUSED,
                         // [6] sequences stopped early on the end-of-sequence id, [7] sequences waiting for a KV-refresh
   int* hist;            // [bs, max_seq] ids of the stored prefix (prompt and stored blocks)
+  int* stat_row;        // [bs] where the statistics of the latest forward's decision begin
   int* refresh_flag;    // [bs] 1: the stored prefix of this sequence is to be recomputed before the next forward
   unsigned long long* commit_hist;  // [COMMIT_HIST_BINS] decisions that committed k tokens (k = bin index)
   uint32_t* error_word;
@@ -506,6 +507,7 @@ __global__ void gen_advance_kernel(GenState g, const float* __restrict__ conf, c
   const int b = blockIdx.x;
   const int lane = threadIdx.x & 31;
   const int mode = g.mode[b];
+  if (lane == 0) g.stat_row[b] = b * R + (mode == SEQ_FUSED && R > B ? B : 0);
   if (mode == SEQ_DONE) return;
   int* ids = g.ids + b * B;
   uint8_t* mask = g.mask + b * B;
@@ -613,6 +615,17 @@ __global__ void gen_advance_kernel(GenState g, const float* __restrict__ conf, c
       g.step[b] = step;
       g.mode[b] = complete ? SEQ_FINALIZE : SEQ_DENOISE;
     }
+  }
+}
+
+// Statistics of the rows that the latest forward of a generate loop decided on, [bs, B] each (any output may be null).
+__global__ void step_stats_kernel(const float* __restrict__ conf, const float* __restrict__ ent, const int* __restrict__ argmax,
+                                  const int* __restrict__ stat_row, int B, float* conf_out, float* ent_out, int* argmax_out) {
+  const int b = blockIdx.x, row0 = stat_row[b];
+  for (int r = threadIdx.x; r < B; r += blockDim.x) {
+    if (conf_out) conf_out[b * B + r] = conf[row0 + r];
+    if (ent_out) ent_out[b * B + r] = ent[row0 + r];
+    if (argmax_out) argmax_out[b * B + r] = argmax[row0 + r];
   }
 }
 

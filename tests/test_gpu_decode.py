@@ -677,6 +677,35 @@ def test_first_steps_of_fused_forwards(block, bs):
         assert ctx.error_word() == 0
 
 
+@pytest.mark.parametrize("bs", [1, 3])
+def test_step_statistics_after_an_early_stop_in_a_fused_forward(bs):
+    """d3_get_step_stats after a request that the end-of-sequence token stops in the first step of a block, which ran
+    together with the finalize forward of the block before: the statistics are those of the rows decided on."""
+    shape = si.scaled_shape(si.LLADA8B, name="eos-stats", n_layers=2, d_model=256, n_q_heads=4, n_kv_heads=2,
+                            d_ffn=640, vocab=1024, d_head=128)
+    ids = np.repeat(np.random.default_rng(2).integers(0, 1000, size=(1, 37)).astype(np.int32), bs, 0)
+    lens = np.full(bs, 37, dtype=np.int32)
+    with Ctx(shape, si.gen_weights(shape), block=32, max_batch=bs, max_seq=160) as ctx:
+        ctx.prefill(ids, lens)
+        tok, _, _ = ctx.generate(bs, 96, 0.0)  # a block a step: blocks 2 and 3 begin in fused forwards
+        new = [int(t) for t in tok[0, 32:64] if t not in tok[0, :32]]
+        assert new
+        d3.d3_set_eos(ctx.ctx, new[0])
+        ctx.prefill(ids, lens)
+        got, _, st = ctx.generate(bs, 96, 0.0)
+        assert d3.d3_early_stops(ctx.ctx) == bs and st.steps == 2 and np.array_equal(got[:, :64], tok[:, :64])
+        stats = [torch.zeros(bs * 32, dtype=dt, device=DEV) for dt in (torch.float32, torch.float32, torch.int32)]
+        d3.d3_get_step_stats(ctx.ctx, *stats, bs)
+        assert np.array_equal(stats[2].cpu().numpy().reshape(bs, 32), got[:, 32:64])
+        # the same step by itself gives the same confidences and entropies, up to the order of its sums
+        ctx.prefill(ids, lens)
+        ctx.commit(got[:, :32])
+        own = ctx.step(np.full((bs, 32), shape.mask_id, dtype=np.int32), np.ones((bs, 32)), 0.0)
+        for a, b in zip(stats, (own["conf"], own["ent"])):
+            assert np.max(np.abs(a.cpu().numpy().reshape(bs, 32) - b)) <= BF16_STAT_ERR_BOUND * max(1.0, np.max(np.abs(b)))
+        assert ctx.error_word() == 0
+
+
 def test_chunk_sums_of_the_embeddings_are_the_residual_epilogue_s():
     """A layer whose output projections are zero leaves the residual stream as it was, and with it the row factors of the
     next layer: two layers with the same q, k, v matrices store the same keys and values, bit for bit."""
