@@ -129,7 +129,7 @@ struct d3_ctx {
   int tune_attn_shape = 0;      // experiment: keys per tile of the tcgen05 attention (0 = by rule, 64, 128)
   int tune_attn_tmem = -1;      // tcgen05 attention: -1 where measured faster, 0 never, 1 wherever the shape allows
   int* row_off = nullptr;      // [max_batch + 1] first row of every sequence where prompts are laid out one after the other
-  int2* row_map = nullptr;     // [max_rows, rounded up to 256] (sequence, row of it) of such a row
+  int2* row_map = nullptr;     // [ws_rows, rounded up to 256] (sequence, row of it) of such a row
   bool packed = false;         // set for the span of such a forward, over packed_bs sequences
   int packed_bs = 0;
   int tune_cta_pairs = -1;      // wide matmuls on CTA pairs (cta_group::2): -1 when the shape allows, 0 never
@@ -2187,13 +2187,14 @@ extern "C" int d3_generate(d3_ctx* c, int32_t gen_len, float threshold, int32_t 
   const long long max_iter = static_cast<long long>(n_blocks) * (B + 1) + 1;
   // (a refresh falls between a block's finalize forward and the next block's first step: no fusing then)
   const bool fuse_any = c->gen_fuse && c->refresh_every == 0 && 2ll * bs * B <= FUSE_MAX_ROWS && 2ll * c->cfg.max_batch * B <= FUSE_MAX_ROWS;
-  const bool fuse_many = c->gen_fuse && c->refresh_every == 0 && 2ll * bs * B <= c->fuse_rows && sk_forward_usable(c, 2 * bs * B);
+  // (a batch's fused forward has more rows than the tap buffers: a tapped context decodes without)
+  const bool fuse_many = c->gen_fuse && c->refresh_every == 0 && c->tap_layer < 0 && 2ll * bs * B <= c->fuse_rows && sk_forward_usable(c, 2 * bs * B);
   const int fuse = fuse_any || fuse_many ? 1 : 0;
   long long steps = 0;
   c->last_refreshes = 0;
   c->draw_step = g.step;  // sampling noise: each sequence's step within its block (the counter is bumped after the forward)
   c->draw_step_add = 1;
-  int R = B;  // rows per sequence of the next forward: 2B while some sequence runs a fused finalize + first step
+  int R = B;  // rows per sequence of the next forward: 2B where enough sequences run a fused finalize + first step (`wide` below)
   for (long long it = 0; it < max_iter; ++it) {
     gen_rowmap_kernel<<<bs, 64, 0, c->stream>>>(g, bs, B, R, c->cfg.mask_id, c->pos_base, c->n_valid, c->kv_len);
     LAUNCHED(c, "gen_rowmap_kernel");

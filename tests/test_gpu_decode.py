@@ -706,6 +706,35 @@ def test_step_statistics_after_an_early_stop_in_a_fused_forward(bs):
         assert ctx.error_word() == 0
 
 
+def test_tap_of_a_batch_that_stops_early():
+    """A tapped layer of a batch keeps the rows of the latest forward, also where the request stops at a block's first
+    step: the same rows, bit for bit, as in that step by itself."""
+    shape, bs = si.scaled_shape(si.LLADA8B, name="eos-tap", n_layers=2, d_model=256, n_q_heads=4, n_kv_heads=2,
+                                d_ffn=640, vocab=1024, d_head=128), 3
+    ids = np.repeat(np.random.default_rng(2).integers(0, 1000, size=(1, 37)).astype(np.int32), bs, 0)
+    lens = np.full(bs, 37, dtype=np.int32)
+    with Ctx(shape, si.gen_weights(shape), block=32, max_batch=bs, max_seq=160) as ctx:
+        def tapped(run):
+            d3.d3_set_tap(ctx.ctx, 0)
+            got = run()
+            t = [torch.zeros((bs * 32, shape.d_model), dtype=torch.float32, device=DEV) for _ in range(2)]
+            d3.d3_read_tap(ctx.ctx, t[0], t[1], bs * 32)
+            d3.d3_set_tap(ctx.ctx, -1)
+            return got, t
+        ctx.prefill(ids, lens)
+        tok, _, _ = ctx.generate(bs, 96, 0.0)
+        new = [int(t) for t in tok[0, 32:64] if t not in tok[0, :32]]
+        assert new
+        d3.d3_set_eos(ctx.ctx, new[0])
+        ctx.prefill(ids, lens)
+        (got, _, _), rows = tapped(lambda: ctx.generate(bs, 96, 0.0))
+        assert d3.d3_early_stops(ctx.ctx) == bs
+        ctx.prefill(ids, lens)
+        ctx.commit(got[:, :32])
+        _, want = tapped(lambda: ctx.logits(np.full((bs, 32), shape.mask_id, dtype=np.int32)))
+        assert want[1].abs().max() > 0 and torch.equal(rows[0], want[0]) and torch.equal(rows[1], want[1])
+
+
 def test_chunk_sums_of_the_embeddings_are_the_residual_epilogue_s():
     """A layer whose output projections are zero leaves the residual stream as it was, and with it the row factors of the
     next layer: two layers with the same q, k, v matrices store the same keys and values, bit for bit."""
