@@ -73,10 +73,13 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
   const int tiles = m_tiles * n_tiles;
   const int my_tiles = pair < tiles ? (tiles - pair + n_pairs - 1) / n_pairs : 0;
   const int KC = p.k_chunks;
-  // Row tiles behind the last row in use are passed over by all three roles alike.  (The row map was written before the
-  // forward's first kernel started: readable before the dependency wait.)
+  // Row tiles behind the last row in use (of all, or of their sequence) are passed over by all three roles alike.  (The row
+  // map was written before the forward's first kernel started: readable before the dependency wait.)
   const int live_rows = p.live_rows != nullptr ? __ldcg(p.live_rows) : p.M;
-  auto tile_dead = [&](int m_t) { return m_t * 256 >= live_rows; };
+  auto tile_dead = [&](int m_t) {
+    const int row0 = m_t * 256;
+    return row0 >= live_rows || (p.live_n_valid != nullptr && row0 % p.live_rps >= __ldcg(p.live_n_valid + row0 / p.live_rps));
+  };
 
   if (threadIdx.x == 0) {
     prefetch_tensormap(&tmap_x);

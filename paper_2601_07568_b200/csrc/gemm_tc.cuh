@@ -61,6 +61,9 @@ struct GemmParams {
   // where each row belongs as (sequence, row of it), sequence -1 for the rows behind the last one in its 256-row tile
   const int* live_rows;
   const int2* row_map;
+  // or (padded prompts): sequences of live_rps rows, none of which shares a 256-row tile with another, and the rows in use of each
+  const int* live_n_valid;
+  int live_rps;
   EpiParams ep;
   // EPI_QKV only
   const float* rope_cos;  // [max_seq][64]

@@ -706,6 +706,34 @@ def test_step_statistics_after_an_early_stop_in_a_fused_forward(bs):
         assert ctx.error_word() == 0
 
 
+@pytest.mark.parametrize("d_model,lens,p_max", [(256, [300], 1024), (256, [1], 1300), (256, [0], 700), (384, [300, 0, 256], 512), (256, [1024], 1024)])
+def test_padded_prompts_pass_over_tiles_without_rows(d_model, lens, p_max):
+    """One prompt in a longer buffer, and batches of a model whose widths keep the padded layout: matmul tiles without a row
+    in use are not computed, and the stored keys and values are those of buffers that end with the prompt."""
+    shape = si.scaled_shape(si.LLADA8B, name="small-padded", n_layers=2, d_model=d_model, n_q_heads=4, n_kv_heads=4,
+                            d_ffn=640, vocab=1024, d_head=128)
+    W, bs = si.gen_weights(shape), len(lens)
+    ids = np.random.default_rng(p_max).integers(0, shape.vocab - 2, size=(bs, p_max)).astype(np.int32)
+    with Ctx(shape, W, block=32, max_batch=bs, max_seq=p_max) as ctx:
+        d3.d3_set_k_cut_pairs(ctx.ctx, 0)
+        d3.d3_set_tuning(ctx.ctx, chain=0)
+        ctx.prefill(ids, np.array(lens, dtype=np.int32))
+        got = [torch.zeros((2, 2, 4, n, 128), dtype=torch.float32, device=DEV) for n in lens]
+        for b, n in enumerate(lens):
+            for layer in range(2 if n else 0):
+                d3.d3_read_kv(ctx.ctx, layer, b, 0, n, got[b][layer, 0], got[b][layer, 1])
+        for b, n in enumerate(lens):
+            if n == 0:
+                continue
+            ctx.prefill(ids[b:b + 1, :n], np.array([n], dtype=np.int32))
+            want = torch.zeros_like(got[b])
+            for layer in range(2):
+                d3.d3_read_kv(ctx.ctx, layer, 0, 0, n, want[layer, 0], want[layer, 1])
+            # (few rows run on other tiles: the bound on two schedules of one forward)
+            assert (got[b] - want).abs().max() <= 1e-2 * want.abs().max()
+        assert ctx.error_word() == 0
+
+
 def test_tap_of_a_batch_that_stops_early():
     """A tapped layer of a batch keeps the rows of the latest forward, also where the request stops at a block's first
     step: the same rows, bit for bit, as in that step by itself."""
