@@ -313,8 +313,10 @@ int get_tmap(d3_ctx* c, const void* ptr, int rows, int cols, int box_rows, const
 // d3_generate then fuses a block's finalize forward with the next block's first denoise step.
 constexpr long long FUSE_MAX_ROWS = 64;
 // Batches, where every sequence pays the doubled rows: a fused forward instead of two where the share f of sequences at
-// a border outweighs them, f c(R) > c(2R) - c(R) with c the forward's time (8B shape, ms: c(96) 4.0, c(128) 4.1, c(192)
-// 5.0, c(256) 5.4, c(512) 10.0): half of the live sequences up to 256 fused rows, all of them up to 512.
+// a border outweighs them, f > (c(2R) - c(R)) / c(R) with c the forward's time: half of the live sequences up to 256 fused
+// rows, all of them up to 512.  Measured bounds on f, d_model 256 to 4096: 0.13-0.31 at 192 fused rows, 0.21-0.33 at 256,
+// 0.03-0.68 at 384, 0.04-0.85 at 512 (the 8B shape the largest; its forwards, ms: c(96) 4.0, c(128) 4.1, c(192) 5.0,
+// c(256) 5.4, c(512) 10.0).
 constexpr long long FUSE_HALF_ROWS = 256, FUSE_ALL_ROWS = 512;
 
 // ---- launches whose CTAs wait for one another
@@ -1509,7 +1511,11 @@ int run_stats_merge(d3_ctx* c, int M, int n_tiles, float* conf, float* ent, int*
 // decode forward of sequences with 128..400 stored positions, one kernel per matmul against this: 8B shape 4.48 -> 4.07
 // at 128 rows, 6.40 -> 5.37 at 256, 9.80 -> 8.37 at 384, 10.46 -> 10.04 at 512, 12.57 -> 12.46 at 640, but 13.31 -> 13.55 at
 // 768 and 16.77 -> 17.76 at 1024 (tiles of an incomplete wave weigh less there, and whole tiles that go through L2 more);
-// 7B shape 6.18 -> 3.63 at 128, 5.91 -> 4.95 at 256, 9.54 -> 8.42 at 512, 11.73 -> 11.41 at 640.
+// 7B shape 6.18 -> 3.63 at 128, 5.91 -> 4.95 at 256, 9.54 -> 8.42 at 512, 11.73 -> 11.41 at 640.  Layers of other widths,
+// this against one kernel per matmul (smallest and largest ratio of times at 96..640 rows): d_model 256 0.68-0.95, 768
+// 0.62-0.81 (to 192 rows), 1024 0.68-0.87, 1536 0.59-0.81, 2048 0.54-0.86, 3072 0.56-0.88.  Only a K of 512 falls out: there
+// the eight slabs that a CTA of gemm_tc_kernel gets are whole tiles and nothing is exchanged, 0.98-1.22 up to 128 rows,
+// 0.72-0.88 from 160 rows on.
 constexpr int SK_FORWARD_ROWS = 640;
 bool sk_forward_usable(const d3_ctx* c, int M) {
   const d3_config& g = c->cfg;
@@ -1520,6 +1526,7 @@ bool sk_forward_usable(const d3_ctx* c, int M) {
   if (c->tune_sk == 1) return true;
   // a schedule asked for by name is another kernel's
   if (c->tune_strip != 0 || c->tune_no_cluster || c->tune_xt == 0 || c->tune_cta_pairs == 0 || c->tune_wide_tiles >= 0 || c->tune_pair >= 0) return false;
+  if (d == 512 && M <= 128) return false;
   return M <= SK_FORWARD_ROWS;
 }
 
@@ -1605,6 +1612,9 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   // A block of up to 32 rows: with large layers the launches of resident pairs, all SMs instead of the 132 that clusters of
   // four leave, make up for attention between them.  Measured, ms per forward, chain against this: 3.46 -> 3.37 at the 8B
   // shape (436 MB a layer), 2.51 -> 2.40 at d_model 3072 (245 MB), but 1.84 -> 1.88 at 2048 (109 MB) and 1.38 -> 1.54 at 1024.
+  // (The line at 32 rows is not where the two cross: 8 layers of the 8B shape take 0.990 against 0.912 at 48 rows, 0.994 against
+  // 0.979 at 64 and 1.022 against 1.002 at two blocks of 32; at d_model 2048 1.009 against 0.913, 1.046 against 1.081 and
+  // 1.042 against 1.082, at 1024 the chain is ahead by 7-27 %.)
   const bool large_layers = static_cast<double>(nq + 2 * nkv + nq + 3.0 * f) * d * c->esz >= 200e6;
   const bool pairs_first = M <= 32 && large_layers && c->tune_chain < 0 && c->tune_chain_clusters == 0 && sk_forward_usable(c, M);
   const bool chain = !pairs_first && chain_usable(c, bs, rows_per_seq, seg);

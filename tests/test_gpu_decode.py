@@ -706,6 +706,26 @@ def test_step_statistics_after_an_early_stop_in_a_fused_forward(bs):
         assert ctx.error_word() == 0
 
 
+@pytest.mark.parametrize("d_model,bs,on_pairs", [(512, 3, False), (512, 4, False), (512, 5, True), (256, 3, True), (768, 4, True)])
+def test_decode_batches_by_width_and_rows(d_model, bs, on_pairs):
+    """Forwards of 96 to 160 rows: launches of resident pairs, except up to 128 rows where the matmuls' K of 512 makes whole
+    tiles of one kernel per matmul.  Either way the logits of the plain bf16 kernels."""
+    shape = dataclasses.replace(si.scaled_shape(si.LLADA8B, name="small-width", n_layers=2, d_model=d_model, n_q_heads=4, n_kv_heads=4,
+                                                d_ffn=640, vocab=1024, d_head=128), logit_scale=10.0)
+    W = si.gen_weights(shape)
+    ids = np.random.default_rng(d_model + bs).integers(0, shape.vocab - 2, size=(bs, 50)).astype(np.int32)
+    blk = np.full((bs, 32), shape.mask_id, dtype=np.int32)
+    lg = []
+    for impl in (0, 1):
+        with Ctx(shape, W, block=32, max_batch=bs, max_seq=96, gemm_impl=impl) as ctx:
+            ctx.prefill(ids, np.full(bs, 50, dtype=np.int32))
+            n0 = d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel")
+            lg.append(ctx.logits(blk))
+            assert (d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel") > n0) == (on_pairs and impl == 0)
+            assert ctx.error_word() == 0
+    assert np.max(np.abs(lg[0] - lg[1])) <= 3e-2 * np.max(np.abs(lg[1]))
+
+
 @pytest.mark.parametrize("d_model,lens,p_max", [(256, [300], 1024), (256, [1], 1300), (256, [0], 700), (384, [300, 0, 256], 512), (256, [1024], 1024)])
 def test_padded_prompts_pass_over_tiles_without_rows(d_model, lens, p_max):
     """One prompt in a longer buffer, and batches of a model whose widths keep the padded layout: matmul tiles without a row
