@@ -303,10 +303,15 @@ int get_tmap(d3_ctx* c, const void* ptr, int rows, int cols, int box_rows, const
                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(c, D3_ERR_CUDA, "cuTensorMapEncodeTiled failed with " + std::to_string(r));
-  if (c->tmaps.size() > 4096) c->tmaps.clear();
   auto ins = c->tmaps.emplace(key, m);
   *out = &ins.first->second;
   return D3_OK;
+}
+
+// The maps are kept for the next call on the same buffers.  They are dropped between calls only: within one, launches hold
+// pointers to several of them.
+void bound_tmaps(d3_ctx* c) {
+  if (c->tmaps.size() > 4096) c->tmaps.clear();
 }
 
 // Up to this many rows a decode forward is bound by weight streaming, so twice the rows cost the same:
@@ -1551,6 +1556,7 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   const int M = bs * rows_per_seq;
   if (M == 0) return D3_OK;
   if (M > c->ws_rows) return fail(c, D3_ERR_SHAPE, "forward over more rows than the workspaces hold");
+  bound_tmaps(c);
   const int d = g.d_model, nq = g.n_q_heads * g.d_head, nkv = g.n_kv_heads * g.d_head, f = g.d_ffn;
   RowMap rm{c->pos_base, c->n_valid, c->kv_len, rows_per_seq, bs, seg};
   c->last_rows = M;
@@ -2457,6 +2463,7 @@ extern "C" int d3_set_state(d3_ctx* c, const int32_t* prefix_len, int32_t bs) {
 extern "C" int d3_op_linear(d3_ctx* c, const void* x, const void* w, void* y, int32_t m, int32_t n, int32_t k,
                             int32_t epilogue, int32_t splits) {
   if (!c) return D3_ERR_INVALID_ARG;
+  bound_tmaps(c);
   if (!x || !w || !y || m <= 0 || n <= 0 || k <= 0 || epilogue < 0 || epilogue > 3)
     return fail(c, D3_ERR_INVALID_ARG, "bad op_linear arguments");
   if (epilogue == EPI_SWIGLU && n % 2 != 0) return fail(c, D3_ERR_SHAPE, "SwiGLU epilogue needs an even n");
@@ -2484,6 +2491,7 @@ extern "C" int d3_pack_weight(d3_ctx* c, const void* w, int32_t n, int32_t k, vo
 extern "C" int d3_op_linear_packed(d3_ctx* c, const void* x, const void* w_packed, void* y, int32_t m, int32_t n,
                                    int32_t k, int32_t epilogue, int32_t splits) {
   if (!c) return D3_ERR_INVALID_ARG;
+  bound_tmaps(c);
   if (!x || !w_packed || !y || m <= 0 || n <= 0 || k <= 0 || epilogue < 0 || epilogue > 3)
     return fail(c, D3_ERR_INVALID_ARG, "bad op_linear_packed arguments");
   if (!c->use_tc) return fail(c, D3_ERR_UNSUPPORTED, "the tiled layout is read by the tensor-core matmul only");
@@ -2497,6 +2505,7 @@ extern "C" int d3_op_linear_packed(d3_ctx* c, const void* x, const void* w_packe
 extern "C" int d3_op_lm_head_stats(d3_ctx* c, const void* x, const void* w, int32_t m, int32_t vocab, int32_t k,
                                    float scale, int32_t mask_id, float* conf, float* entropy, int32_t* argmax) {
   if (!c) return D3_ERR_INVALID_ARG;
+  bound_tmaps(c);
   if (!x || !w || !conf || !entropy || !argmax || m <= 0 || vocab <= 0 || k <= 0)
     return fail(c, D3_ERR_INVALID_ARG, "bad op_lm_head_stats arguments");
   const int n_tiles = (vocab + 127) / 128;
@@ -2511,6 +2520,7 @@ extern "C" int d3_op_lm_head_stats(d3_ctx* c, const void* x, const void* w, int3
 extern "C" int d3_op_attention(d3_ctx* c, const void* q, int32_t layer, int32_t bs, int32_t rows,
                                const int32_t* kv_len, void* out) {
   if (!c) return D3_ERR_INVALID_ARG;
+  bound_tmaps(c);
   if (!q || !out || !kv_len || layer < 0 || layer >= c->cfg.n_layers || bs <= 0 || bs > c->cfg.max_batch || rows <= 0)
     return fail(c, D3_ERR_INVALID_ARG, "bad op_attention arguments");
   // all rows live, positions irrelevant here

@@ -205,6 +205,29 @@ def test_linear_bf16_k_cut_pairs(ctx_bf16, m, n, k):
     assert ctx_bf16.error_word() == 0
 
 
+def test_tensor_maps_of_thousands_of_buffers(ctx_bf16):
+    """One operand against 4400 others at other addresses: the maps kept for earlier calls are dropped in between, never
+    under a call that uses one."""
+    rng = np.random.default_rng(11)
+    _, x = rand_bf16(rng, (160, 64))
+    xd = torch.from_numpy(x).to(torch.bfloat16).to(DEV)
+    size = d3.d3_packed_weight_elems(256, 64)
+    wt, w = rand_bf16(rng, (256, 64), 0.05)
+    one = torch.zeros(size, dtype=torch.bfloat16, device=DEV)
+    d3.d3_pack_weight(ctx_bf16.ctx, wt.to(DEV), one)
+    want, room = x @ w.T, torch.zeros(size + 8 * 4400, dtype=torch.bfloat16, device=DEV)
+    y = torch.zeros((160, 256), dtype=torch.float32, device=DEV)
+    for i in range(4400):
+        packed = room[8 * i:8 * i + size]
+        if i % 40 == 0 or i > 4050:
+            packed.copy_(one)
+            y.zero_()
+        d3.d3_op_linear_packed(ctx_bf16.ctx, xd, packed, y, 256, 0, 0)
+        if i % 40 == 0 or i > 4050:
+            assert np.max(np.abs(y.cpu().numpy() - want)) <= 2e-5 * 8 * np.abs(want).max() + 1e-6
+    assert ctx_bf16.error_word() == 0
+
+
 @pytest.mark.parametrize("m,n,k", [(512, 256, 64), (1024, 512, 512), (640, 768, 1024), (1000, 256, 4096), (2048, 4096, 1024),
                                    (513, 12288, 256), (256, 19200, 128), (130, 19200, 64)])
 def test_linear_bf16_cta_pairs(ctx_bf16, m, n, k):
