@@ -14,7 +14,7 @@ import torch
 from oracle import d3_oracle as o
 from paper_2601_07568_b200 import binding as d3
 from paper_2601_07568_b200 import synth_inputs as si
-from gpu_utils import DEV, EPS, Ctx, assert_rounding_bounded, free_running_p2, record_report, top2_gap
+from gpu_utils import DEV, EPS, ROUNDING_SHARE_MAX, Ctx, assert_rounding_bounded, free_running_p2, record_report, top2_gap
 
 pytestmark = pytest.mark.gpu
 # Largest |statistic difference| between a bf16 path and the mirrored oracle that a step-locked run may
@@ -934,41 +934,113 @@ def test_launches_that_wait_are_cooperative_between_streams():
                 assert together and torch.equal(got, want)
 
 
+def replay(ctx, ids, lens, tok, cs, tau, block, mask_id):
+    """The decisions of a d3_generate run, taken again one denoise step at a time with every block stored by a finalize
+    forward of its own.  A position may differ where the confidence is within twice the bound on the statistics' rounding
+    of the threshold, or of the best masked position's where nothing cleared it.  Returns (pairs compared, positions that
+    differ, tokens compared, tokens that differ); ctx holds the stored blocks of every sequence afterwards."""
+    bs = len(lens)
+    pairs = differ = tokens = other = 0
+    ctx.prefill(ids, lens)
+    for j in range(tok.shape[1] // block):
+        t, c = tok[:, j * block:(j + 1) * block], cs[:, j * block:(j + 1) * block]
+        for s in range(1, int(c.max()) + 1):
+            todo = (c >= s) | ((c == 0) & (t == mask_id))  # (0: never decided, in a sequence that stopped)
+            todo &= (c >= s).any(axis=1, keepdims=True)
+            r = ctx.step(np.where(todo, mask_id, t).astype(np.int32), todo, tau)
+            now, conf = todo & ~r["mask"], r["conf"]
+            was = c == s
+            for b in range(bs):
+                best = np.max(np.where(todo[b], conf[b], -1.0))
+                for q in np.flatnonzero(now[b] != was[b]):
+                    margin = abs(conf[b, q] - tau)
+                    if now[b].sum() == 1 or was[b].sum() == 1:  # a forced commit on either side
+                        margin = min(margin, best - conf[b, q])
+                    assert margin <= 2 * BF16_STAT_ERR_BOUND, (j, s, b, q, margin)
+            both = now & was
+            pairs, differ = pairs + int(todo.sum()), differ + int((now != was).sum())
+            tokens, other = tokens + int(both.sum()), other + int((r["ids"] != t)[both].sum())
+        ctx.commit(t)
+    return pairs, differ, tokens, other
+
+
+def stored_kv(ctx, layer, b, n):
+    kv = torch.zeros((2, ctx.shape.n_kv_heads, n, ctx.shape.d_head), dtype=torch.float32, device=DEV)
+    d3.d3_read_kv(ctx.ctx, layer, b, 0, n, kv[0], kv[1])
+    return kv
+
+
 @pytest.mark.parametrize("lens,tau", [([40, 7, 97], 0.0), ([40, 7, 97, 64], 0.0), ([40, 7, 97, 64], 0.3), ([33] * 6, 0.3), ([33, 5] * 4, 0.0)])
 def test_fused_finalize_of_batches(lens, tau):
     """Batches finalize a block together with the next block's first step where half of the sequences are at a border (up to
     256 fused rows) or all of them (up to 512).  At threshold 0 every step decodes a block: all sequences cross the borders
-    together and the forwards are counted; at 0.3 they drift, and borders are crossed either way.  The stored keys and
-    values of layer 0 (a function of the stored tokens alone) are those of a prefill of the same tokens."""
+    together and the forwards are counted; at 0.3 they drift, and borders are crossed either way.  Every decision, and the
+    keys and values that both layers store, against the same steps and finalize forwards one at a time."""
     shape = si.scaled_shape(si.LLADA8B, name="small-fused", n_layers=2, d_model=256, n_q_heads=4, n_kv_heads=2,
                             d_ffn=640, vocab=1024, d_head=128)
     W = si.gen_weights(shape)
     bs, gen, n_blocks = len(lens), 128, 4
     wl, ids, lens = si.small_workload("small-fused", shape, bs, lens, gen, 32, 0.9, 80)
     with Ctx(shape, W, block=32, max_batch=bs, max_seq=wl.max_seq) as ctx:
-        def stored(b, n):
-            kv = torch.zeros((2, shape.n_kv_heads, n, 128), dtype=torch.float32, device=DEV)
-            d3.d3_read_kv(ctx.ctx, 0, b, 0, n, kv[0], kv[1])
-            return kv.cpu().numpy()
         ctx.prefill(ids, lens)
         tok, cs, st = ctx.generate(bs, gen, tau)
         assert st.tokens_committed == bs * gen and st.finalize_forwards == bs * n_blocks
-        if tau == 0.0:
-            assert st.steps == n_blocks + 1 and st.denoise_forwards == bs * n_blocks
-        else:
-            assert st.steps < st.denoise_forwards + st.finalize_forwards
-        got = [stored(b, lens[b] + gen) for b in range(bs)]
-        full = np.full((bs, max(lens) + gen), shape.pad_id, dtype=np.int32)
-        for b in range(bs):
-            full[b, :lens[b] + gen] = np.concatenate([ids[b, :lens[b]], tok[b]])
-        ctx.prefill(full, np.array([n + gen for n in lens], dtype=np.int32))
-        for b in range(bs):
-            want = stored(b, lens[b] + gen)
-            assert np.max(np.abs(got[b] - want)) <= 2 ** -7 * np.max(np.abs(want))  # one bf16 rounding either side
+        got = [[stored_kv(ctx, layer, b, int(lens[b]) + gen) for layer in range(2)] for b in range(bs)]
         d3.d3_set_fused_finalize(ctx.ctx, False)
         ctx.prefill(ids, lens)
         _, _, alone = ctx.generate(bs, gen, tau)
-        assert tau != 0.0 or alone.steps == 2 * n_blocks
+        if tau == 0.0:
+            assert st.steps == n_blocks + 1 and st.denoise_forwards == bs * n_blocks and alone.steps == 2 * n_blocks
+        else:
+            assert st.steps < alone.steps
+        pairs, differ, tokens, other = replay(ctx, ids, lens, tok, cs, tau, 32, shape.mask_id)
+        record_report(f"fused_finalize_of_{bs}_at_{tau}", dict(pairs=pairs, differ=differ, tokens=tokens, other_tokens=other,
+                                                             forwards=int(st.steps), forwards_unfused=int(alone.steps)))
+        assert tokens > 0 and differ <= ROUNDING_SHARE_MAX * pairs and other <= ROUNDING_SHARE_MAX * tokens
+        for b in range(bs):
+            for layer, bound in ((0, 2 ** -7), (1, 2e-2)):  # one bf16 rounding; two schedules of a layer (a wrong key limit: 0.4)
+                want = stored_kv(ctx, layer, b, int(lens[b]) + gen)
+                assert (got[b][layer] - want).abs().max() <= bound * want.abs().max()
+        assert ctx.error_word() == 0
+
+
+def test_batch_that_stops_early_at_its_own_pace():
+    """Six sequences that drift at threshold 0.3 (blocks are finalized alone and together with first steps) and stop on an
+    end-of-sequence token: nothing is committed after the step that commits it, the unfinished block is not stored, and
+    every decision up to there, and every stored key and value, is that of the same steps one at a time."""
+    shape = si.scaled_shape(si.LLADA8B, name="small-fused", n_layers=2, d_model=256, n_q_heads=4, n_kv_heads=2,
+                            d_ffn=640, vocab=1024, d_head=128)
+    bs, gen = 6, 128
+    wl, ids, lens = si.small_workload("small-eos", shape, bs, [40, 7, 97, 64, 33, 12], gen, 32, 0.9, 80)
+    with Ctx(shape, si.gen_weights(shape), block=32, max_batch=bs, max_seq=wl.max_seq) as ctx:
+        ctx.prefill(ids, lens)
+        free, _, _ = ctx.generate(bs, gen, 0.3)
+        # the token that appears first in the second half of most responses
+        late = [t for t in np.unique(free[:, 64:]) if not (free[:, :32] == t).any()]
+        assert late
+        eos = max(late, key=lambda t: int((free == t).any(axis=1).sum()))
+        d3.d3_set_eos(ctx.ctx, int(eos))
+        ctx.prefill(ids, lens)
+        tok, cs, st = ctx.generate(bs, gen, 0.3)
+        stopped = d3.d3_early_stops(ctx.ctx)
+        assert 1 <= stopped == int((tok == eos).any(axis=1).sum())
+        prefix = ctx.get_prefix(bs)
+        for b in range(bs):
+            hit = np.flatnonzero(tok[b] == eos)
+            if len(hit) == 0:
+                assert prefix[b] == lens[b] + gen and (tok[b] != shape.mask_id).all()
+                continue
+            j, step = hit[0] // 32, cs[b, hit[0]]
+            assert (cs[b, j * 32:(j + 1) * 32] <= step).all() and (tok[b, (j + 1) * 32:] == shape.mask_id).all()
+            assert ((tok[b] == shape.mask_id) == (cs[b] == 0)).all()
+            assert prefix[b] == lens[b] + 32 * j
+        got = [stored_kv(ctx, 1, b, int(prefix[b])) for b in range(bs)]
+        d3.d3_set_eos(ctx.ctx, -1)
+        pairs, differ, tokens, other = replay(ctx, ids, lens, tok, cs, 0.3, 32, shape.mask_id)
+        assert differ <= ROUNDING_SHARE_MAX * pairs and other <= ROUNDING_SHARE_MAX * tokens
+        for b in range(bs):
+            want = stored_kv(ctx, 1, b, int(prefix[b]))
+            assert (got[b] - want).abs().max() <= 2e-2 * want.abs().max()
         assert ctx.error_word() == 0
 
 
@@ -983,12 +1055,17 @@ def test_small_bf16_batch_on_cta_pairs_step_locked():
     model = o.model_from_shape(shape, W, np.float32, mirror_bf16=True)
     exact = o.model_from_shape(shape, W, np.float32)
     with Ctx(shape, W, block=32, max_batch=6, max_seq=wl.max_seq) as ctx:
+        d3.d3_set_k_cut_pairs(ctx.ctx, 0)  # (the default for these rows is one launch for four matmuls, tested above)
+        ctx.prefill(ids, lens)
+        n0 = d3.d3_launch_count_of(ctx.ctx, "gemm_pair_kernel")
+        assert n0 > 0 and d3.d3_launch_count_of(ctx.ctx, "attn_tmem_kernel") > 0
+        ctx.step(np.full((6, 32), shape.mask_id, dtype=np.int32), np.ones((6, 32)), 0.9)
+        assert d3.d3_launch_count_of(ctx.ctx, "gemm_pair_kernel") >= n0 + 2 * shape.n_layers + 1  # QKV, gate/up; the LM head
         rep, traces = step_locked(ctx, model, ids, lens, 64, 32, 0.9, logit_tol=3e-2, exact_model=exact)
         record_report("small_bf16_step_locked_on_cta_pairs", rep)
         assert rep["max_logit_err"] <= 3e-2
         assert_rounding_bounded(rep, BF16_STAT_ERR_BOUND)
-        assert d3.d3_launch_count_of(ctx.ctx, "gemm_pair_kernel") > 0
-        assert d3.d3_launch_count_of(ctx.ctx, "attn_tmem_kernel") > 0
+        assert d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel") == 0
         ctx.prefill(ids, lens)
         tok, cs, st = ctx.generate(6, 64, 0.9)
         assert st.tokens_committed == 6 * 64
@@ -1194,11 +1271,15 @@ def test_chain_launch_small_models(hq, hkv, bs, plens):
         n0 = d3.d3_launch_count_of(ctx.ctx, "chain_kernel")
         got = ctx.logits(blk)
         assert d3.d3_launch_count_of(ctx.ctx, "chain_kernel") == n0 + 1  # one launch for all layers
+        n_sk = d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel")
         d3.d3_set_tuning(ctx.ctx, chain=0)
+        d3.d3_set_k_cut_pairs(ctx.ctx, 0)
         ctx.prefill(ids, lens)
         base = ctx.logits(blk)
         assert d3.d3_launch_count_of(ctx.ctx, "chain_kernel") == n0 + 1
+        assert d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel") == n_sk
         d3.d3_set_tuning(ctx.ctx)
+        d3.d3_set_k_cut_pairs(ctx.ctx, -1)
         for b in range(bs):
             assert np.max(np.abs(got[b] - base[b])) <= 1e-2 * np.max(np.abs(base[b]))
         rep, _ = step_locked(ctx, model, ids, lens, 64, 32, 0.9, logit_tol=3e-2, exact_model=exact)
