@@ -83,7 +83,6 @@ struct ChainParams {
   int l2_ahead;            // weight slabs the L2 prefetch thread runs ahead of the weight thread (0: no prefetch)
   unsigned int* sync;      // [operators of the program] border counters, zero before the forward's first launch
   uint32_t* error_word;
-  const int* skip_flag;
   // EPI_QKV and CHAIN_ATTN
   const float* rope_cos;
   const float* rope_sin;
@@ -421,7 +420,6 @@ inline size_t chain_smem_bytes(int a_rows, uint32_t w_stage_bytes, int stages, s
 __global__ void __launch_bounds__(CHAIN_THREADS, 1)
 chain_kernel(const __grid_constant__ CUtensorMap tmap_x0, const __grid_constant__ CUtensorMap tmap_x1,
              const __grid_constant__ CUtensorMap tmap_x2, const __grid_constant__ CUtensorMap tmap_kv, const ChainParams p) {
-  if (p.skip_flag != nullptr && *p.skip_flag != 0) return;
   grid_dep_launch();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));

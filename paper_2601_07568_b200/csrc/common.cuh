@@ -55,7 +55,7 @@ struct EpiParams {
 };
 
 // Row factor of a matmul whose operand rows were left un-normalised; chunk sums added in index
-// order (the same bits whichever thread or kernel asks).
+// order (the same bits in every kernel that asks here; gemm_sk_kernel adds them as a tree over a warp's lanes).
 __device__ __forceinline__ float row_rstd(const EpiParams& ep, int m) {
   const float* r = ep.ssq_in + static_cast<size_t>(m) * ep.ssq_chunks;
   float tot = 0.f;

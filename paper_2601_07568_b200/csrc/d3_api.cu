@@ -97,7 +97,6 @@ struct d3_ctx {
   // per-class kernel timing (off by default)
   bool prof_on = false;
   bool pdl = true;           // programmatic dependent launch between the kernels of a forward
-  int* skip_flag = nullptr;  // device flag: non-zero turns the forward's kernels into no-ops
   int tune_producers = 0;
   int tune_attn_div = 0;  // experiment: key tiles per attention split
   int tune_pair = -1;     // -1: by row count; 0 / 1: one / two row tiles per matmul unit
@@ -480,7 +479,6 @@ int run_linear_tc_bn(d3_ctx* c, const void* X, const void* W, int M, int N, int 
   p.partial = c->partial;
   p.tile_count = c->tile_count;
   p.error_word = c->error_word;
-  p.skip_flag = c->skip_flag;
   p.w_tiled = w_tiled;
   p.n_producers = c->tune_producers > 0 ? c->tune_producers : 2;
   p.ep = ep;
@@ -586,7 +584,6 @@ int run_linear_ck(d3_ctx* c, const void* X, const void* W, int M, int N, int K, 
   p.total_units = static_cast<long long>(T) * KC;
   p.stages = stages;
   p.error_word = c->error_word;
-  p.skip_flag = c->skip_flag;
   p.w_tiled = w_tiled;
   p.n_producers = 2;
   p.ep = ep;
@@ -678,7 +675,6 @@ int run_linear_xt(d3_ctx* c, const void* X, const void* W, int M, int N, int K, 
   p.k_chunks = (K + 63) / 64;
   p.stages = stages;
   p.error_word = c->error_word;
-  p.skip_flag = c->skip_flag;
   p.w_tiled = 1;
   p.w_packed = static_cast<const bf16*>(W);
   p.w_blocks = static_cast<long long>(N / 128) * p.k_chunks;
@@ -756,7 +752,6 @@ int run_linear_strip(d3_ctx* c, const void* X, const void* W, int M, int N, int 
       return fail(c, D3_ERR_UNSUPPORTED, "strip_stages outside 2..min(32, K slabs) or beyond 200 KB of shared memory");
   }
   p.error_word = c->error_word;
-  p.skip_flag = c->skip_flag;
   p.w_tiled = 1;
   p.w_packed = static_cast<const bf16*>(W);
   p.w_blocks = static_cast<long long>((N + 127) / 128) * KC;
@@ -937,7 +932,6 @@ int run_chain(d3_ctx* c, int op_begin, int op_end, const RowMap& rm) {
   p.stages = plan.stages;
   p.sync = c->chain_sync;
   p.error_word = c->error_word;
-  p.skip_flag = c->skip_flag;
   p.rope_cos = c->rope_cos; p.rope_sin = c->rope_sin;
   p.rm = rm;
   p.n_q_heads = g.n_q_heads; p.n_kv_heads = g.n_kv_heads; p.max_seq = g.max_seq;
@@ -1023,7 +1017,6 @@ int run_linear_pair(d3_ctx* c, const void* X, const void* W, int M, int N, int K
   p.k_chunks = K / 64;
   p.m_tiles = (M + 255) / 256; p.n_tiles = N / 256;
   p.error_word = c->error_word;
-  p.skip_flag = c->skip_flag;
   p.w_tiled = 1;
   if ((reinterpret_cast<uintptr_t>(W) & 15) != 0) return fail(c, D3_ERR_UNSUPPORTED, "tiled weights must be 16-byte aligned");
   p.w_packed = static_cast<const bf16*>(W);
@@ -1113,7 +1106,6 @@ int run_sk(d3_ctx* c, const SkMatmul* mm, int n, int M) {
   if (static_cast<size_t>(P) * 6 * p.tok_n * 128 > c->partial_slots * 128 * 128) return fail(c, D3_ERR_SHAPE, "partial tiles exceed the workspace");
   p.partial = c->partial;
   p.error_word = c->error_word;
-  p.skip_flag = c->skip_flag;
   p.rope_cos = c->rope_cos; p.rope_sin = c->rope_sin;
   p.n_q_heads = c->cfg.n_q_heads; p.n_kv_heads = c->cfg.n_kv_heads; p.max_seq = c->cfg.max_seq;
   p.rows_per_seq = 1;
@@ -2643,7 +2635,6 @@ extern "C" int d3_debug_stall_probe(d3_ctx* c, int32_t limit_us) {
   p.partial = c->partial;
   p.tile_count = c->tile_count;
   p.error_word = c->error_word;
-  p.skip_flag = nullptr;
   p.wait_limit_us = static_cast<uint32_t>(limit_us);
   p.stall = 1;
   p.n_producers = 1;

@@ -55,7 +55,6 @@ inline size_t gemm_pair_smem_bytes() { return 1024 + PAIR_STAGES * PAIR_STAGE_BY
 template <int EPI>
 __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_x,
                                                                     const __grid_constant__ CUtensorMap tmap_w, const GemmParams p) {
-  if (p.skip_flag != nullptr && *p.skip_flag != 0) return;  // uniform over the grid
   grid_dep_launch();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));

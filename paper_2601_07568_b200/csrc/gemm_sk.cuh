@@ -69,7 +69,6 @@ struct SkParams {
   float* partial;         // [pairs][3: first cut tile, second, whole tile][2 CTAs][tok_n][128] fp32
   unsigned int* border;   // [n_ops] CTAs that have finished the matmul, zero before the launch
   uint32_t* error_word;
-  const int* skip_flag;
   const float* rope_cos;  // [max_seq][64]
   const float* rope_sin;
   const int* pos_base;
@@ -197,7 +196,8 @@ __device__ __forceinline__ void sk_lane_sums16(float (&a)[16], int lane) {
   a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
 }
 // Row factors of the folded RMSNorm for rows m0 .. m0 + 15 into rs[0 .. 15] (rows from M on: whatever): a row's chunk
-// sums over a warp's lanes, all rows' loads in flight at once.
+// sums over a warp's lanes, all rows' loads in flight at once.  (A tree of 32-bit sums where row_rstd has a chain: the last
+// bits differ from the other kernels', as those of the K-cut sums do.)
 __device__ __forceinline__ void sk_row_rstd16(const EpiParams& ep, int m0, int M, int lane, float* rs) {
   float a[16];
   const int chunks = ep.ssq_chunks;  // a multiple of 4
@@ -434,9 +434,8 @@ __device__ __forceinline__ void sk_finish(const SkParams& p, const SkOp& o, cons
 }
 
 // grid = 2 x pairs (all resident at once), cluster (2, 1, 1).  Dynamic shared memory (1024-byte aligned inside the
-// kernel): [stages] weight blocks, [stages] rows of X, barriers, two sets of row tables.
+// kernel): [stages] weight blocks, [stages] rows of X, barriers, row table, row factors, plans.
 __global__ void __launch_bounds__(SK_THREADS, 1) gemm_sk_kernel(const __grid_constant__ SkParams p) {
-  if (p.skip_flag != nullptr && *p.skip_flag != 0) return;  // uniform over the grid
   grid_dep_launch();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));

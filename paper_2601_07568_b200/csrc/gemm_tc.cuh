@@ -47,7 +47,6 @@ struct GemmParams {
   float* partial;   // partial tiles [2 * grid][row tiles per unit][BLOCK_N][128] fp32: slot 2i = CTA i's first segment, 2i+1 = its last
   int* tile_count;  // arrival counters [tiles], zero on entry and on exit
   uint32_t* error_word;
-  const int* skip_flag;  // optional: non-zero -> the whole launch is a no-op
   uint32_t wait_limit_us;  // unit-range kernel: limit of every wait in microseconds (0: the default of ptx::mbar_wait)
   int stall;               // unit-range kernel, give-up path probe: the producers issue no loads at all
   int n_producers;       // 1 or 2 TMA-issuing warps
@@ -436,7 +435,6 @@ template <int EPI, int BLOCK_N, int MT>
 __global__ void __launch_bounds__(NUM_THREADS, 2)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                const GemmParams p) {
-  if (p.skip_flag != nullptr && *p.skip_flag != 0) return;  // written at least one whole graph launch earlier
   grid_dep_launch();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -784,7 +782,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 2)
 gemm_ck_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w,
                const GemmParams p, const ClusterSplit cs) {
   constexpr int BLOCK_N = 128;
-  if (p.skip_flag != nullptr && *p.skip_flag != 0) return;
   grid_dep_launch();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -1123,7 +1120,6 @@ struct TmemPairSource {
 template <int EPI, int TCOLS>
 __global__ void __launch_bounds__(STRIP_THREADS, 2)
 gemm_strip_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams p, const int S) {
-  if (p.skip_flag != nullptr && *p.skip_flag != 0) return;
   grid_dep_launch();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));

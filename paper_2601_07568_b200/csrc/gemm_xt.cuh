@@ -51,7 +51,6 @@ inline size_t gemm_xt_smem_bytes(int n_cols, int stages) {
 template <int EPI>
 __global__ void __launch_bounds__(XT_THREADS, 1)
 gemm_xt_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams p, const XtSplit xs) {
-  if (p.skip_flag != nullptr && *p.skip_flag != 0) return;
   grid_dep_launch();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
