@@ -274,6 +274,37 @@ def gemm_flops(shape, M):
             "gemm_down": 2 * M * d * f, "gemm_head": 2 * M * V * d}
 
 
+def profiled_request(ctx, w, ids_dev, lens_dev, out_dev, mode):
+    """One request with an event pair around every launch of the decode loop (mode 1: every matmul a launch of its own; 2: the
+    launches that the loop makes).  Returns (classes, stats, rows of all its forwards)."""
+    import torch
+    from paper_2601_07568_b200 import binding as d3
+    d3.d3_prefill(ctx, ids_dev, lens_dev)
+    torch.cuda.synchronize()
+    rows0 = d3.d3_launch_count_of(ctx, "forward_rows")
+    d3.d3_profile_enable(ctx, mode)
+    st = d3.d3_generate(ctx, w.gen_len, w.threshold, out_dev)
+    prof = d3.d3_profile_read(ctx)
+    d3.d3_profile_enable(ctx, 0)
+    return prof, st, d3.d3_launch_count_of(ctx, "forward_rows") - rows0
+
+
+def matmul_totals(shape, prof, forwards, rows, fused_rows):
+    """Matmul launches of a profiled request, those inside chain launches left out: (ms, launches, bytes, flops).  Forwards
+    that ran as a chain, where not all did, are those with `fused_rows` rows."""
+    layer_keys = ("gemm_qkv", "gemm_o", "gemm_gate_up", "gemm_down")
+    keys = layer_keys + ("gemm_head", "gemm_other")
+    chained = min(prof["chain"]["launches"], forwards)
+    own = forwards - chained
+    rows_chained = rows if own == 0 else chained * fused_rows
+    tot_bytes = tot_flops = 0
+    for n, m, layers in ((own, (rows - rows_chained) / max(own, 1), shape.n_layers), (chained, rows_chained / max(chained, 1), 0)):
+        gb, gf = gemm_bytes(shape, m), gemm_flops(shape, m)
+        tot_bytes += n * (layers * sum(gb[k] for k in layer_keys) + gb["gemm_head"])
+        tot_flops += n * (layers * sum(gf[k] for k in layer_keys) + gf["gemm_head"])
+    return sum(prof[k]["ms"] for k in keys), sum(prof[k]["launches"] for k in keys), tot_bytes, tot_flops
+
+
 def measure_batched(name, W, dev, local, world, dist, peaks, steps):
     """The batched companion workload (same model, batch 32): decoded tokens/s resident and end to end,
     ms per forward, and the tensor roofline of its matmul launches (flops / CUDA-event time / sustained peak)."""
@@ -326,20 +357,12 @@ def measure_batched(name, W, dev, local, world, dist, peaks, steps):
     ms_e2e, _ = timed(step_e2e, steps)
     ms_prefill, _ = timed(lambda: d3.d3_prefill(ctx, ids_dev, lens_dev), 3)
     ms_prefill /= 3
-    d3.d3_prefill(ctx, ids_dev, lens_dev)
-    torch.cuda.synchronize()
-    d3.d3_profile_enable(ctx, True)
-    d3.d3_generate(ctx, w.gen_len, w.threshold, out_dev)
-    prof = d3.d3_profile_read(ctx)
-    d3.d3_profile_enable(ctx, False)
+    prof, st_prof, rows = profiled_request(ctx, w, ids_dev, lens_dev, out_dev, 2)
     err_word = d3.d3_get_error_word(ctx)
     d3.d3_destroy(ctx)
     tokens = w.batch * w.gen_len
-    M = w.batch * w.block
-    gf = gemm_flops(shape, M)
-    tot_flops = sum(gf[k] * prof[k]["launches"] for k in gf)
-    tot_ms = sum(prof[k]["ms"] for k in gf)
-    n_gemm = sum(prof[k]["launches"] for k in gf)
+    gf = gemm_flops(shape, rows / max(st_prof.steps, 1))
+    tot_ms, n_gemm, _, tot_flops = matmul_totals(shape, prof, st_prof.steps, rows, 2 * w.batch * w.block)
     ms_step = ms_total / steps
     ms_fwd = (ms_step - ms_prefill) / max(st.steps, 1)
     layer_keys = ("gemm_qkv", "gemm_o", "gemm_gate_up", "gemm_down")
@@ -354,7 +377,7 @@ def measure_batched(name, W, dev, local, world, dist, peaks, steps):
                    "ms_per_forward": ms_fwd, "prefill_ms": ms_prefill},
         "roofline": {"bound": "tensor", "achieved": achieved, "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                      "frac": achieved / peaks["bf16_tflops_sustained"], "traffic": None,
-                     "kernel": "gemm_pair_kernel (all matmul launches of the decode loop, LM head included; CUDA events around every launch, launched serialized)",
+                     "kernel": "gemm_pair_kernel (all matmul launches of the decode loop as it makes them, LM head included; CUDA events around every launch, which keep it from overlapping the next)",
                      "peak_source": f"of {peaks['source']} (sustained)", "launches": n_gemm, "avg_launch_us": 1e3 * tot_ms / max(n_gemm, 1),
                      "flops_per_launch": tot_flops / max(n_gemm, 1),
                      "step_effective": {"TFLOP/s": fwd_flops / (ms_fwd / 1e3) / 1e12,
@@ -509,13 +532,9 @@ def run_ours(args):
                                      "GB/s": 3 * nb * nn * 4 / (ms_ns * 1e-3) / 1e9}}
     del y_big, rank_big, noisy
 
-    # per-class kernel times of the decode loop (one request, events around every launch)
-    d3.d3_prefill(ctx, ids_dev, lens_dev)
-    torch.cuda.synchronize()
-    d3.d3_profile_enable(ctx, True)
-    st_prof = d3.d3_generate(ctx, w.gen_len, w.threshold, out_dev)
-    prof = d3.d3_profile_read(ctx)
-    d3.d3_profile_enable(ctx, False)
+    # kernel times of the decode loop, events around every launch: as it makes them, and with every matmul by itself
+    prof, st_prof, prof_rows = profiled_request(ctx, w, ids_dev, lens_dev, out_dev, 2)
+    split, st_split, split_rows = profiled_request(ctx, w, ids_dev, lens_dev, out_dev, 1)
     # prefill alone
     ms_prefill, _ = timed(lambda: d3.d3_prefill(ctx, ids_dev, lens_dev), 3)
     ms_prefill /= 3
@@ -526,28 +545,25 @@ def run_ours(args):
     ms_step = ms_total / args.steps
 
     peaks = measured_peaks()
-    M = w.batch * w.block
-    gb = gemm_bytes(shape, M)
-    gf = gemm_flops(shape, M)
+    gb, gf = (fn(shape, prof_rows / max(st_prof.steps, 1)) for fn in (gemm_bytes, gemm_flops))  # of a forward with the mean rows
     layer_keys = ("gemm_qkv", "gemm_o", "gemm_gate_up", "gemm_down")
     # K/V read by the attention of one forward at mid-generation
     kv_mid = 2 * shape.n_layers * shape.n_kv_heads * shape.d_head * 2 * sum(int(l) + w.gen_len // 2 for l in lens_np)
-    chain = prof.get("chain", {"ms": 0.0, "launches": 0})
-    if chain["ms"] > sum(prof[k]["ms"] for k in gb):
-        # the decode forward's layers run as one launch (chain_kernel): matmuls of all layers and attention
+    tot_ms, n_dom, tot_bytes, tot_flops = matmul_totals(shape, prof, st_prof.steps, prof_rows, 2 * w.batch * w.block)
+    chain = prof["chain"]
+    if chain["ms"] > tot_ms:
+        # most decode forwards run their layers as one launch (chain_kernel): matmuls of all layers and attention
         dominant = "chain_kernel (all layers of a decode forward: QKV, attention, O-proj, gate/up, down)"
-        per_launch_bytes = sum(gb[k] for k in layer_keys) * shape.n_layers + kv_mid
-        per_launch_flops = sum(gf[k] for k in layer_keys) * shape.n_layers
-        tot_bytes, tot_flops = per_launch_bytes * chain["launches"], per_launch_flops * chain["launches"]
+        m = prof_rows / st_prof.steps if chain["launches"] >= st_prof.steps else 2 * w.batch * w.block
+        bm, fm = gemm_bytes(shape, m), gemm_flops(shape, m)
+        tot_bytes = (sum(bm[k] for k in layer_keys) * shape.n_layers + kv_mid) * chain["launches"]
+        tot_flops = sum(fm[k] for k in layer_keys) * shape.n_layers * chain["launches"]
         tot_ms, n_dom = chain["ms"], chain["launches"]
         traffic_kernel = "chain_kernel"
     else:
-        dominant = "gemm_sk_kernel, gemm_pair_kernel, gemm_strip_kernel, gemm_ck_kernel, gemm_xt_kernel, gemm_tc_kernel (all matmul launches of the decode loop)"
-        tot_bytes = sum(gb[k] * prof[k]["launches"] for k in gb)
-        tot_flops = sum(gf[k] * prof[k]["launches"] for k in gf)
-        tot_ms = sum(prof[k]["ms"] for k in gb)
-        n_dom = sum(prof[k]["launches"] for k in gb)
-        traffic_kernel = "matmul kernels"
+        dominant = ("gemm_sk_kernel (O-proj, gate/up, down and the next layer's QKV or the LM head in a launch) and the other matmul launches of "
+                    "the decode loop as it makes them; CUDA events around every launch, which keep it from overlapping the next")
+        traffic_kernel = "gemm_sk_kernel"
     hbm_bound = tot_flops / max(tot_bytes, 1) < peaks["bf16_tflops_sustained"] * 1e12 / (peaks["hbm_gbs"] * 1e9)
     if hbm_bound:
         achieved = tot_bytes / (tot_ms / 1e3) / 1e9 if tot_ms > 0 else 0.0
@@ -569,20 +585,23 @@ def run_ours(args):
                                   "ms_per_forward": ms_fwd, "bytes_per_forward": fwd_bytes}
     cap = ncu_traffic(traffic_kernel, w.name) if hbm_bound else None
     if cap is not None and n_dom > 0:
-        # the capture ran the model cut to a few layers: traffic grows in proportion to the layers of a launch
-        roofline["traffic"] = float(cap["bytes_per_layer"]) * shape.n_layers + float(cap.get("bytes_fixed", 0.0))
+        # the capture ran the model cut to a few layers: a forward's traffic and launches grow in proportion to them; per launch
+        per_forward = float(cap["bytes_per_layer"]) * shape.n_layers + float(cap.get("bytes_fixed", 0.0))
+        roofline["traffic"] = per_forward / (float(cap.get("launches_per_layer", 0)) * shape.n_layers + float(cap.get("launches_fixed", 1)))
         roofline["traffic_source"] = cap.get("source", "ncu")
     roofline.update({"kernel": dominant, "peak_source": f"of {peaks['source']}",
                      "launches": n_dom, "avg_launch_us": 1e3 * tot_ms / max(n_dom, 1),
                      "algorithmic_bytes_per_launch": tot_bytes / max(n_dom, 1)})
-    per_class = {}
-    for k, v in prof.items():
+    # (the split schedule: what a matmul takes by itself, not what the decode loop runs)
+    per_class = {"schedule": "every matmul a launch of its own"}
+    gbs, gfs = (fn(shape, split_rows / max(st_split.steps, 1)) for fn in (gemm_bytes, gemm_flops))
+    for k, v in split.items():
         if v["launches"] == 0:
             continue
         e = {"ms": round(v["ms"], 3), "launches": v["launches"], "us_per_launch": round(1e3 * v["ms"] / v["launches"], 2)}
-        if k in gb and v["ms"] > 0:
-            e["GB/s"] = round(gb[k] * v["launches"] / (v["ms"] / 1e3) / 1e9, 1)
-            e["TFLOP/s"] = round(gf[k] * v["launches"] / (v["ms"] / 1e3) / 1e12, 1)
+        if k in gbs and v["ms"] > 0:
+            e["GB/s"] = round(gbs[k] * v["launches"] / (v["ms"] / 1e3) / 1e9, 1)
+            e["TFLOP/s"] = round(gfs[k] * v["launches"] / (v["ms"] / 1e3) / 1e12, 1)
         per_class[k] = e
     forwards = st.steps
     line = {

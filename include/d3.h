@@ -354,7 +354,9 @@ int d3_set_overlap(d3_ctx *ctx, int on);
  * bracketed by a CUDA event pair on the context's stream; d3_profile_read waits for the stream and
  * returns, per class, the summed elapsed milliseconds and the number of launches since enabling.
  * ms, launches: [host] arrays of D3_PROF_CLASSES entries.  Off by default (it costs two event
- * records per launch). */
+ * records per launch).  on = 1: every matmul is a launch of its own, timed under its class, also where a
+ * forward would run several in one launch; on = 2: the launches that forwards make, those of several
+ * matmuls under D3_PROF_GEMM_OTHER. */
 enum { D3_PROF_GEMM_QKV = 0, D3_PROF_GEMM_O = 1, D3_PROF_GEMM_GATE_UP = 2, D3_PROF_GEMM_DOWN = 3,
        D3_PROF_GEMM_HEAD = 4, D3_PROF_GEMM_OTHER = 5, D3_PROF_ATTENTION = 6, D3_PROF_RMSNORM = 7,
        D3_PROF_OTHER = 8, D3_PROF_CHAIN = 9 /* a decode forward's layers as one launch */, D3_PROF_CLASSES = 10 };
@@ -369,7 +371,7 @@ int d3_get_error_word(d3_ctx *ctx, uint32_t *word);
 /* Number of this library's kernels launched on the context since creation. */
 int64_t d3_launch_count(d3_ctx *ctx);
 /* The same for one kernel, by its name in the source (e.g. "gemm_strip_kernel"); 0 for unknown names.  "cooperative": the
- * cooperative launches among all of them. */
+ * cooperative launches among all of them; "forward_rows": rows of all forwards so far. */
 int64_t d3_launch_count_of(d3_ctx *ctx, const char *kernel);
 /* Bytes of device memory the context holds. */
 int64_t d3_device_bytes(d3_ctx *ctx);

@@ -398,8 +398,9 @@ def d3_status_of_error_word(word: int) -> int:
     return int(lib().d3_status_of_error_word(C.c_uint32(word)))
 
 
-def d3_profile_enable(ctx, on: bool) -> None:
-    _check(ctx, lib().d3_profile_enable(ctx, C.c_int(1 if on else 0)))
+def d3_profile_enable(ctx, on: int) -> None:
+    """on: False / 0 off, True / 1 every matmul as a launch of its own, 2 the launches that forwards make."""
+    _check(ctx, lib().d3_profile_enable(ctx, C.c_int(int(on))))
 
 
 def d3_profile_read(ctx) -> Dict[str, Dict[str, float]]:

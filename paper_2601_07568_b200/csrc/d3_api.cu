@@ -96,6 +96,7 @@ struct d3_ctx {
   int64_t dev_bytes = 0;
   // per-class kernel timing (off by default)
   bool prof_on = false;
+  bool prof_split = false;   // every matmul a launch of its own while timing is on
   bool pdl = true;           // programmatic dependent launch between the kernels of a forward
   int tune_producers = 0;
   int tune_attn_div = 0;  // experiment: key tiles per attention split
@@ -1552,6 +1553,7 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   const int d = g.d_model, nq = g.n_q_heads * g.d_head, nkv = g.n_kv_heads * g.d_head, f = g.d_ffn;
   RowMap rm{c->pos_base, c->n_valid, c->kv_len, rows_per_seq, bs, seg};
   c->last_rows = M;
+  c->launches_by_kernel["forward_rows"] += M;
   // Prompts of different lengths: their rows are laid out one after the other, and the matmuls, which know the padded
   // count only, stop at the last row in use.
   const bool packed = ragged && pack_usable(c, bs, M);
@@ -1648,9 +1650,11 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
       qx = QkvExtra{rm, k_plane(c, l), v_plane(c, l)};
       return SkMatmul{c->xb, c->wqkv[l], nq + 2 * nkv, d, EPI_QKV, ep, &qx};
     };
-    // (while classes are timed every matmul is a launch of its own)
     auto launch = [&](const SkMatmul* mm, const int* cls, int n) {
-      if (!c->prof_on) return run_sk(c, mm, n, M);
+      if (!c->prof_on || !c->prof_split) {
+        ProfScope ps(c, n > 1 ? static_cast<int>(D3_PROF_GEMM_OTHER) : cls[0]);
+        return run_sk(c, mm, n, M);
+      }
       for (int j = 0; j < n; ++j) {
         ProfScope ps(c, cls[j]);
         TRY(run_sk(c, mm + j, 1, M));
@@ -2677,6 +2681,7 @@ extern "C" int d3_profile_enable(d3_ctx* c, int on) {
     }
   }
   c->prof_on = on != 0;
+  c->prof_split = on != 2;
   return D3_OK;
 }
 extern "C" int d3_profile_read(d3_ctx* c, double* ms, int64_t* launches) {

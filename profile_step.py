@@ -36,7 +36,8 @@ def main() -> int:
     ap.add_argument("--steps", type=int, default=3)
     ap.add_argument("--warmup", type=int, default=1)
     ap.add_argument("--prefix", type=int, default=0, help="override the cached prefix length (0 = after prefill)")
-    ap.add_argument("--no-chain", action="store_true", help="one kernel per matmul instead of the chain launch")
+    ap.add_argument("--no-chain", action="store_true", help="launches of resident CTA pairs instead of the chain launch")
+    ap.add_argument("--per-kernel", action="store_true", help="one kernel per matmul instead of either")
     args = ap.parse_args()
 
     d3build.build()
@@ -54,8 +55,10 @@ def main() -> int:
     del W
     ids_np, lens_np = si.gen_prompts(w)
     d3.d3_prefill(ctx, torch.from_numpy(ids_np).to(dev), torch.from_numpy(lens_np).to(dev))
-    if args.no_chain:
+    if args.no_chain or args.per_kernel:
         d3.d3_set_tuning(ctx, chain=0)
+    if args.per_kernel:
+        d3.d3_set_k_cut_pairs(ctx, 0)
     if args.prefix > 0:
         d3.d3_set_state(ctx, torch.full((w.batch,), args.prefix, dtype=torch.int32, device=dev))
     bs, B = w.batch, w.block

@@ -147,3 +147,29 @@ def test_column_strips_refuse_an_odd_pipeline_depth():
         with pytest.raises(d3.D3Error):
             d3.d3_set_tuning(ctx.ctx, strip_stages=33)
         assert ctx.error_word() == 0
+
+
+def test_profile_modes_time_split_and_real_launches():
+    """Mode 1 times every matmul of a batch's forward as a launch of its own, mode 2 the launches that the forward makes
+    (four matmuls each, under the class of several); statistics are the same bits in both and without timing."""
+    shape = si.scaled_shape(si.LLADA8B, name="profile-modes", n_layers=3, d_model=256, n_q_heads=4, n_kv_heads=2,
+                            d_ffn=640, vocab=1024, d_head=128)
+    ids = np.random.default_rng(9).integers(0, shape.vocab - 2, size=(3, 20)).astype(np.int32)
+    blk, mask = np.full((3, 32), shape.mask_id, dtype=np.int32), np.ones((3, 32))
+    with Ctx(shape, si.gen_weights(shape), block=32, max_batch=3, max_seq=64) as ctx:
+        ctx.prefill(ids, np.array([20, 4, 11], dtype=np.int32))
+        got = []
+        for mode, want in ((0, {}), (1, dict(gemm_qkv=3, gemm_o=3, gemm_gate_up=3, gemm_down=3, gemm_head=1, attention=3)),
+                           (2, dict(gemm_qkv=1, gemm_other=3, attention=3))):
+            rows0 = d3.d3_launch_count_of(ctx.ctx, "forward_rows")
+            d3.d3_profile_enable(ctx.ctx, mode)
+            got.append(ctx.step(blk, mask, 0.9))
+            prof = d3.d3_profile_read(ctx.ctx)
+            d3.d3_profile_enable(ctx.ctx, 0)
+            assert d3.d3_launch_count_of(ctx.ctx, "forward_rows") == rows0 + 96
+            if mode:
+                assert {k: v["launches"] for k, v in prof.items() if v["launches"] and k != "other"} == want
+                assert all(prof[k]["ms"] > 0 for k in want)
+        for r in got[1:]:
+            assert np.array_equal(r["conf"], got[0]["conf"]) and np.array_equal(r["ent"], got[0]["ent"])
+        assert ctx.error_word() == 0
