@@ -93,6 +93,7 @@ struct d3_ctx {
   int last_rows = 0;
   int64_t launches = 0;
   std::map<std::string, int64_t> launches_by_kernel;  // the same, per kernel name
+  int64_t forward_rows = 0;  // of all forwards so far
   int64_t dev_bytes = 0;
   // per-class kernel timing (off by default)
   bool prof_on = false;
@@ -1553,7 +1554,7 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   const int d = g.d_model, nq = g.n_q_heads * g.d_head, nkv = g.n_kv_heads * g.d_head, f = g.d_ffn;
   RowMap rm{c->pos_base, c->n_valid, c->kv_len, rows_per_seq, bs, seg};
   c->last_rows = M;
-  c->launches_by_kernel["forward_rows"] += M;
+  c->forward_rows += M;
   // Prompts of different lengths: their rows are laid out one after the other, and the matmuls, which know the padded
   // count only, stop at the last row in use.
   const bool packed = ragged && pack_usable(c, bs, M);
@@ -2696,6 +2697,7 @@ extern "C" int d3_profile_read(d3_ctx* c, double* ms, int64_t* launches) {
 extern "C" int64_t d3_launch_count(d3_ctx* c) { return c ? c->launches : 0; }
 extern "C" int64_t d3_launch_count_of(d3_ctx* c, const char* kernel) {
   if (!c || !kernel) return 0;
+  if (std::strcmp(kernel, "forward_rows") == 0) return c->forward_rows;
   auto it = c->launches_by_kernel.find(kernel);
   return it == c->launches_by_kernel.end() ? 0 : it->second;
 }

@@ -472,7 +472,7 @@ struct GenState {
   long long* counters;  // [0] denoise fwd, [1] finalize fwd, [2] tokens, [3] forced, [4] seqs not done, [5] seqs in SEQ_FUSED,
                         // [6] sequences stopped early on the end-of-sequence id, [7] sequences waiting for a KV-refresh
   int* hist;            // [bs, max_seq] ids of the stored prefix (prompt and stored blocks)
-  int* stat_row;        // [bs] where the statistics of the latest forward's decision begin
+  int* stat_row;        // [bs] where the statistics of the latest fused forward's decision begin
   int* refresh_flag;    // [bs] 1: the stored prefix of this sequence is to be recomputed before the next forward
   unsigned long long* commit_hist;  // [COMMIT_HIST_BINS] decisions that committed k tokens (k = bin index)
   uint32_t* error_word;
@@ -507,7 +507,7 @@ __global__ void gen_advance_kernel(GenState g, const float* __restrict__ conf, c
   const int b = blockIdx.x;
   const int lane = threadIdx.x & 31;
   const int mode = g.mode[b];
-  if (lane == 0) g.stat_row[b] = b * R + (mode == SEQ_FUSED && R > B ? B : 0);
+  if (lane == 0 && R > B) g.stat_row[b] = b * R + (mode == SEQ_FUSED ? B : 0);
   if (mode == SEQ_DONE) return;
   int* ids = g.ids + b * B;
   uint8_t* mask = g.mask + b * B;
