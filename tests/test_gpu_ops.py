@@ -141,7 +141,7 @@ def test_linear_bf16_weights_as_rows(ctx_bf16, m, n, k, cluster):
     assert ctx_bf16.error_word() == 0
 
 
-@pytest.mark.parametrize("m,n,k", [(1, 16, 4), (16, 128, 512), (17, 130, 260), (33, 384, 128), (48, 200, 1028), (5, 514, 64)])
+@pytest.mark.parametrize("m,n,k", [(1, 16, 4), (16, 128, 512), (17, 130, 260), (33, 384, 128), (48, 200, 1028), (5, 514, 64), (3, 96, 256), (9, 48, 292)])
 @pytest.mark.parametrize("epi", [0, 2, 3])
 def test_linear_fp32_small_tiles_same_bits(ctx_f32, m, n, k, epi):
     """fp32 matmuls of few tiles run on 16 x 16 tiles: against the fp64 product, and bit for bit what a matmul of many
