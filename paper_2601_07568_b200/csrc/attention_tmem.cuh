@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) attn_tmem_stream_kernel(const _
           ptx::mbar_arrive_expect_tx(&q_full[qb], static_cast<uint32_t>(R) * 256u);
           for (int hg = 0; hg < group; ++hg)
             for (int h = 0; h < 2; ++h)
-              ptx::tma_load_2d(qd + h * q_slab + hg * rps * 128, &tmap_q, &q_full[qb], (g * group + hg) * 128 + h * 64, b * rps);
+              ptx::tma_load_2d(qd + h * q_slab + hg * rps * 128, &tmap_q, &q_full[qb], (g * group + hg) * 128 + h * 64, static_cast<int>(first_row(p.rm, b)));
         }
         return true;
       };
@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) attn_tmem_stream_kernel(const _
         ptx::tc_fence_before();  // the next pair's first P (and with it the product that overwrites O) comes after this
         if (row_ok) {
           const float inv = 1.0f / l_run;
-          __nv_bfloat16* o = p.out + (static_cast<size_t>(b) * rps + r_seq) * p.hq * 128 + (g * group + hg) * 128;
+          __nv_bfloat16* o = p.out + (first_row(p.rm, b) + r_seq) * p.hq * 128 + (g * group + hg) * 128;
 #pragma unroll
           for (int d = 0; d < 128; d += 8)
             *reinterpret_cast<uint4*>(o + d) =

@@ -1419,9 +1419,10 @@ int run_attention_tc(d3_ctx* c, const void* q, int layer, void* out, const RowMa
   // is the faster one (measured: 60-70 against 84-110 us per layer at 64 rows x 4200-5100 keys, 27 against 33-37 at
   // 224 rows x 550-1000 keys, a third of the time on 4096-row prompts); at 32 rows the two are level on batches and
   // the mma.sync kernel, with its cheaper start, is ahead on a single sequence (15 against 19 us).
-  // (the persistent form finds its query rows by a tensor map over equal sequences)
-  if (c->tune_attn_shape == 2 && rm.row_off == nullptr ? attn_stream_usable(c, rm)
-                              : (rm.row_off == nullptr && c->tune_attn_tmem < 0 && attn_stream_usable(c, rm) && rm.bs * g.n_kv_heads >= 2 * c->n_sms))
+  // (Where rows of different sequences lie one after the other, the box of rows_per_seq query rows that the persistent form
+  // loads for a sequence ends in the next one's: rows that no thread owns.)
+  if (c->tune_attn_shape == 2 ? attn_stream_usable(c, rm)
+                              : (c->tune_attn_tmem < 0 && attn_stream_usable(c, rm) && rm.bs * g.n_kv_heads >= 2 * c->n_sms))
     return run_attention_tmem_stream(c, q, layer, out, rm);
   // (the mma.sync kernel has one key limit for 16 rows: segments that are not multiples of 16 rows are never its business)
   if (c->tune_attn_tmem == 1 || (c->tune_attn_tmem < 0 && R >= 64) || rm.seg % 16 != 0) return run_attention_tmem(c, q, layer, out, rm);

@@ -783,6 +783,28 @@ def test_tap_of_a_batch_that_stops_early():
         assert want[1].abs().max() > 0 and torch.equal(rows[0], want[0]) and torch.equal(rows[1], want[1])
 
 
+@pytest.mark.parametrize("hkv,lens", [(8, [24, 1, 17, 0, 23, 8, 24, 9] * 5), (8, [24] * 40), (16, [61, 64, 3, 0, 33] * 4), (4, [8 * (i % 5) + 1 for i in range(75)])])
+def test_many_short_prompts_on_the_persistent_attention(hkv, lens):
+    """Prompt batches with many (sequence, kv head) pairs and few rows each take the persistent attention kernel, whose
+    query rows lie one after the other like all others: bit for bit the keys and values of the padded layout."""
+    shape = si.scaled_shape(si.LLADA8B, name="small-short", n_layers=2, d_model=256, n_q_heads=hkv, n_kv_heads=hkv,
+                            d_ffn=640, vocab=1024, d_head=128)
+    bs, p_max = len(lens), (max(lens) + 7) // 8 * 8
+    assert bs * p_max > 640 and bs * hkv >= 300
+    ids = np.random.default_rng(bs).integers(0, shape.vocab - 2, size=(bs, p_max)).astype(np.int32)
+    with Ctx(shape, si.gen_weights(shape), block=8, max_batch=bs, max_seq=p_max + 8) as ctx:
+        got = []
+        for tap in (-1, 0):  # (a tapped context keeps the padded layout)
+            d3.d3_set_tap(ctx.ctx, tap)
+            n0 = [d3.d3_launch_count_of(ctx.ctx, k) for k in ("pack_rows_kernel", "attn_tmem_stream_kernel")]
+            ctx.prefill(ids, np.array(lens, dtype=np.int32))
+            n = [d3.d3_launch_count_of(ctx.ctx, k) - m for k, m in zip(("pack_rows_kernel", "attn_tmem_stream_kernel"), n0)]
+            assert n == [1 if tap < 0 else 0, 2]
+            got.append([stored_kv(ctx, layer, b, k) for b, k in enumerate(lens) if k for layer in range(2)])
+        assert all(torch.equal(a, b) for a, b in zip(*got))
+        assert ctx.error_word() == 0
+
+
 def test_chunk_sums_of_the_embeddings_are_the_residual_epilogue_s():
     """A layer whose output projections are zero leaves the residual stream as it was, and with it the row factors of the
     next layer: two layers with the same q, k, v matrices store the same keys and values, bit for bit."""
