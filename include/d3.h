@@ -150,10 +150,12 @@ int d3_commit_block(d3_ctx *ctx, const int32_t *block_ids, int32_t bs);
  * [device][bs, gen_len]: 1-based step within its block at which each position was committed;
  * host_stats [host] may be NULL.  Waits for the stream.  Errors: SHAPE when gen_len is not a
  * multiple of B or prefix + gen_len > max_seq; INVALID_ARG when a prefix is negative.
- * While 2 * bs * B <= 64 rows (and the context was created with 2 * max_batch * B <= 64), the finalize
- * forward of a block and the first denoise step of the next block run as one forward of 2B rows per
- * sequence, the finished block unable to see the new one: same results as separate forwards (bit for
- * bit on the fp32 path), one batched forward less per block. */
+ * The finalize forward of a block and the first denoise step of the next block may run as one forward of 2B rows per
+ * sequence, the finished block unable to see the new one: same results as separate forwards up to the order of sums (bit
+ * for bit on the fp32 path), one batched forward less per block.  Without a refresh period (d3_set_cache_policy) this is
+ * done while 2 * bs * B <= 64 rows (and 2 * max_batch * B <= 64); on the bfloat16 tensor-core path also in batches, while
+ * no layer is tapped, of up to 512 such rows: up to 256 when at least half of the live sequences are at a border,
+ * beyond when all are.  d3_create makes room for it (2 * max_batch * B rows, at most 512). */
 int d3_generate(d3_ctx *ctx, int32_t gen_len, float threshold, int32_t bs, int32_t *out_ids,
                 int32_t *commit_step, d3_stats *host_stats);
 
