@@ -61,7 +61,7 @@ int d3_set_tuning(d3_ctx *ctx, const d3_tuning *t);
 int d3_set_fused_finalize(d3_ctx *ctx, int on);
 
 /* Matmuls of decode-sized forwards on resident CTA pairs, the tiles of an incomplete wave cut along K (gemm_sk_kernel, up
- * to 1024 rows): mode -1 = by row count (default), 0 never, 1 wherever the shape allows, every cut that gives each pair
+ * to 1024 rows): mode -1 = by rows and widths (default), 0 never, 1 wherever the shape allows, every cut that gives each pair
  * work included, and for d3_op_linear_packed.  INVALID_ARG for other values. */
 int d3_set_k_cut_pairs(d3_ctx *ctx, int32_t mode);
 

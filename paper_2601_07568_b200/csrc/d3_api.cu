@@ -90,7 +90,6 @@ struct d3_ctx {
   int tap_layer = -1;
   float *tap_in = nullptr, *tap_out = nullptr;
   int tap_rows = 0;
-  int last_rows = 0;
   int64_t launches = 0;
   std::map<std::string, int64_t> launches_by_kernel;  // the same, per kernel name
   int64_t forward_rows = 0;  // of all forwards so far
@@ -1554,7 +1553,6 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   bound_tmaps(c);
   const int d = g.d_model, nq = g.n_q_heads * g.d_head, nkv = g.n_kv_heads * g.d_head, f = g.d_ffn;
   RowMap rm{c->pos_base, c->n_valid, c->kv_len, rows_per_seq, bs, seg};
-  c->last_rows = M;
   c->forward_rows += M;
   // Prompts of different lengths: their rows are laid out one after the other, and the matmuls, which know the padded
   // count only, stop at the last row in use.

@@ -338,32 +338,6 @@ __global__ void __launch_bounds__(MERGE_THREADS) stats_merge_sample_kernel(const
   }
 }
 
-// Statistics straight from fp32 logits rows (SIMT path and tests): one block per row.
-__global__ void stats_from_logits_kernel(const float* __restrict__ logits, int V, int mask_id, float4* __restrict__ part,
-                                         int n_tiles) {
-  // one warp per (row, 128-column tile); lanes stride the tile, then a fixed shuffle tree
-  const int m = blockIdx.y;
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (t >= n_tiles) return;
-  const float* row = logits + static_cast<size_t>(m) * V;
-  SoftStat st = stat_empty();
-  for (int j = lane; j < 128; j += 32) {
-    int n = t * 128 + j;
-    if (n < V && n != mask_id) stat_add(st, row[n], n);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    SoftStat other;
-    other.m = __shfl_xor_sync(0xffffffffu, st.m, o);
-    other.z = __shfl_xor_sync(0xffffffffu, st.z, o);
-    other.s = __shfl_xor_sync(0xffffffffu, st.s, o);
-    other.a = __shfl_xor_sync(0xffffffffu, st.a, o);
-    st = (lane & o) ? stat_merge(other, st) : stat_merge(st, other);
-  }
-  if (lane == 0) part[static_cast<size_t>(m) * n_tiles + t] = make_float4(st.m, st.z, st.s, __int_as_float(st.a));
-}
-
 // ----------------------------------------------------------------------------- decision
 // One warp per sequence.  Commits every masked position clearing the threshold and always the most
 // confident masked one (lowest index on ties); writes ids, clears mask bytes, emits (pos, id) in
@@ -1071,12 +1045,7 @@ __global__ void cast_from_f32_kernel(const float* __restrict__ src, T* __restric
   if (i < n) dst[i] = TypeOps<T>::from_f(src[i]);
 }
 
-// Weight repacking on the device: dst rows [r0, r0+rows) <- src rows; and gate/up interleave.
-template <typename T>
-__global__ void copy_rows_kernel(const T* __restrict__ src, T* __restrict__ dst, size_t n) {
-  size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = src[i];
-}
+// Weight repacking on the device: gate/up interleave.
 // dst [2f, d]: row 2j = gate row j, row 2j+1 = up row j.
 template <typename T>
 __global__ void interleave_gate_up_kernel(const T* __restrict__ gate, const T* __restrict__ up, T* __restrict__ dst,
