@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(TM_THREADS, KT == 64 ? 2 : 1) attn_tmem_kernel
   // Producer and MMA thread walk the tiles in the same order: K_0 .. K_(SBUF-1), then V_j, K_(j+SBUF) for every j.
   if (warp_id == 4) {
     // ------------------------------------------------------------------ producer
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       const long long krow = p.k_row0 + (static_cast<long long>(b) * p.hkv + g) * p.max_seq;
       const long long vrow = p.v_row0 + (static_cast<long long>(b) * p.hkv + g) * p.max_seq;
       bool waited = false, ok = true;
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(TM_THREADS, KT == 64 ? 2 : 1) attn_tmem_kernel
     }
   } else if (warp_id == 5) {
     // ------------------------------------------------------------------ MMA issue
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       constexpr uint32_t idesc_qk = tm_idesc(128, KT, false);
       constexpr uint32_t idesc_pv = tm_idesc(128, 128, true);
       bool ok = ptx::mbar_wait(q_full, 0, abort_flag, p.error_word);
@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) attn_tmem_stream_kernel(const _
   // Producer and MMA thread walk the stream in the same order: K(0), K(1), then V(g), K(g + 2) for every tile g.
   if (warp_id == 4) {
     // ------------------------------------------------------------------ producer
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       bool waited = false, ok = true;
       int s = 0;  // position in the ring
       auto load = [&](bool is_k, const TmCursor& c) {
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(TM_THREADS, 1) attn_tmem_stream_kernel(const _
     }
   } else if (warp_id == 5) {
     // ------------------------------------------------------------------ MMA issue
-    if (lane == 0) {
+    if (ptx::elect_one()) {
       constexpr uint32_t idesc_qk = tm_idesc(128, KT, false);
       constexpr uint32_t idesc_pv = tm_idesc(128, 128, true);
       bool ok = true;

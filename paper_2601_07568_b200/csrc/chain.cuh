@@ -497,7 +497,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmap_x0, const __grid_constant_
 
   if (warp == 0) {
     // ---------------- weights: never waits for data, only for ring space
-    if (lane == 0) {
+    if (elect_one()) {
       int s = 0, n_req = 0;
       uint32_t ph = 1;  // parity to wait for on the empty barrier (first lap: passes at once)
       bool ok = true;
@@ -595,7 +595,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmap_x0, const __grid_constant_
     }
   } else if (warp == 6) {
     // ---------------- activations: behind the border of each matmul
-    if (lane == 0) {
+    if (elect_one()) {
       int s = 0;
       uint32_t ph = 1;
       int tile_it = 0;  // attention tiles requested so far
@@ -640,7 +640,7 @@ chain_kernel(const __grid_constant__ CUtensorMap tmap_x0, const __grid_constant_
     }
   } else if (warp == 1) {
     // ---------------- MMA issue
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t adesc0 = make_smem_desc(smem_u32(smem_a)), bdesc0 = make_smem_desc(smem_u32(smem_b));
       const uint64_t a_step = a_stage_bytes >> 4, b_step = b_stage_bytes >> 4;
       int s = 0;

@@ -105,9 +105,11 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer
-    if (lane == 0) {
+    if (elect_one()) {
       grid_dep_wait();  // X comes from the kernel before this one
-      int it = 0;
+      const uint32_t lead_full = map_to_cta(smem_u32(full_bar), 0);
+      int s = 0;
+      uint32_t ph = 1;  // parity to wait for on the empty barrier (first lap: passes at once)
       bool ok = true;
       for (int t = 0; t < my_tiles && ok; ++t) {
         const int q = pair + t * n_pairs;
@@ -116,26 +118,23 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
         if (tile_dead(m_t)) continue;
         const int row0 = m_t * 256 + static_cast<int>(rank) * 128;
         const int wrow0 = (n_t * 2 + static_cast<int>(rank)) * KC * 128;  // first row of this CTA's first weight block
-        for (int kc = 0; kc < KC; ++kc, ++it) {
-          const int s = it % PAIR_STAGES;
-          if (it >= PAIR_STAGES && !mbar_wait(&empty_bar[s], static_cast<uint32_t>(it / PAIR_STAGES - 1) & 1u, abort_flag, p.error_word)) {
-            ok = false;
-            break;
-          }
+        for (int kc = 0; kc < KC; ++kc) {
+          if (!mbar_wait(&empty_bar[s], ph, abort_flag, p.error_word)) { ok = false; break; }
           uint8_t* st = smem + s * PAIR_STAGE_BYTES;
           if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 2 * PAIR_STAGE_BYTES);
-          const uint32_t lead_full = map_to_cta(smem_u32(&full_bar[s]), 0);
-          tma_load_2d_pair(st, &tmap_x, lead_full, kc * 64, row0);
-          tma_load_2d_pair(st + PAIR_A_BYTES, &tmap_w, lead_full, 0, wrow0 + kc * 128);
+          tma_load_2d_pair(st, &tmap_x, lead_full + 8u * s, kc * 64, row0);
+          tma_load_2d_pair(st + PAIR_A_BYTES, &tmap_w, lead_full + 8u * s, 0, wrow0 + kc * 128);
+          if (++s == PAIR_STAGES) { s = 0; ph ^= 1u; }
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       if (rank == 0) {
         // -------------------------------------------------------------- MMA issue (leader)
-        const uint32_t sb = smem_u32(smem);
-        int it = 0;
+        const uint64_t adesc0 = make_smem_desc(smem_u32(smem)), bdesc0 = make_smem_desc(smem_u32(smem + PAIR_A_BYTES));
+        int s = 0;
+        uint32_t ph = 0;
         bool ok = true;
         int n_done = 0;  // tiles computed so far: accumulator buffer and barrier phases
         for (int t = 0; t < my_tiles && ok; ++t) {
@@ -147,19 +146,17 @@ __global__ void __launch_bounds__(PAIR_THREADS, 1) gemm_pair_kernel(const __grid
           if (!ok) break;
           tc_fence_after();
           const uint32_t tmem_d = tmem_base + static_cast<uint32_t>(buf * 256);
-          for (int kc = 0; kc < KC; ++kc, ++it) {
-            const int s = it % PAIR_STAGES;
-            const uint32_t ph = static_cast<uint32_t>(it / PAIR_STAGES) & 1u;
+          for (int kc = 0; kc < KC; ++kc) {
             ok = mbar_wait_cluster(&full_bar[s], ph, abort_flag, p.error_word);
             if (!ok) break;
             tc_fence_after();
-            const uint64_t adesc = make_smem_desc(sb + s * PAIR_STAGE_BYTES);
-            const uint64_t bdesc = make_smem_desc(sb + s * PAIR_STAGE_BYTES + PAIR_A_BYTES);
+            const uint64_t adesc = adesc0 + static_cast<uint64_t>(s) * (PAIR_STAGE_BYTES >> 4), bdesc = bdesc0 + static_cast<uint64_t>(s) * (PAIR_STAGE_BYTES >> 4);
 #pragma unroll
             for (int kk = 0; kk < BLOCK_K / UMMA_K; ++kk)
               umma_bf16_pair(tmem_d, adesc + static_cast<uint64_t>(2 * kk), bdesc + static_cast<uint64_t>(2 * kk), PAIR_IDESC,
                              (kc > 0 || kk > 0) ? 1u : 0u);
             umma_commit_pair(&empty_bar[s], 3);
+            if (++s == PAIR_STAGES) { s = 0; ph ^= 1u; }
           }
           if (ok) umma_commit_pair(&acc_full[buf], 3);
           ++n_done;

@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_sk_kernel(const __grid_con
 
   if (warp == 0) {
     // ------------------------------------------------------------------ weights: held back by ring space only
-    if (lane == 0) {
+    if (elect_one()) {
       // weights that are read once leave L2 first: partials and activations stay
       const uint64_t stream_policy = l2_evict_first_policy();
       const bool once = p.tok_tiles == 1;
@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_sk_kernel(const __grid_con
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------------ rows of X: behind the border of each matmul
-    if (lane == 0) {
+    if (elect_one()) {
       int s = 0;
       uint32_t ph = 1;
       bool ok = true;
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1) gemm_sk_kernel(const __grid_con
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issue (leader)
-    if (lane == 0 && rank == 0) {
+    if (rank == 0 && elect_one()) {
       const uint32_t idesc = make_idesc(256, p.tok_n);
       const uint64_t adesc0 = make_smem_desc(smem_u32(smem_w)), bdesc0 = make_smem_desc(smem_u32(smem_x));
       const uint64_t a_step = SK_W_BYTES >> 4, b_step = x_bytes >> 4;

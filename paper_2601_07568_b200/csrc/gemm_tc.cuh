@@ -511,7 +511,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
   if (warp == 0 || warp == 6) {
     // ---------------- TMA producers: warp 0 alone, or warps 0 and 6 taking alternate units
     const int n_prod = p.n_producers, pi = warp == 0 ? 0 : 1;
-    if (lane == 0 && pi < n_prod && !p.stall) {
+    const bool one = elect_one();
+    if (one && pi < n_prod && !p.stall) {
       const uint32_t tx = a_stage_bytes + b_stage_bytes;
       const long long n_total = u1 - u0;
       // Arms the stage's barrier with the bytes that will arrive and issues the weight loads.
@@ -578,12 +579,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
         s += n_prod;
         if (s >= stages) { s -= stages; ph ^= 1u; }
       }
-    } else if (lane == 0) {
+    } else if (one) {
       grid_dep_wait();
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = make_idesc(BLOCK_M, BLOCK_N);
       const uint64_t adesc0 = make_smem_desc(smem_u32(smem_a)), bdesc0 = make_smem_desc(smem_u32(smem_b));
       const uint64_t a_step = a_stage_bytes >> 4, b_step = b_stage_bytes >> 4;  // stage strides in descriptor units
@@ -845,7 +846,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
   if (warp == 0 || warp == 6) {
     // ---------------- TMA producers: alternate units
     const int pi = warp == 0 ? 0 : 1;
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t tx = a_stage_bytes + b_stage_bytes;
       // unit i of this CTA = (tile t0 + i / n_k, slab kc0 + i % n_k), kept as running counters (no
       // division per slab: these single-thread loops pace the CTA)
@@ -891,7 +892,7 @@ gemm_ck_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer: one accumulator per tile, alternating TMEM halves
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = make_idesc(BLOCK_M, BLOCK_N);
       const uint64_t adesc0 = make_smem_desc(smem_u32(smem_a)), bdesc0 = make_smem_desc(smem_u32(smem_b));
       const uint64_t a_step = a_stage_bytes >> 4, b_step = b_stage_bytes >> 4;
@@ -1170,7 +1171,7 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams p
   const int pipe = (warp == 0 || warp == 1) ? 0 : 1;
   if ((warp == 0 || warp == 6) && pipe < n_pipe) {
     // ---------------- producer of pipeline `pipe`: slabs pipe, pipe + n_pipe, ...
-    if (lane == 0) {
+    if (elect_one()) {
       // the strip's rows inside the 128-row blocks it touches: up to three runs of whole 8-row groups
       const __nv_bfloat16* piece_src[3];
       uint32_t piece_bytes[3], piece_dst[3];
@@ -1228,7 +1229,7 @@ gemm_strip_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams p
     }
   } else if ((warp == 1 || warp == 7) && pipe < n_pipe) {
     // ---------------- MMA issuer of pipeline `pipe`
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = make_idesc(BLOCK_M, S);
       const uint64_t adesc0 = make_smem_desc(smem_u32(smem_a)), bdesc0 = make_smem_desc(smem_u32(smem_b));
       const uint64_t a_step = a_stage_bytes >> 4, b_step = b_stage_bytes >> 4;  // stage strides in descriptor units

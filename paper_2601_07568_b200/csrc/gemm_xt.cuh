@@ -98,7 +98,7 @@ gemm_xt_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams p, c
 
   if (warp == 0) {
     // ---------------- requests: weights of the first ring lap before the dependency wait, activations after it
-    if (lane == 0) {
+    if (elect_one()) {
       const __nv_bfloat16* wsrc = p.w_packed + (static_cast<long long>(tile) * KC + kc0) * (128 * 64);
       const uint32_t tx = w_stage_bytes + x_stage_bytes;
       const int pre = n_k < stages ? n_k : stages;
@@ -121,7 +121,7 @@ gemm_xt_kernel(const __grid_constant__ CUtensorMap tmap_x, const GemmParams p, c
     }
   } else if (warp == 1) {
     // ---------------- MMA issue: A = weights (128 rows), B = activations (n_cols rows)
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = make_idesc(128, xs.n_cols);
       const uint64_t adesc0 = make_smem_desc(smem_u32(smem_w)), bdesc0 = make_smem_desc(smem_u32(smem_x));
       const uint64_t a_step = w_stage_bytes >> 4, b_step = x_stage_bytes >> 4;

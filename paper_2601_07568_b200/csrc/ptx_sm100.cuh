@@ -13,6 +13,21 @@ constexpr uint64_t WAIT_LIMIT_NS = 4000000000ull;  // every spin gives up after 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
+// One thread of a converged warp, for the roles that a single thread plays (bulk loads, MMAs and their commits).  Told by
+// this instruction the compiler knows that exactly one thread goes on; behind `lane == 0` it has to provide for operands
+// that differ between threads around every MMA, which took the issuing thread about 600 clocks per 64-wide K slab, more
+// than the four pair MMAs of a slab (512 at 256 rows) and more than its weights take to arrive.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "elect.sync _|p, 0xffffffff;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(r));
+  return r != 0;
+}
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
