@@ -726,6 +726,29 @@ def test_decode_batches_by_width_and_rows(d_model, bs, on_pairs):
     assert np.max(np.abs(lg[0] - lg[1])) <= 3e-2 * np.max(np.abs(lg[1]))
 
 
+@pytest.mark.parametrize("d_model,d_ffn,bs", [(256, 9728, 3), (1024, 10880, 3), (1024, 10880, 1), (1024, 10880, 9), (256, 9728, 6)])
+def test_whole_gate_up_tiles_of_resident_pairs(d_model, d_ffn, bs):
+    """Gate/up of more 256-row tiles than pairs: 76 (none cut, some pairs have two) and 85 (74 whole ones behind the exchange
+    of 11 cut ones), at 32, 96, 192 and 288 rows (two tiles of 160 rows of X, the last 32 of them without any).  The logits
+    of the plain bf16 kernels."""
+    shape = dataclasses.replace(si.scaled_shape(si.LLADA8B, name="small-wide-ffn", n_layers=2, d_model=d_model, n_q_heads=2, n_kv_heads=2,
+                                                d_ffn=d_ffn, vocab=1024, d_head=128), logit_scale=10.0)
+    W = si.gen_weights(shape)
+    ids = np.random.default_rng(d_ffn + bs).integers(0, shape.vocab - 2, size=(bs, 50)).astype(np.int32)
+    blk = np.full((bs, 32), shape.mask_id, dtype=np.int32)
+    lg = []
+    for impl in (0, 1):
+        with Ctx(shape, W, block=32, max_batch=bs, max_seq=96, gemm_impl=impl) as ctx:
+            ctx.prefill(ids, np.full(bs, 50, dtype=np.int32))
+            if impl == 0:
+                d3.d3_set_tuning(ctx.ctx, chain=0)
+            n0 = d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel")
+            lg.append(ctx.logits(blk))
+            assert (d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel") > n0) == (impl == 0)
+            assert ctx.error_word() == 0
+    assert np.max(np.abs(lg[0] - lg[1])) <= 3e-2 * np.max(np.abs(lg[1]))  # two schedules of one forward, as above
+
+
 @pytest.mark.parametrize("d_model,lens,p_max", [(256, [300], 1024), (256, [1], 1300), (256, [0], 700), (384, [300, 0, 256], 512), (256, [1024], 1024)])
 def test_padded_prompts_pass_over_tiles_without_rows(d_model, lens, p_max):
     """One prompt in a longer buffer, and batches of a model whose widths keep the padded layout: matmul tiles without a row
