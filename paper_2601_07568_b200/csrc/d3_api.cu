@@ -2321,7 +2321,7 @@ extern "C" int d3_trajectory_rank(d3_ctx* c, const int32_t* commit_step, int32_t
   if (gen_len % c->cfg.block != 0) return fail(c, D3_ERR_SHAPE, "gen_len not a multiple of the block size");
   const int B = c->cfg.block;
   if (B >= 4 && B <= 128 && (B & (B - 1)) == 0 && aligned16(commit_step) && aligned16(rank)) {
-    trajectory_rank4_kernel<<<(bs + 7) / 8, 256, 0, c->stream>>>(commit_step, bs, gen_len, B, rank);
+    CUDA_TRY(c, launch_pdl(c, trajectory_rank4_kernel, dim3((bs + 7) / 8), dim3(256), 0, commit_step, bs, gen_len, B, rank));
     LAUNCHED(c, "trajectory_rank4_kernel");
     return D3_OK;
   }
@@ -2336,8 +2336,8 @@ extern "C" int d3_noisy_sequence(d3_ctx* c, const int32_t* y, const int32_t* ran
   if (bs > 65535) return fail(c, D3_ERR_SHAPE, "more than 65535 sequences in one call");
   if (n % 4 == 0 && aligned16(y) && aligned16(rank) && aligned16(out)) {
     const long long quads = static_cast<long long>(bs) * (n / 4);
-    noisy_sequence4_kernel<<<static_cast<unsigned>((quads + 255) / 256), 256, 0, c->stream>>>(
-        reinterpret_cast<const int4*>(y), reinterpret_cast<const int4*>(rank), s, k, m, bs, n / 4, c->cfg.mask_id, reinterpret_cast<int4*>(out));
+    CUDA_TRY(c, launch_pdl(c, noisy_sequence4_kernel, dim3(static_cast<unsigned>((quads + 255) / 256)), dim3(256), 0, reinterpret_cast<const int4*>(y), reinterpret_cast<const int4*>(rank),
+                           s, k, m, bs, n / 4, c->cfg.mask_id, reinterpret_cast<int4*>(out)));
     LAUNCHED(c, "noisy_sequence4_kernel");
     return D3_OK;
   }

@@ -910,6 +910,8 @@ __global__ void trajectory_rank_kernel(const int* __restrict__ commit_step, int 
 // to 128, 16-byte aligned rows.  Bound by memory (8 bytes a position); a warp per 32-thread block that waits for every
 // decoding block's load in turn takes 22 us for 16384 x 256 positions, this one 8.
 __global__ void __launch_bounds__(256) trajectory_rank4_kernel(const int* __restrict__ commit_step, int bs, int gen_len, int B, int* __restrict__ rank) {
+  ptx::grid_dep_wait();  // (dependent launches, here and below: the gap between two kernels of 6 us each is a fifth of the pair)
+  ptx::grid_dep_launch();
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (b >= bs) return;  // warp-uniform
   const int4* cs = reinterpret_cast<const int4*>(commit_step + static_cast<size_t>(b) * gen_len);
@@ -968,6 +970,8 @@ __global__ void noisy_sequence_kernel(const int* __restrict__ y, const int* __re
 __global__ void __launch_bounds__(256) noisy_sequence4_kernel(const int4* __restrict__ y, const int4* __restrict__ rank, const int* __restrict__ s_arr,
                                                               const int* __restrict__ k_arr, const int* __restrict__ m_arr, int bs, int n4, int mask_id,
                                                               int4* __restrict__ out) {
+  ptx::grid_dep_wait();
+  ptx::grid_dep_launch();
   const long long at = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (at >= static_cast<long long>(bs) * n4) return;
   const int b = static_cast<int>(at / n4), i = 4 * static_cast<int>(at - static_cast<long long>(b) * n4) + 1;  // first position
