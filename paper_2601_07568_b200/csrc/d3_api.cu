@@ -1609,14 +1609,14 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
     after_norm(ep);
     return ep;
   };
-  // A block of up to 32 rows: with large layers the launches of resident pairs, all SMs instead of the 132 that clusters of
-  // four leave, make up for attention between them.  Measured, ms per forward, chain against this: 3.46 -> 3.37 at the 8B
-  // shape (436 MB a layer), 2.51 -> 2.40 at d_model 3072 (245 MB), but 1.84 -> 1.88 at 2048 (109 MB) and 1.38 -> 1.54 at 1024.
-  // (The line at 32 rows is not where the two cross: 8 layers of the 8B shape take 0.990 against 0.912 at 48 rows, 0.994 against
-  // 0.979 at 64 and 1.022 against 1.002 at two blocks of 32; at d_model 2048 1.009 against 0.913, 1.046 against 1.081 and
-  // 1.042 against 1.082, at 1024 the chain is ahead by 7-27 %.)
+  // Forwards of up to 64 rows (the chain takes no more): with large layers the launches of resident pairs, all SMs instead of the
+  // 132 that clusters of four leave, make up for attention between them.  Measured, ms per 32-row forward, chain against this:
+  // 3.46 -> 3.37 at the 8B shape (436 MB a layer), 2.51 -> 2.40 at d_model 3072 (245 MB), but 1.84 -> 1.88 at 2048 (109 MB) and
+  // 1.38 -> 1.54 at 1024.  33 to 64 rows at the 8B shape: a request whose finished blocks share their forward with the next
+  // block's first step 116.9 -> 116.0, one with windows of 64 and 128 rows 66.0 -> 63.8; at d_model 2048 48 rows gain 10 % and 64
+  // rows lose 3, at 1024 the chain is ahead by 7-27 %.
   const bool large_layers = static_cast<double>(nq + 2 * nkv + nq + 3.0 * f) * d * c->esz >= 200e6;
-  const bool pairs_first = M <= 32 && large_layers && c->tune_chain < 0 && c->tune_chain_clusters == 0 && sk_forward_usable(c, M);
+  const bool pairs_first = M <= 64 && large_layers && c->tune_chain < 0 && c->tune_chain_clusters == 0 && sk_forward_usable(c, M);
   const bool chain = !pairs_first && chain_usable(c, bs, rows_per_seq, seg);
   // The LM head is the last matmul of the last layer's launch.  (Behind the chain it stays a launch of its own on 128-row tiles,
   // whose weights are on their way while the chain drains: 3.79 ms a 64-row forward against 3.83.)
