@@ -57,30 +57,37 @@ __global__ void __launch_bounds__(THREADS) attn_simt_kernel(const T* __restrict_
       Vs[j][d] = in ? TypeOps<T>::to_f(vb[static_cast<size_t>(j0 + j) * DH + d]) : 0.f;
     }
     __syncthreads();
+    // A warp's rows side by side and the keys unrolled (the sums of a row in the same order as one row and one key at a time):
+    // what bounds it is the chain of dependent instructions.  (Rows that do not exist are computed and not written.)
+    float sc[RPW], pr[RPW];
+#pragma unroll
+    for (int i = 0; i < RPW; ++i) sc[i] = 0.f;
+#pragma unroll 8
+    for (int d = 0; d < DH; ++d)
+#pragma unroll
+      for (int i = 0; i < RPW; ++i) sc[i] = fmaf(Qs[warp * RPW + i][d], Ks[lane][d], sc[i]);
 #pragma unroll
     for (int i = 0; i < RPW; ++i) {
-      const int r = warp * RPW + i;
-      if (r0 + r >= n_valid) continue;  // warp-uniform
-      float s = 0.f;
-#pragma unroll 8
-      for (int d = 0; d < DH; ++d) s = fmaf(Qs[r][d], Ks[lane][d], s);
-      if (j0 + lane >= row_kv_limit(rm, b, r0 + r, kv_len)) s = -INFINITY;  // keys of later segments stay unseen
-      float mx = s;
+      if (j0 + lane >= row_kv_limit(rm, b, r0 + warp * RPW + i, kv_len)) sc[i] = -INFINITY;  // keys of later segments stay unseen
+      float mx = sc[i];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       const float m_new = fmaxf(m_run[i], mx);
-      const float p = __expf(s - m_new);  // -inf -> 0
+      pr[i] = __expf(sc[i] - m_new);  // -inf -> 0
       const float corr = __expf(m_run[i] - m_new);
-      l_run[i] = l_run[i] * corr + warp_sum(p);
+      l_run[i] = l_run[i] * corr + warp_sum(pr[i]);
       m_run[i] = m_new;
 #pragma unroll
       for (int d = 0; d < DPL; ++d) acc[i][d] *= corr;
-      for (int j = 0; j < KC; ++j) {
-        const float pj = __shfl_sync(0xffffffffu, p, j);
+    }
+#pragma unroll 16
+    for (int j = 0; j < KC; ++j)
+#pragma unroll
+      for (int i = 0; i < RPW; ++i) {
+        const float pj = __shfl_sync(0xffffffffu, pr[i], j);
 #pragma unroll
         for (int d = 0; d < DPL; ++d) acc[i][d] = fmaf(pj, Vs[j][lane + 32 * d], acc[i][d]);
       }
-    }
   }
 #pragma unroll
   for (int i = 0; i < RPW; ++i) {

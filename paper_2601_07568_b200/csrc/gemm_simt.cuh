@@ -152,24 +152,38 @@ __global__ void __launch_bounds__(THREADS) gemm_simt_small_kernel(const T* __res
   float acc[OUT];
 #pragma unroll
   for (int i = 0; i < OUT; ++i) acc[i] = 0.f;
-  for (int k0 = 0; k0 < K; k0 += KC) {
-    auto stage = [&](float* dst, const T* src, int row, int rows, int k) {
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (row < rows && k < K) {
-        if constexpr (sizeof(T) == 4) {
-          v = *reinterpret_cast<const float4*>(src + static_cast<size_t>(row) * K + k);
-        } else {
-          const uint2 w = *reinterpret_cast<const uint2*>(src + static_cast<size_t>(row) * K + k);
-          v = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
-        }
+  // A thread's pieces of the next KC columns are requested before the products of the present ones.
+  constexpr int XN = BM_ * (KC / 4), WN = BN_ * (KC / 4), XP = (XN + THREADS - 1) / THREADS, WP = WN / THREADS;
+  static_assert(WN % THREADS == 0 && (XN % THREADS == 0 || XN < THREADS), "pieces deal out evenly");
+  float4 xv[XP], wv[WP];
+  auto piece = [&](const T* src, int row, int rows, int k) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row < rows && k < K) {
+      if constexpr (sizeof(T) == 4) {
+        v = *reinterpret_cast<const float4*>(src + static_cast<size_t>(row) * K + k);
+      } else {
+        const uint2 w = *reinterpret_cast<const uint2*>(src + static_cast<size_t>(row) * K + k);
+        v = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
       }
-      *reinterpret_cast<float4*>(dst) = v;
-    };
-#pragma unroll 4
-    for (int e = t; e < BM_ * (KC / 4); e += THREADS) stage(&Xs[e / (KC / 4)][e % (KC / 4) * 4], X, m0 + e / (KC / 4), M, k0 + e % (KC / 4) * 4);
-#pragma unroll 4
-    for (int e = t; e < BN_ * (KC / 4); e += THREADS) stage(&Ws[e / (KC / 4)][e % (KC / 4) * 4], W, n0 + e / (KC / 4), N, k0 + e % (KC / 4) * 4);
+    }
+    return v;
+  };
+  auto request = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < XP; ++i)
+      if (XN >= THREADS || t < XN) xv[i] = piece(X, m0 + (t + i * THREADS) / (KC / 4), M, k0 + (t + i * THREADS) % (KC / 4) * 4);
+#pragma unroll
+    for (int i = 0; i < WP; ++i) wv[i] = piece(W, n0 + (t + i * THREADS) / (KC / 4), N, k0 + (t + i * THREADS) % (KC / 4) * 4);
+  };
+  request(0);
+  for (int k0 = 0; k0 < K; k0 += KC) {
+#pragma unroll
+    for (int i = 0; i < XP; ++i)
+      if (XN >= THREADS || t < XN) *reinterpret_cast<float4*>(&Xs[(t + i * THREADS) / (KC / 4)][(t + i * THREADS) % (KC / 4) * 4]) = xv[i];
+#pragma unroll
+    for (int i = 0; i < WP; ++i) *reinterpret_cast<float4*>(&Ws[(t + i * THREADS) / (KC / 4)][(t + i * THREADS) % (KC / 4) * 4]) = wv[i];
     __syncthreads();
+    if (k0 + KC < K) request(k0 + KC);
     // (up to the last column in whole slabs of the other kernel, the same bits: 1 x 5842 x 4 takes 5.2 us, all KC of them 10.4)
     const int columns = min(KC, (K - k0 + BK - 1) / BK * BK);
 #pragma unroll 1
