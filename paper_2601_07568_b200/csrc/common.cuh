@@ -41,6 +41,7 @@ struct EpiParams {
   const float* ssq_in = nullptr; // any epilogue but EPI_RESID: chunk sums of the operand rows
   int ssq_chunks = 0;
   float inv_k = 0.f, rms_eps = 0.f;
+  const float* norm_gain = nullptr;  // gemm_simt_small_kernel on fp32: RMSNorm of the operand rows with these gains, on their way in
   // EPI_STATS with temperature sampling (sample_part != nullptr): per (row, 128-column tile) also the
   // largest perturbed logit l + temperature * g (g standard Gumbel noise), the index attaining it
   // (lowest on ties) and the unperturbed logit there.  The noise of row m is keyed by

@@ -1196,21 +1196,35 @@ int run_linear_tc(d3_ctx* c, const void* X, const void* W, int M, int N, int K, 
   return run_linear_tc_bn<128, 1>(c, X, W, M, N, K, epi, ep, ctas_hint, qx, w_tiled);
 }
 
+// Fewer 32 x 128 tiles than half the SMs: small tiles (same bits).  A statistic belongs to 128 columns.
+bool simt_small(const d3_ctx* c, const void* x, const void* w, int M, int N, int K, size_t esz) {
+  const long long tiles = static_cast<long long>((N + simt::BN - 1) / simt::BN) * ((M + simt::BM - 1) / simt::BM);
+  return K % 4 == 0 && reinterpret_cast<uintptr_t>(x) % (4 * esz) == 0 && reinterpret_cast<uintptr_t>(w) % (4 * esz) == 0 && tiles * 2 <= c->n_sms;
+}
 template <typename T, int EPI>
 int launch_simt(d3_ctx* c, const T* x, const T* w, int M, int N, int K, const EpiParams& ep) {
   const dim3 grid((N + simt::BN - 1) / simt::BN, (M + simt::BM - 1) / simt::BM);
-  // Fewer 32 x 128 tiles than half the SMs: small tiles (same bits).  A statistic belongs to 128 columns.
-  const bool vec = K % 4 == 0 && reinterpret_cast<uintptr_t>(x) % (4 * sizeof(T)) == 0 && reinterpret_cast<uintptr_t>(w) % (4 * sizeof(T)) == 0;
-  if (vec && grid.x * grid.y * 2 <= static_cast<unsigned>(c->n_sms)) {
+  if (simt_small(c, x, w, M, N, K, sizeof(T))) {
     if constexpr (EPI == EPI_STATS)
-      CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<T, EPI, 4, 128, 64>, dim3(grid.x, (M + 3) / 4), dim3(simt::THREADS), 0, x, w, M, N, K, ep));
+      CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<T, EPI, 4, 128, 64>, dim3(grid.x, (M + 3) / 4), dim3(simt::THREADS), 0, x, w, M, N, K, ep, simt::SimtQkv{}));
     else
-      CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<T, EPI, 16, 16, 256>, dim3((N + 15) / 16, (M + 15) / 16), dim3(simt::THREADS), 0, x, w, M, N, K, ep));
+      CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<T, EPI, 16, 16, 256>, dim3((N + 15) / 16, (M + 15) / 16), dim3(simt::THREADS), 0, x, w, M, N, K, ep, simt::SimtQkv{}));
     LAUNCHED(c, "gemm_simt_small_kernel");
     return D3_OK;
   }
   CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_kernel<T, EPI>, grid, dim3(simt::THREADS), 0, x, w, M, N, K, ep));
   LAUNCHED(c, "gemm_simt_kernel");
+  return D3_OK;
+}
+// QKV of an fp32 model on small tiles, rotated and stored by the matmul's epilogue.
+int run_simt_qkv(d3_ctx* c, const void* X, const void* W, int M, int N, int K, const EpiParams& ep, const QkvExtra& qx) {
+  ProfScope ps(c, D3_PROF_GEMM_QKV);
+  const d3_config& g = c->cfg;
+  const simt::SimtQkv q{static_cast<float*>(qx.k_cache), static_cast<float*>(qx.v_cache), c->rope_cos, c->rope_sin, qx.rm.pos_base, qx.rm.n_valid,
+                        qx.rm.rows_per_seq, g.n_q_heads, g.n_kv_heads, g.d_head, g.max_seq, c->error_word};
+  CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<float, EPI_QKV, 16, 16, 256>, dim3((N + 15) / 16, (M + 15) / 16), dim3(simt::THREADS), 0,
+                         static_cast<const float*>(X), static_cast<const float*>(W), M, N, K, ep, q));
+  LAUNCHED(c, "gemm_simt_small_kernel");
   return D3_OK;
 }
 template <typename T>
@@ -1584,6 +1598,18 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   // their accumulator rows; the matmuls that update the residual stream refresh the copy and the
   // chunk sums of squares.
   const void* normed = c->fold_norm ? c->xb : c->xn;
+  // fp32: a matmul on small tiles takes the rows in front of the norm and normalises its own few of them.
+  auto norm_first = [&](const float* gain, const void* w, int N, EpiParams& ep) -> int {
+    if (c->fold_norm) return D3_OK;
+    if (!c->is_bf16 && !c->use_tc && simt_small(c, c->x, w, M, N, d, sizeof(float))) {
+      ep.norm_gain = gain;
+      ep.rms_eps = g.rms_eps;
+      normed = c->x;
+      return D3_OK;
+    }
+    normed = c->xn;
+    return run_rmsnorm(c, c->x, gain, c->xn, M);
+  };
   auto after_norm = [&](EpiParams& ep) {
     if (!c->fold_norm) return;
     ep.ssq_in = c->ssq; ep.ssq_chunks = (d + 31) / 32; ep.inv_k = 1.0f / static_cast<float>(d); ep.rms_eps = g.rms_eps;
@@ -1697,15 +1723,19 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   for (int l = 0; l < g.n_layers; ++l) {
     if (l == c->tap_layer && M <= c->tap_rows)
       CUDA_TRY(c, cudaMemcpyAsync(c->tap_in, c->x, sizeof(float) * M * d, cudaMemcpyDeviceToDevice, c->stream));
-    if (!c->fold_norm) TRY(run_rmsnorm(c, c->x, c->attn_norm[l], c->xn, M));
     if (c->fuse_qkv) {
       EpiParams ep;
+      TRY(norm_first(c->attn_norm[l], c->wqkv[l], nq + 2 * nkv, ep));
       ep.y = c->q; ep.ldy = nq;
       after_norm(ep);
       QkvExtra qx{rm, k_plane(c, l), v_plane(c, l)};
       TRY(run_linear(c, normed, c->wqkv[l], M, nq + 2 * nkv, d, EPI_QKV, ep, 0, &qx, D3_PROF_GEMM_QKV, c->w_tiled));
+    } else if (EpiParams ep; !c->is_bf16 && !c->use_tc && simt_small(c, c->x, c->wqkv[l], M, nq + 2 * nkv, d, sizeof(float))) {
+      TRY(norm_first(c->attn_norm[l], c->wqkv[l], nq + 2 * nkv, ep));
+      ep.y = c->q; ep.ldy = nq;
+      TRY(run_simt_qkv(c, normed, c->wqkv[l], M, nq + 2 * nkv, d, ep, QkvExtra{rm, k_plane(c, l), v_plane(c, l)}));
     } else {
-      EpiParams ep;
+      TRY(norm_first(c->attn_norm[l], c->wqkv[l], nq + 2 * nkv, ep));
       ep.y = c->qkv_f32; ep.ldy = nq + 2 * nkv;
       after_norm(ep);
       TRY(run_linear(c, normed, c->wqkv[l], M, nq + 2 * nkv, d, EPI_F32, ep, 0, nullptr, D3_PROF_GEMM_QKV, c->w_tiled));
@@ -1723,9 +1753,9 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
       updates_resid(ep);
       TRY(run_linear(c, c->o, c->wo[l], M, d, nq, EPI_RESID, ep, 0, nullptr, D3_PROF_GEMM_O, c->w_tiled));
     }
-    if (!c->fold_norm) TRY(run_rmsnorm(c, c->x, c->ffn_norm[l], c->xn, M));
     {
       EpiParams ep;
+      TRY(norm_first(c->ffn_norm[l], c->wgu[l], 2 * f, ep));
       ep.y = c->h; ep.ldy = f;
       after_norm(ep);
       TRY(run_linear(c, normed, c->wgu[l], M, 2 * f, d, EPI_SWIGLU, ep, 0, nullptr, D3_PROF_GEMM_GATE_UP, c->w_tiled));
@@ -1740,14 +1770,18 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
       CUDA_TRY(c, cudaMemcpyAsync(c->tap_out, c->x, sizeof(float) * M * d, cudaMemcpyDeviceToDevice, c->stream));
   }
   if (head == 0) return D3_OK;
-  if (!c->fold_norm) TRY(run_rmsnorm(c, c->x, c->final_norm, c->xn, M));
   if (head == 1) {
     c->stat_fused = false;
-    if (!head_sk) TRY(run_linear(c, normed, c->lm_head, M, g.vocab, d, EPI_STATS, head_epi(), 0, nullptr, D3_PROF_GEMM_HEAD, c->w_tiled));
+    if (!head_sk) {
+      EpiParams ep = head_epi();
+      TRY(norm_first(c->final_norm, c->lm_head, g.vocab, ep));
+      TRY(run_linear(c, normed, c->lm_head, M, g.vocab, d, EPI_STATS, ep, 0, nullptr, D3_PROF_GEMM_HEAD, c->w_tiled));
+    }
     TRY(run_stats_merge(c, M, (g.vocab + 127) / 128, c->conf, c->ent, c->argmax, c->temperature > 0.f));
   } else {
     EpiParams ep;
     ep.y = logits; ep.ldy = g.vocab; ep.scale = g.logit_scale;
+    TRY(norm_first(c->final_norm, c->lm_head, g.vocab, ep));
     after_norm(ep);
     TRY(run_linear(c, normed, c->lm_head, M, g.vocab, d, EPI_F32, ep, 0, nullptr, D3_PROF_GEMM_HEAD, c->w_tiled));
   }

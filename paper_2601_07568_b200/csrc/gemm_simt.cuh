@@ -84,6 +84,45 @@ __device__ __forceinline__ void simt_epilogue(const float (*Cs)[BN_ + 1], int m0
   }
 }
 
+// EPI_QKV on small fp32 tiles: what rope_kv_kernel does with the projected rows, from the tile (its columns 2k and 2k + 1 of a
+// q or k head are the dims k and k + d_head / 2).  A launch fewer per layer.
+struct SimtQkv {
+  float *k_cache, *v_cache;  // this layer's planes
+  const float *rope_cos, *rope_sin;
+  const int *pos_base, *n_valid;
+  int rows_per_seq, hq, hkv, dh, max_seq;
+  uint32_t* error_word;
+};
+template <int BM_, int BN_>
+__device__ __forceinline__ void simt_qkv_epilogue(const float (*Cs)[BN_ + 1], int m0, int n0, int M, int N, const EpiParams& ep, const SimtQkv& q) {
+  const int half = q.dh / 2;
+  for (int e = threadIdx.x; e < BM_ * (BN_ / 2); e += THREADS) {
+    const int r = e / (BN_ / 2), c = e % (BN_ / 2) * 2, m = m0 + r, n = n0 + c;
+    if (m >= M || n >= N) continue;
+    const int b = m / q.rows_per_seq, row = m - b * q.rows_per_seq;
+    if (row >= q.n_valid[b]) continue;
+    const int pos = q.pos_base[b] + row;
+    if (pos < 0 || pos >= q.max_seq) {
+      if (n == 0) atomicOr(q.error_word, ERRW_BAD_POSITION);
+      continue;
+    }
+    const int head = n / q.dh, d = n - head * q.dh;
+    const float x = Cs[r][c], y = Cs[r][c + 1];
+    if (head >= q.hq + q.hkv) {  // a v head keeps its order
+      float* dst = q.v_cache + ((static_cast<size_t>(b) * q.hkv + (head - q.hq - q.hkv)) * q.max_seq + pos) * q.dh + d;
+      dst[0] = x;
+      dst[1] = y;
+      continue;
+    }
+    const int k = d >> 1;
+    const float co = q.rope_cos[static_cast<size_t>(pos) * half + k], si = q.rope_sin[static_cast<size_t>(pos) * half + k];
+    float* dst = head < q.hq ? static_cast<float*>(ep.y) + static_cast<size_t>(m) * ep.ldy + head * q.dh
+                             : q.k_cache + ((static_cast<size_t>(b) * q.hkv + (head - q.hq)) * q.max_seq + pos) * q.dh;
+    dst[k] = x * co - y * si;
+    dst[k + half] = y * co + x * si;
+  }
+}
+
 template <typename T, int EPI>
 __global__ void __launch_bounds__(THREADS) gemm_simt_kernel(const T* __restrict__ X, const T* __restrict__ W, int M,
                                                             int N, int K, EpiParams ep) {
@@ -139,8 +178,10 @@ __global__ void __launch_bounds__(THREADS) gemm_simt_kernel(const T* __restrict_
 // would leave most SMs idle: BM_ x BN_ tiles, 256 threads, KC columns of X and W in shared memory at a time, read four at
 // a time.  What bounds it is the chain of K multiply-adds and, per KC columns, one trip to memory.  A 16 x 128 x 512
 // product took 50 us as one 32 x 128 tile on one SM; as 8 tiles of 16 x 16 it takes 6.  K % 4 == 0, rows aligned to 4 elements.
+// With ep.norm_gain the rows of X are those in front of an RMSNorm: every block works out the factors of its few rows (the bits
+// of rmsnorm_kernel) while its first columns are on their way; a launch for them took 3 us of a tiny model's 100 a forward, five times.
 template <typename T, int EPI, int BM_, int BN_, int KC>
-__global__ void __launch_bounds__(THREADS) gemm_simt_small_kernel(const T* __restrict__ X, const T* __restrict__ W, int M, int N, int K, EpiParams ep) {
+__global__ void __launch_bounds__(THREADS) gemm_simt_small_kernel(const T* __restrict__ X, const T* __restrict__ W, int M, int N, int K, EpiParams ep, const SimtQkv qkv) {
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
   constexpr int OUT = BM_ * BN_ / THREADS, ROWS = THREADS / BN_;
@@ -176,7 +217,39 @@ __global__ void __launch_bounds__(THREADS) gemm_simt_small_kernel(const T* __res
     for (int i = 0; i < WP; ++i) wv[i] = piece(W, n0 + (t + i * THREADS) / (KC / 4), N, k0 + (t + i * THREADS) % (KC / 4) * 4);
   };
   request(0);
+  __shared__ float rstd[BM_];
+  const bool norm = sizeof(T) == 4 && ep.norm_gain != nullptr;
+  if (norm) {
+    const int lane = t & 31, n4 = K >> 2;
+    for (int r = t >> 5; r < BM_; r += THREADS / 32) {
+      const float4* row = reinterpret_cast<const float4*>(X + static_cast<size_t>(min(m0 + r, M - 1)) * K);
+      float tot = 0.f;
+      for (int w = 0; w < 8 && w * 32 < n4; ++w) {  // what warp w of rmsnorm_kernel adds up
+        float ss = 0.f;
+        for (int i = w * 32 + lane; i < n4; i += 256) {
+          const float4 v = row[i];
+          ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        tot += ss;
+      }
+      if (lane == 0) rstd[r] = rsqrtf(tot / static_cast<float>(K) + ep.rms_eps);
+    }
+    __syncthreads();
+  }
   for (int k0 = 0; k0 < K; k0 += KC) {
+    if (norm) {
+#pragma unroll
+      for (int i = 0; i < XP; ++i) {
+        const int e = t + i * THREADS, k = k0 + e % (KC / 4) * 4;
+        if ((XN >= THREADS || t < XN) && k < K) {
+          const float f = rstd[e / (KC / 4)];
+          const float4 g = *reinterpret_cast<const float4*>(ep.norm_gain + k);
+          xv[i] = make_float4(xv[i].x * f * g.x, xv[i].y * f * g.y, xv[i].z * f * g.z, xv[i].w * f * g.w);
+        }
+      }
+    }
 #pragma unroll
     for (int i = 0; i < XP; ++i)
       if (XN >= THREADS || t < XN) *reinterpret_cast<float4*>(&Xs[(t + i * THREADS) / (KC / 4)][(t + i * THREADS) % (KC / 4) * 4]) = xv[i];
@@ -206,7 +279,8 @@ __global__ void __launch_bounds__(THREADS) gemm_simt_small_kernel(const T* __res
 #pragma unroll
   for (int i = 0; i < OUT; ++i) Cs[r0 + i * ROWS][c] = acc[i];
   __syncthreads();
-  simt_epilogue<T, EPI, BM_, BN_>(Cs, m0, n0, M, N, ep);
+  if constexpr (EPI == EPI_QKV) simt_qkv_epilogue<BM_, BN_>(Cs, m0, n0, M, N, ep, qkv);
+  else simt_epilogue<T, EPI, BM_, BN_>(Cs, m0, n0, M, N, ep);
 }
 
 }  // namespace simt

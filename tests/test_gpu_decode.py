@@ -147,6 +147,27 @@ def test_c1_logits_fp32(c1):
     assert rel.max() <= 1e-4, rel.max()
 
 
+@pytest.mark.parametrize("d_model,hq,hkv,d_head,lens", [(1032, 3, 1, 64, [21, 40]), (128, 4, 4, 32, [1]), (264, 2, 2, 128, [5, 0, 17]), (8, 1, 1, 32, [33]), (2056, 2, 1, 32, [7])])
+def test_fp32_norms_and_rotation_inside_the_matmuls(d_model, hq, hkv, d_head, lens):
+    """Small fp32 matmuls normalise their operand rows themselves and QKV stores the rotated heads: rows of more than 1024
+    and of 8 columns, columns that are no multiple of a tile's 256, rows that are no multiple of 16, ragged prompts."""
+    shape = si.scaled_shape(si.TINY, name="tiny-widths", n_layers=2, d_model=d_model, n_q_heads=hq, n_kv_heads=hkv, d_ffn=64, vocab=130, d_head=d_head)
+    W, bs = si.gen_weights(shape), len(lens)
+    model = o.model_from_shape(shape, W, np.float64)
+    ids = np.random.default_rng(d_model).integers(0, shape.vocab - 2, size=(bs, max(lens))).astype(np.int32)
+    blk = np.full((bs, 8), shape.mask_id, dtype=np.int32)
+    blk[:, 3] = 17
+    with Ctx(shape, W, block=8, max_batch=bs, max_seq=max(lens) + 8) as ctx:
+        n0 = d3.d3_launch_count_of(ctx.ctx, "rmsnorm_kernel") + d3.d3_launch_count_of(ctx.ctx, "rope_kv_kernel")
+        ctx.prefill(ids, np.array(lens, dtype=np.int32))
+        got = ctx.logits(blk)
+        assert d3.d3_launch_count_of(ctx.ctx, "rmsnorm_kernel") + d3.d3_launch_count_of(ctx.ctx, "rope_kv_kernel") == n0
+        for b, n in enumerate(lens):
+            ref = model.denoise_forward(model.prefill(ids[b, :n]), blk[b])[0]
+            assert np.max(np.abs(got[b] - ref)) <= 1e-4 * np.max(np.abs(ref))  # the bound of the tiny model's logits above
+        assert ctx.error_word() == 0
+
+
 @pytest.mark.parametrize("tau", [0.9, 0.3, 0.29])
 def test_c1_step_locked(c1, tau):
     w, model, ids, lens, ctx = c1
