@@ -289,10 +289,11 @@ def test_c2_full_size_sampling_refresh_and_multiblock(llada_weights):
 
 def test_c2_full_size_windows_of_two_and_four_blocks(llada_weights):
     """The 64-row forward of two segments (the form in which d3_generate runs a block's finalize forward
-    together with the next block's first step) and the 128-row round of four segments (multi-block
-    decoding) at the full 8B shape: a tapped layer is recomputed by the oracle segment by segment from
-    the GPU's own inputs (segment k sees the prefix and segments 0..k-1 as the same forward wrote them),
-    and the statistics of the last layer's rows are compared with the oracle's."""
+    together with the next block's first step), on either of the two schedules that take it, and the
+    128-row round of four segments (multi-block decoding) at the full 8B shape: a tapped layer is
+    recomputed by the oracle segment by segment from the GPU's own inputs (segment k sees the prefix and
+    segments 0..k-1 as the same forward wrote them), and the statistics of the last layer's rows are
+    compared with the oracle's."""
     w = si.WORKLOADS["c2"]
     shape = w.model
     ids, lens = si.gen_prompts(w)
@@ -301,7 +302,10 @@ def test_c2_full_size_windows_of_two_and_four_blocks(llada_weights):
     report = {}
     rng = np.random.default_rng(11)
     with Ctx(shape, llada_weights, block=B, max_batch=4, max_seq=w.max_seq, max_prefill_rows=w.prompt_max) as ctx:
-        for n_win in (2, 4):
+        # by default every decode forward of this model is launches of resident pairs; one of up to 64 rows can be asked for as a chain
+        for n_win, clusters in ((2, 0), (4, 0), (2, 64)):
+            d3.d3_set_tuning(ctx.ctx, chain_clusters=clusters)
+            tag = f"win{n_win}" + (":chain" if clusters else "")
             # segment 0 complete (random real tokens), later segments progressively more masked
             blocks = []
             for k in range(n_win):
@@ -315,7 +319,10 @@ def test_c2_full_size_windows_of_two_and_four_blocks(llada_weights):
                 conf = torch.empty(R, dtype=torch.float32, device=DEV)
                 ent = torch.empty_like(conf)
                 am = torch.empty(R, dtype=torch.int32, device=DEV)
+                before = [d3.d3_launch_count_of(ctx.ctx, name) for name in ("gemm_sk_kernel", "chain_kernel")]
                 d3.d3_denoise_window(ctx.ctx, win, n_win, conf, ent, am)
+                ran = [d3.d3_launch_count_of(ctx.ctx, name) > n for name, n in zip(("gemm_sk_kernel", "chain_kernel"), before)]
+                assert ran == [clusters == 0, clusters > 0], (tag, ran)
                 x_in = torch.empty((R, d), dtype=torch.float32, device=DEV)
                 x_out = torch.empty_like(x_in)
                 d3.d3_read_tap(ctx.ctx, x_in, x_out, R)
@@ -333,19 +340,18 @@ def test_c2_full_size_windows_of_two_and_four_blocks(llada_weights):
                     err = float(np.max(np.abs(upd_got - upd_ref)) / np.max(np.abs(upd_ref)))
                     kerr = float(np.max(np.abs(k_all[seen:seen + B] - k_rows)) / np.max(np.abs(k_rows)))
                     verr = float(np.max(np.abs(v_all[seen:seen + B] - v_rows)) / np.max(np.abs(v_rows)))
-                    report[f"win{n_win}:layer{layer}:seg{k}"] = [err, kerr, verr]
-                    assert err <= 3e-2 and kerr <= 3e-2 and verr <= 3e-2, (n_win, layer, k, err, kerr, verr)
+                    report[f"{tag}:layer{layer}:seg{k}"] = [err, kerr, verr]
+                    assert err <= 3e-2 and kerr <= 3e-2 and verr <= 3e-2, (tag, layer, k, err, kerr, verr)
                     if layer == shape.n_layers - 1:
                         lg = model.logits(x_out[rows].astype(np.float32))
                         _, o_conf, o_tok, _ = o.softmax_stats(lg, shape.mask_id)
                         gap = top2_gap(lg, shape.mask_id)
                         g_conf, g_tok = conf.cpu().numpy()[rows], am.cpu().numpy()[rows]
                         serr = float(np.max(np.abs(g_conf - o_conf)))
-                        report[f"win{n_win}:stat_err:seg{k}"] = serr
+                        report[f"{tag}:stat_err:seg{k}"] = serr
                         assert serr <= 5e-2
                         assert not ((g_tok != o_tok) & (gap > 2 * serr + EPS)).any()
             assert ctx.error_word() == 0
-        # which kernels ran: the 64-row forward as a chain launch, the 128-row one on the per-matmul kernels
         assert d3.d3_launch_count_of(ctx.ctx, "chain_kernel") > 0
     record_report("fullsize_c2_windows", report)
 
