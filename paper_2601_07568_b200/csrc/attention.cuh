@@ -57,8 +57,10 @@ __global__ void __launch_bounds__(THREADS) attn_simt_kernel(const T* __restrict_
       Vs[j][d] = in ? TypeOps<T>::to_f(vb[static_cast<size_t>(j0 + j) * DH + d]) : 0.f;
     }
     __syncthreads();
-    // A warp's rows side by side and the keys unrolled (the sums of a row in the same order as one row and one key at a time):
-    // what bounds it is the chain of dependent instructions.  (Rows that do not exist are computed and not written.)
+    // Scores of a warp's rows side by side (what bounds them is the chain of dependent instructions), their values a row at a
+    // time: the sums of a row are in the same order either way.  Both by rows, both side by side and this, us for 4 heads x 16
+    // rows on fp32: d_head 32, 300 keys 29.4, 39.5, 20.8, 2000 keys 160, 230, 101; d_head 64, 2000 keys 392, 410, 297;
+    // d_head 128, 2000 keys 287, 233, 228.  (Rows that do not exist are computed and not written.)
     float sc[RPW], pr[RPW];
 #pragma unroll
     for (int i = 0; i < RPW; ++i) sc[i] = 0.f;
@@ -80,10 +82,9 @@ __global__ void __launch_bounds__(THREADS) attn_simt_kernel(const T* __restrict_
 #pragma unroll
       for (int d = 0; d < DPL; ++d) acc[i][d] *= corr;
     }
-#pragma unroll 16
-    for (int j = 0; j < KC; ++j)
 #pragma unroll
-      for (int i = 0; i < RPW; ++i) {
+    for (int i = 0; i < RPW; ++i)
+      for (int j = 0; j < KC; ++j) {
         const float pj = __shfl_sync(0xffffffffu, pr[i], j);
 #pragma unroll
         for (int d = 0; d < DPL; ++d) acc[i][d] = fmaf(pj, Vs[j][lane + 32 * d], acc[i][d]);
