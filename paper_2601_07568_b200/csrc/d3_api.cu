@@ -1201,17 +1201,26 @@ bool simt_small(const d3_ctx* c, const void* x, const void* w, int M, int N, int
   const long long tiles = static_cast<long long>((N + simt::BN - 1) / simt::BN) * ((M + simt::BM - 1) / simt::BM);
   return K % 4 == 0 && reinterpret_cast<uintptr_t>(x) % (4 * esz) == 0 && reinterpret_cast<uintptr_t>(w) % (4 * esz) == 0 && tiles * 2 <= c->n_sms;
 }
+template <typename T, int EPI, int BM, int BN, int KC>
+int launch_simt_small(d3_ctx* c, const T* x, const T* w, int M, int N, int K, const EpiParams& ep, const simt::SimtQkv& q) {
+  const dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
+  if constexpr (sizeof(T) == 4 && (EPI == EPI_QKV || EPI == EPI_SWIGLU || EPI == EPI_STATS || EPI == EPI_F32))
+    if (ep.norm_gain != nullptr) {
+      CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<T, EPI, BM, BN, KC, true>, grid, dim3(simt::THREADS), 0, x, w, M, N, K, ep, q));
+      LAUNCHED(c, "gemm_simt_small_kernel");
+      return D3_OK;
+    }
+  CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<T, EPI, BM, BN, KC, false>, grid, dim3(simt::THREADS), 0, x, w, M, N, K, ep, q));
+  LAUNCHED(c, "gemm_simt_small_kernel");
+  return D3_OK;
+}
 template <typename T, int EPI>
 int launch_simt(d3_ctx* c, const T* x, const T* w, int M, int N, int K, const EpiParams& ep) {
-  const dim3 grid((N + simt::BN - 1) / simt::BN, (M + simt::BM - 1) / simt::BM);
   if (simt_small(c, x, w, M, N, K, sizeof(T))) {
-    if constexpr (EPI == EPI_STATS)
-      CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<T, EPI, 4, 128, 64>, dim3(grid.x, (M + 3) / 4), dim3(simt::THREADS), 0, x, w, M, N, K, ep, simt::SimtQkv{}));
-    else
-      CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<T, EPI, 16, 16, 256>, dim3((N + 15) / 16, (M + 15) / 16), dim3(simt::THREADS), 0, x, w, M, N, K, ep, simt::SimtQkv{}));
-    LAUNCHED(c, "gemm_simt_small_kernel");
-    return D3_OK;
+    if constexpr (EPI == EPI_STATS) return launch_simt_small<T, EPI, 4, 128, 64>(c, x, w, M, N, K, ep, simt::SimtQkv{});
+    else return launch_simt_small<T, EPI, 16, 16, 256>(c, x, w, M, N, K, ep, simt::SimtQkv{});
   }
+  const dim3 grid((N + simt::BN - 1) / simt::BN, (M + simt::BM - 1) / simt::BM);
   CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_kernel<T, EPI>, grid, dim3(simt::THREADS), 0, x, w, M, N, K, ep));
   LAUNCHED(c, "gemm_simt_kernel");
   return D3_OK;
@@ -1222,10 +1231,7 @@ int run_simt_qkv(d3_ctx* c, const void* X, const void* W, int M, int N, int K, c
   const d3_config& g = c->cfg;
   const simt::SimtQkv q{static_cast<float*>(qx.k_cache), static_cast<float*>(qx.v_cache), c->rope_cos, c->rope_sin, qx.rm.pos_base, qx.rm.n_valid,
                         qx.rm.rows_per_seq, g.n_q_heads, g.n_kv_heads, g.d_head, g.max_seq, c->error_word};
-  CUDA_TRY(c, launch_pdl(c, simt::gemm_simt_small_kernel<float, EPI_QKV, 16, 16, 256>, dim3((N + 15) / 16, (M + 15) / 16), dim3(simt::THREADS), 0,
-                         static_cast<const float*>(X), static_cast<const float*>(W), M, N, K, ep, q));
-  LAUNCHED(c, "gemm_simt_small_kernel");
-  return D3_OK;
+  return launch_simt_small<float, EPI_QKV, 16, 16, 256>(c, static_cast<const float*>(X), static_cast<const float*>(W), M, N, K, ep, q);
 }
 template <typename T>
 int run_linear_simt(d3_ctx* c, const void* X, const void* W, int M, int N, int K, int epi, const EpiParams& ep) {

@@ -178,9 +178,10 @@ __global__ void __launch_bounds__(THREADS) gemm_simt_kernel(const T* __restrict_
 // would leave most SMs idle: BM_ x BN_ tiles, 256 threads, KC columns of X and W in shared memory at a time, read four at
 // a time.  What bounds it is the chain of K multiply-adds and, per KC columns, one trip to memory.  A 16 x 128 x 512
 // product took 50 us as one 32 x 128 tile on one SM; as 8 tiles of 16 x 16 it takes 6.  K % 4 == 0, rows aligned to 4 elements.
-// With ep.norm_gain the rows of X are those in front of an RMSNorm: every block works out the factors of its few rows (the bits
-// of rmsnorm_kernel) while its first columns are on their way; a launch for them took 3 us of a tiny model's 100 a forward, five times.
-template <typename T, int EPI, int BM_, int BN_, int KC>
+// NORM (fp32): the rows of X are those in front of an RMSNorm with the gains ep.norm_gain; every block works out the factors of
+// its few rows (the bits of rmsnorm_kernel) while its first columns are on their way.  (An instance of its own: with the norm as a
+// branch the LM head without one took 26.1 us instead of 22.9 at 4 x 9000 x 1024 and 15.8 instead of 14.2 at 16 x 2000 x 512.)
+template <typename T, int EPI, int BM_, int BN_, int KC, bool NORM>
 __global__ void __launch_bounds__(THREADS) gemm_simt_small_kernel(const T* __restrict__ X, const T* __restrict__ W, int M, int N, int K, EpiParams ep, const SimtQkv qkv) {
   ptx::grid_dep_wait();
   ptx::grid_dep_launch();
@@ -217,9 +218,8 @@ __global__ void __launch_bounds__(THREADS) gemm_simt_small_kernel(const T* __res
     for (int i = 0; i < WP; ++i) wv[i] = piece(W, n0 + (t + i * THREADS) / (KC / 4), N, k0 + (t + i * THREADS) % (KC / 4) * 4);
   };
   request(0);
-  __shared__ float rstd[BM_];
-  const bool norm = sizeof(T) == 4 && ep.norm_gain != nullptr;
-  if (norm) {
+  __shared__ float rstd[NORM ? BM_ : 1];
+  if constexpr (NORM) {
     const int lane = t & 31, n4 = K >> 2;
     for (int r = t >> 5; r < BM_; r += THREADS / 32) {
       const float4* row = reinterpret_cast<const float4*>(X + static_cast<size_t>(min(m0 + r, M - 1)) * K);
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(THREADS) gemm_simt_small_kernel(const T* __res
     __syncthreads();
   }
   for (int k0 = 0; k0 < K; k0 += KC) {
-    if (norm) {
+    if constexpr (NORM) {
 #pragma unroll
       for (int i = 0; i < XP; ++i) {
         const int e = t + i * THREADS, k = k0 + e % (KC / 4) * 4;
