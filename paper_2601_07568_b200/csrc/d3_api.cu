@@ -1201,6 +1201,11 @@ bool simt_small(const d3_ctx* c, const void* x, const void* w, int M, int N, int
   const long long tiles = static_cast<long long>((N + simt::BN - 1) / simt::BN) * ((M + simt::BM - 1) / simt::BM);
   return K % 4 == 0 && reinterpret_cast<uintptr_t>(x) % (4 * esz) == 0 && reinterpret_cast<uintptr_t>(w) % (4 * esz) == 0 && tiles * 2 <= c->n_sms;
 }
+// fp32 norms inside the small matmuls: up to 256 columns.  A block adds up its rows one chunk of 128 columns after the other, which
+// the launch that it saves pays for in short rows only.  us a layer, 16 / 64 rows, inside against rmsnorm_kernel: 31.1 / 38.4
+// against 32.8 / 39.5 at d_model 128, 36.6 / 49.7 against 36.7 / 53.5 at 256, but 42.6 / 55.8 against 40.6 / 58.7 at 320, 55.4 / 93.7
+// against 49.5 / 83.7 at 512, 106 / 212 against 103 / 193 at 1024, and a head of 4000 columns at 1024 98 / 133 against 74 / 117.
+constexpr int SIMT_NORM_COLUMNS = 256;
 template <typename T, int EPI, int BM, int BN, int KC>
 int launch_simt_small(d3_ctx* c, const T* x, const T* w, int M, int N, int K, const EpiParams& ep, const simt::SimtQkv& q) {
   const dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
@@ -1604,10 +1609,10 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   // their accumulator rows; the matmuls that update the residual stream refresh the copy and the
   // chunk sums of squares.
   const void* normed = c->fold_norm ? c->xb : c->xn;
-  // fp32: a matmul on small tiles takes the rows in front of the norm and normalises its own few of them.
+  // fp32: a matmul on small tiles takes the rows in front of the norm and normalises its own few of them, up to 256 columns.
   auto norm_first = [&](const float* gain, const void* w, int N, EpiParams& ep) -> int {
     if (c->fold_norm) return D3_OK;
-    if (!c->is_bf16 && !c->use_tc && simt_small(c, c->x, w, M, N, d, sizeof(float))) {
+    if (!c->is_bf16 && !c->use_tc && d <= SIMT_NORM_COLUMNS && simt_small(c, c->x, w, M, N, d, sizeof(float))) {
       ep.norm_gain = gain;
       ep.rms_eps = g.rms_eps;
       normed = c->x;

@@ -149,8 +149,8 @@ def test_c1_logits_fp32(c1):
 
 @pytest.mark.parametrize("d_model,hq,hkv,d_head,lens", [(1032, 3, 1, 64, [21, 40]), (128, 4, 4, 32, [1]), (264, 2, 2, 128, [5, 0, 17]), (8, 1, 1, 32, [33]), (2056, 2, 1, 32, [7])])
 def test_fp32_norms_and_rotation_inside_the_matmuls(d_model, hq, hkv, d_head, lens):
-    """Small fp32 matmuls normalise their operand rows themselves and QKV stores the rotated heads: rows of more than 1024
-    and of 8 columns, columns that are no multiple of a tile's 256, rows that are no multiple of 16, ragged prompts."""
+    """Small fp32 matmuls normalise their operand rows themselves (up to 256 columns) and QKV stores the rotated heads: rows of
+    more than 1024 and of 8 columns, columns that are no multiple of a tile's 256, rows that are no multiple of 16, ragged prompts."""
     shape = si.scaled_shape(si.TINY, name="tiny-widths", n_layers=2, d_model=d_model, n_q_heads=hq, n_kv_heads=hkv, d_ffn=64, vocab=130, d_head=d_head)
     W, bs = si.gen_weights(shape), len(lens)
     model = o.model_from_shape(shape, W, np.float64)
@@ -158,14 +158,40 @@ def test_fp32_norms_and_rotation_inside_the_matmuls(d_model, hq, hkv, d_head, le
     blk = np.full((bs, 8), shape.mask_id, dtype=np.int32)
     blk[:, 3] = 17
     with Ctx(shape, W, block=8, max_batch=bs, max_seq=max(lens) + 8) as ctx:
-        n0 = d3.d3_launch_count_of(ctx.ctx, "rmsnorm_kernel") + d3.d3_launch_count_of(ctx.ctx, "rope_kv_kernel")
         ctx.prefill(ids, np.array(lens, dtype=np.int32))
         got = ctx.logits(blk)
-        assert d3.d3_launch_count_of(ctx.ctx, "rmsnorm_kernel") + d3.d3_launch_count_of(ctx.ctx, "rope_kv_kernel") == n0
+        assert d3.d3_launch_count_of(ctx.ctx, "rope_kv_kernel") == 0
+        assert (d3.d3_launch_count_of(ctx.ctx, "rmsnorm_kernel") == 0) == (d_model <= 256)
         for b, n in enumerate(lens):
             ref = model.denoise_forward(model.prefill(ids[b, :n]), blk[b])[0]
             assert np.max(np.abs(got[b] - ref)) <= 1e-4 * np.max(np.abs(ref))  # the bound of the tiny model's logits above
         assert ctx.error_word() == 0
+
+
+@pytest.mark.parametrize("d_model,heads,d_head", [(128, 4, 32), (256, 4, 64), (264, 3, 64)])
+def test_fp32_bits_do_not_depend_on_the_batch(d_model, heads, d_head):
+    """One sequence alone (norms and rotation inside the small matmuls, up to 256 columns) and among forty (rmsnorm_kernel,
+    rope_kv_kernel and the 32 x 128 tiles): its logits and its stored keys and values bit for bit, with gains of all sizes."""
+    shape = si.scaled_shape(si.TINY, name="tiny-batch", n_layers=2, d_model=d_model, n_q_heads=heads, n_kv_heads=heads, d_ffn=576, vocab=1000, d_head=d_head)
+    W, rng = si.gen_weights(shape), np.random.default_rng(d_model)
+    gain = lambda: rng.uniform(0.25, 2.0, d_model).astype(np.float32)
+    W = {**W, "final_norm": gain(), "layers": {l: dict(W["layers"][l], attn_norm=gain(), ffn_norm=gain()) for l in range(2)}}
+    bs, B, n = 40, 32, 21
+    ids = rng.integers(0, shape.vocab - 2, size=(bs, n)).astype(np.int32)
+    blk = rng.integers(0, shape.vocab - 2, size=(bs, B)).astype(np.int32)
+    out, norms = [], []
+    for seqs in (1, bs):
+        with Ctx(shape, W, block=B, max_batch=bs, max_seq=n + B, max_prefill_rows=bs * n) as ctx:
+            ctx.prefill(ids[:seqs], np.full(seqs, n, dtype=np.int32))
+            lg = ctx.logits(blk[:seqs])[0]
+            kv = torch.zeros(2, heads, n + B, d_head, device=DEV)
+            d3.d3_read_kv(ctx.ctx, 1, 0, 0, n + B, kv[0], kv[1])
+            torch.cuda.synchronize()
+            out.append((lg, kv.cpu().numpy()))
+            norms.append([d3.d3_launch_count_of(ctx.ctx, name) > 0 for name in ("rmsnorm_kernel", "rope_kv_kernel", "gemm_simt_kernel")])
+            assert ctx.error_word() == 0
+    assert norms == [[d_model > 256, False, False], [True, True, True]]
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
 
 @pytest.mark.parametrize("tau", [0.9, 0.3, 0.29])
