@@ -1230,7 +1230,13 @@ int launch_simt(d3_ctx* c, const T* x, const T* w, int M, int N, int K, const Ep
   LAUNCHED(c, "gemm_simt_kernel");
   return D3_OK;
 }
-// QKV of an fp32 model on small tiles, rotated and stored by the matmul's epilogue.
+// QKV of an fp32 model on small tiles, rotated and stored by the matmul's epilogue: where its tiles are resident at once (three
+// blocks an SM).  Behind more than one wave the epilogue is not hidden any more: 1152 tiles at d_model 2048 took 143 us where the
+// matmul and rope_kv_kernel take 132 and 10 and overlap with what is around them (a layer 776 against 730); at 576 to 864 tiles the
+// two are level, at 432 (d_model 768, 96 rows) a layer gains 2 %, at d_model 128 15 %.
+bool simt_qkv_fused(const d3_ctx* c, const void* w, int M, int N, int K) {
+  return simt_small(c, c->x, w, M, N, K, sizeof(float)) && static_cast<long long>((N + 15) / 16) * ((M + 15) / 16) <= 3ll * c->n_sms;
+}
 int run_simt_qkv(d3_ctx* c, const void* X, const void* W, int M, int N, int K, const EpiParams& ep, const QkvExtra& qx) {
   ProfScope ps(c, D3_PROF_GEMM_QKV);
   const d3_config& g = c->cfg;
@@ -1741,7 +1747,7 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
       after_norm(ep);
       QkvExtra qx{rm, k_plane(c, l), v_plane(c, l)};
       TRY(run_linear(c, normed, c->wqkv[l], M, nq + 2 * nkv, d, EPI_QKV, ep, 0, &qx, D3_PROF_GEMM_QKV, c->w_tiled));
-    } else if (EpiParams ep; !c->is_bf16 && !c->use_tc && simt_small(c, c->x, c->wqkv[l], M, nq + 2 * nkv, d, sizeof(float))) {
+    } else if (EpiParams ep; !c->is_bf16 && !c->use_tc && simt_qkv_fused(c, c->wqkv[l], M, nq + 2 * nkv, d)) {
       TRY(norm_first(c->attn_norm[l], c->wqkv[l], nq + 2 * nkv, ep));
       ep.y = c->q; ep.ldy = nq;
       TRY(run_simt_qkv(c, normed, c->wqkv[l], M, nq + 2 * nkv, d, ep, QkvExtra{rm, k_plane(c, l), v_plane(c, l)}));
