@@ -147,10 +147,12 @@ def test_c1_logits_fp32(c1):
     assert rel.max() <= 1e-4, rel.max()
 
 
-@pytest.mark.parametrize("d_model,hq,hkv,d_head,lens", [(1032, 3, 1, 64, [21, 40]), (128, 4, 4, 32, [1]), (264, 2, 2, 128, [5, 0, 17]), (8, 1, 1, 32, [33]), (2056, 2, 1, 32, [7])])
+@pytest.mark.parametrize("d_model,hq,hkv,d_head,lens", [(1032, 3, 1, 64, [21, 40]), (128, 4, 4, 32, [1]), (264, 2, 2, 128, [5, 0, 17]), (8, 1, 1, 32, [33]), (2056, 2, 1, 32, [7]),
+                                                             (64, 16, 16, 64, [32, 7, 30])])
 def test_fp32_norms_and_rotation_inside_the_matmuls(d_model, hq, hkv, d_head, lens):
     """Small fp32 matmuls normalise their operand rows themselves (up to 256 columns) and QKV stores the rotated heads: rows of
-    more than 1024 and of 8 columns, columns that are no multiple of a tile's 256, rows that are no multiple of 16, ragged prompts."""
+    more than 1024 and of 8 columns, columns that are no multiple of a tile's 256, rows that are no multiple of 16, ragged prompts;
+    prompts whose QKV has more tiles than one wave (1152) go through rope_kv_kernel, the block behind them (384) does not."""
     shape = si.scaled_shape(si.TINY, name="tiny-widths", n_layers=2, d_model=d_model, n_q_heads=hq, n_kv_heads=hkv, d_ffn=64, vocab=130, d_head=d_head)
     W, bs = si.gen_weights(shape), len(lens)
     model = o.model_from_shape(shape, W, np.float64)
@@ -160,7 +162,9 @@ def test_fp32_norms_and_rotation_inside_the_matmuls(d_model, hq, hkv, d_head, le
     with Ctx(shape, W, block=8, max_batch=bs, max_seq=max(lens) + 8) as ctx:
         ctx.prefill(ids, np.array(lens, dtype=np.int32))
         got = ctx.logits(blk)
-        assert d3.d3_launch_count_of(ctx.ctx, "rope_kv_kernel") == 0
+        wave, columns = 3 * torch.cuda.get_device_properties(0).multi_processor_count, (hq + 2 * hkv) * d_head // 16
+        rotated_apart = sum(columns * ((rows + 15) // 16) > wave for rows in (bs * max(lens), bs * 8))
+        assert d3.d3_launch_count_of(ctx.ctx, "rope_kv_kernel") == shape.n_layers * rotated_apart and (rotated_apart > 0) == (d_model == 64)
         assert (d3.d3_launch_count_of(ctx.ctx, "rmsnorm_kernel") == 0) == (d_model <= 256)
         for b, n in enumerate(lens):
             ref = model.denoise_forward(model.prefill(ids[b, :n]), blk[b])[0]
@@ -777,13 +781,14 @@ def test_decode_batches_by_width_and_rows(d_model, bs, on_pairs):
 def test_whole_gate_up_tiles_of_resident_pairs(d_model, d_ffn, bs):
     """Gate/up of more 256-row tiles than pairs: 76 (none cut, some pairs have two) and 85 (74 whole ones behind the exchange
     of 11 cut ones), at 32, 96, 192 and 288 rows (two tiles of 160 rows of X, the last 32 of them without any).  The logits
-    of the plain bf16 kernels."""
+    of the plain bf16 kernels, and a layer's update row by row."""
     shape = dataclasses.replace(si.scaled_shape(si.LLADA8B, name="small-wide-ffn", n_layers=2, d_model=d_model, n_q_heads=2, n_kv_heads=2,
                                                 d_ffn=d_ffn, vocab=1024, d_head=128), logit_scale=10.0)
     W = si.gen_weights(shape)
     ids = np.random.default_rng(d_ffn + bs).integers(0, shape.vocab - 2, size=(bs, 50)).astype(np.int32)
     blk = np.full((bs, 32), shape.mask_id, dtype=np.int32)
-    lg = []
+    tokens = np.random.default_rng(bs).integers(0, shape.vocab - 2, size=(bs, 32)).astype(np.int32)
+    lg, update = [], []
     for impl in (0, 1):
         with Ctx(shape, W, block=32, max_batch=bs, max_seq=96, gemm_impl=impl) as ctx:
             ctx.prefill(ids, np.full(bs, 50, dtype=np.int32))
@@ -791,9 +796,18 @@ def test_whole_gate_up_tiles_of_resident_pairs(d_model, d_ffn, bs):
                 d3.d3_set_tuning(ctx.ctx, chain=0)
             n0 = d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel")
             lg.append(ctx.logits(blk))
+            d3.d3_set_tap(ctx.ctx, 0)
+            ctx.logits(tokens)
+            x = torch.empty(2, bs * 32, shape.d_model, dtype=torch.float32, device=DEV)
+            d3.d3_read_tap(ctx.ctx, x[0], x[1], bs * 32)
+            torch.cuda.synchronize()
+            update.append((x[1] - x[0]).cpu().numpy())
             assert (d3.d3_launch_count_of(ctx.ctx, "gemm_sk_kernel") > n0) == (impl == 0)
             assert ctx.error_word() == 0
     assert np.max(np.abs(lg[0] - lg[1])) <= 3e-2 * np.max(np.abs(lg[1]))  # two schedules of one forward, as above
+    # layer 0 begins with the same bits: its update differs by the bf16 roundings on the way (normed rows twice, q, k, v, o, h: at
+    # most 2^-9 each, about 2^-10 in the 2-norm, on either side); a row of X that is left out is off by all of it
+    assert np.all(np.linalg.norm(update[0] - update[1], axis=1) <= 1e-2 * np.linalg.norm(update[1], axis=1))
 
 
 @pytest.mark.parametrize("d_model,lens,p_max", [(256, [300], 1024), (256, [1], 1300), (256, [0], 700), (384, [300, 0, 256], 512), (256, [1024], 1024)])

@@ -165,11 +165,12 @@ def test_linear_fp32_small_tiles_same_bits(ctx_f32, m, n, k, epi):
 
 
 @pytest.mark.parametrize("m,n,k", [(1, 256, 64), (32, 512, 4096), (33, 3584, 3584), (96, 256, 8192), (128, 12288, 512), (129, 4096, 1024),
-                                   (200, 768, 2048), (256, 4096, 4096), (257, 1280, 1920), (501, 3584, 1024), (640, 19200, 256)])
+                                   (200, 768, 2048), (256, 4096, 4096), (257, 1280, 1920), (501, 3584, 1024), (640, 19200, 256),
+                                   (96, 19456, 256), (288, 21760, 1024)])
 def test_linear_bf16_k_cut_pairs(ctx_bf16, m, n, k):
     """Weights as the row operand of CTA pairs with the tiles of an incomplete wave cut along K: one tile and no cut,
-    one tile shared by all pairs, ranges that touch two tiles, a whole wave followed by cut tiles (640 x 19200), one
-    to three tiles of rows, row counts on both sides of a multiple of 16, 32 and 256; fp32, residual, bf16 and SwiGLU
+    one tile shared by all pairs, ranges that touch two tiles, a whole wave behind cut tiles (640 x 19200, 288 x 21760), a
+    wave and two tiles none of which is cut (96 x 19456), one to three tiles of rows, row counts on both sides of a multiple of 16, 32 and 256; fp32, residual, bf16 and SwiGLU
     epilogues against the fp64 product (bounds as in the other matmul tests), twice with the same bits."""
     rng = np.random.default_rng(m + n + k)
     xt, x = rand_bf16(rng, (m, k))
