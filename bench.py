@@ -289,20 +289,13 @@ def profiled_request(ctx, w, ids_dev, lens_dev, out_dev, mode):
     return prof, st, d3.d3_launch_count_of(ctx, "forward_rows") - rows0
 
 
-def matmul_totals(shape, prof, forwards, rows, fused_rows):
-    """Matmul launches of a profiled request, those inside chain launches left out: (ms, launches, bytes, flops).  Forwards
-    that ran as a chain, where not all did, are those with `fused_rows` rows."""
+def matmul_totals(shape, prof, forwards, rows):
+    """Matmul launches of a profiled request of `forwards` forwards over `rows` rows in all: (ms, launches, bytes, flops)."""
     layer_keys = ("gemm_qkv", "gemm_o", "gemm_gate_up", "gemm_down")
     keys = layer_keys + ("gemm_head", "gemm_other")
-    chained = min(prof["chain"]["launches"], forwards)
-    own = forwards - chained
-    rows_chained = rows if own == 0 else chained * fused_rows
-    tot_bytes = tot_flops = 0
-    for n, m, layers in ((own, (rows - rows_chained) / max(own, 1), shape.n_layers), (chained, rows_chained / max(chained, 1), 0)):
-        gb, gf = gemm_bytes(shape, m), gemm_flops(shape, m)
-        tot_bytes += n * (layers * sum(gb[k] for k in layer_keys) + gb["gemm_head"])
-        tot_flops += n * (layers * sum(gf[k] for k in layer_keys) + gf["gemm_head"])
-    return sum(prof[k]["ms"] for k in keys), sum(prof[k]["launches"] for k in keys), tot_bytes, tot_flops
+    totals = [forwards * (shape.n_layers * sum(t[k] for k in layer_keys) + t["gemm_head"])
+              for t in (fn(shape, rows / max(forwards, 1)) for fn in (gemm_bytes, gemm_flops))]
+    return sum(prof[k]["ms"] for k in keys), sum(prof[k]["launches"] for k in keys), *totals
 
 
 def measure_batched(name, W, dev, local, world, dist, peaks, steps):
@@ -362,7 +355,7 @@ def measure_batched(name, W, dev, local, world, dist, peaks, steps):
     d3.d3_destroy(ctx)
     tokens = w.batch * w.gen_len
     gf = gemm_flops(shape, rows / max(st_prof.steps, 1))
-    tot_ms, n_gemm, _, tot_flops = matmul_totals(shape, prof, st_prof.steps, rows, 2 * w.batch * w.block)
+    tot_ms, n_gemm, _, tot_flops = matmul_totals(shape, prof, st_prof.steps, rows)
     ms_step = ms_total / steps
     ms_fwd = (ms_step - ms_prefill) / max(st.steps, 1)
     layer_keys = ("gemm_qkv", "gemm_o", "gemm_gate_up", "gemm_down")
@@ -549,21 +542,9 @@ def run_ours(args):
     layer_keys = ("gemm_qkv", "gemm_o", "gemm_gate_up", "gemm_down")
     # K/V read by the attention of one forward at mid-generation
     kv_mid = 2 * shape.n_layers * shape.n_kv_heads * shape.d_head * 2 * sum(int(l) + w.gen_len // 2 for l in lens_np)
-    tot_ms, n_dom, tot_bytes, tot_flops = matmul_totals(shape, prof, st_prof.steps, prof_rows, 2 * w.batch * w.block)
-    chain = prof["chain"]
-    if chain["ms"] > tot_ms:
-        # most decode forwards run their layers as one launch (chain_kernel): matmuls of all layers and attention
-        dominant = "chain_kernel (all layers of a decode forward: QKV, attention, O-proj, gate/up, down)"
-        m = prof_rows / st_prof.steps if chain["launches"] >= st_prof.steps else 2 * w.batch * w.block
-        bm, fm = gemm_bytes(shape, m), gemm_flops(shape, m)
-        tot_bytes = (sum(bm[k] for k in layer_keys) * shape.n_layers + kv_mid) * chain["launches"]
-        tot_flops = sum(fm[k] for k in layer_keys) * shape.n_layers * chain["launches"]
-        tot_ms, n_dom = chain["ms"], chain["launches"]
-        traffic_kernel = "chain_kernel"
-    else:
-        dominant = ("gemm_sk_kernel (O-proj, gate/up, down and the next layer's QKV or the LM head in a launch) and the other matmul launches of "
-                    "the decode loop as it makes them; CUDA events around every launch, which keep it from overlapping the next")
-        traffic_kernel = "gemm_sk_kernel"
+    tot_ms, n_dom, tot_bytes, tot_flops = matmul_totals(shape, prof, st_prof.steps, prof_rows)
+    dominant = ("gemm_sk_kernel (O-proj, gate/up, down and the next layer's QKV or the LM head in a launch) and the other matmul launches of "
+                "the decode loop as it makes them; CUDA events around every launch, which keep it from overlapping the next")
     hbm_bound = tot_flops / max(tot_bytes, 1) < peaks["bf16_tflops_sustained"] * 1e12 / (peaks["hbm_gbs"] * 1e9)
     if hbm_bound:
         achieved = tot_bytes / (tot_ms / 1e3) / 1e9 if tot_ms > 0 else 0.0
@@ -583,7 +564,7 @@ def run_ours(args):
                                   "frac_of_8TBs_nominal": fwd_bytes / (ms_fwd / 1e3) / 1e9 / 8000.0,
                                   "frac_of_measured_tensor": fwd_flops / (ms_fwd / 1e3) / 1e12 / peaks["bf16_tflops_sustained"],
                                   "ms_per_forward": ms_fwd, "bytes_per_forward": fwd_bytes}
-    cap = ncu_traffic(traffic_kernel, w.name) if hbm_bound else None
+    cap = ncu_traffic("gemm_sk_kernel", w.name) if hbm_bound else None
     if cap is not None and n_dom > 0:
         # the capture ran the model cut to a few layers: a forward's traffic and launches grow in proportion to them; per launch
         per_forward = float(cap["bytes_per_layer"]) * shape.n_layers + float(cap.get("bytes_fixed", 0.0))

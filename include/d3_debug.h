@@ -35,10 +35,12 @@ typedef struct d3_tuning {
   int32_t strip_stages;     /* explicit pipeline depth of the column-strip kernel, 0 = from ring_kb.  With two
                                issue pipelines every stage belongs to one pipeline, which takes an even
                                count: an odd one is refused (D3_ERR_UNSUPPORTED at the launch), not rounded */
-  int32_t chain;            /* decode forwards of up to 64 rows run the matmuls between two attention kernels
-                               as one persistent launch: -1 = when the shapes allow (default), 0 never */
+  int32_t chain;            /* decode forwards of up to 64 rows run the matmuls and attention of all layers as one
+                               persistent launch: -1 = when the shapes allow and a layer has less than 200 MB of
+                               weights (default), 0 never */
   int32_t chain_clusters;   /* clusters of four CTAs the chain launches use: 0 = as many as are resident at once
-                               (default); a smaller count is taken as given, a larger one is cut to that */
+                               (default); a smaller count is taken as given, a larger one is cut to that.  With a count
+                               the chain also takes models of larger layers */
   int32_t chain_l2_ahead;   /* weight slabs the chain's L2 prefetch warp runs ahead of the ring: -1 = default
                                (0: no prefetch; measured neutral at 12 slabs and slower beyond), at most 256 */
   int32_t weights_as_rows;  /* matmuls of 129..256 rows with at most one 128-column tile per SM run with the weights as the

@@ -22,7 +22,7 @@ enum : int {
   EPI_RESID = 2,   // y fp32 [m, n] += acc
   EPI_SWIGLU = 3,  // y T [m, n/2]: columns come in groups of 128 = 64 gate then 64 up
   EPI_STATS = 4,   // per (row, 128-column tile): (max, sum exp, sum exp*(l-max), argmax) of scale*acc
-  EPI_QKV = 5,     // RoPE on q and k heads (d_head = 128 = one tile), q -> y T, k/v -> cache
+  EPI_QKV = 5,     // RoPE on q and k heads, q -> y T, k/v -> cache (tensor-core kernels: d_head = 128 = one tile; fp32: any)
 };
 
 struct EpiParams {

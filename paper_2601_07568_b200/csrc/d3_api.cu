@@ -1538,10 +1538,13 @@ int run_stats_merge(d3_ctx* c, int M, int n_tiles, float* conf, float* ent, int*
 }
 
 // Forwards whose matmuls run on gemm_sk_kernel (those that the chain does not take): up to 640 rows.  Measured, ms per
-// decode forward of sequences with 128..400 stored positions, one kernel per matmul against this: 8B shape 4.48 -> 4.07
-// at 128 rows, 6.40 -> 5.37 at 256, 9.80 -> 8.37 at 384, 10.46 -> 10.04 at 512, 12.57 -> 12.46 at 640, but 13.31 -> 13.55 at
-// 768 and 16.77 -> 17.76 at 1024 (tiles of an incomplete wave weigh less there, and whole tiles that go through L2 more);
-// 7B shape 6.18 -> 3.63 at 128, 5.91 -> 4.95 at 256, 9.54 -> 8.42 at 512, 11.73 -> 11.41 at 640.  Layers of other widths,
+// decode forward of sequences with 128..400 stored positions, one kernel per matmul against this, when the line was drawn: 8B
+// shape 4.48 -> 4.07 at 128 rows, 6.40 -> 5.37 at 256, 9.80 -> 8.37 at 384, 10.46 -> 10.04 at 512, 12.57 -> 12.46 at 640, but 13.31 ->
+// 13.55 at 768 and 16.77 -> 17.76 at 1024; 7B shape 6.18 -> 3.63 at 128, 5.91 -> 4.95 at 256, 9.54 -> 8.42 at 512, 11.73 -> 11.41 at 640.
+// With both kernels as they are, us a layer with prefixes of 264: 8B 141 -> 117 at 128, 193 -> 145 at 256, 270 -> 198 at 384, 284 -> 263
+// at 512, 347 -> 332 at 640, 351 -> 346 at 704, 370 -> 359 at 768, 439 -> 410 at 864, 463 -> 464 at 1024; 7B 223 -> 123, 202 -> 148, 291 -> 198,
+// 308 -> 251, 375 -> 321, 374 -> 344, 388 -> 348, 447 -> 387, 454 -> 442: up to the line nothing is slower here, beyond it to
+// 864 rows one kernel per matmul has become the slower one (prompts without their padding need it, see pack_usable).  Layers of other widths,
 // this against one kernel per matmul (smallest and largest ratio of times at 96..640 rows): d_model 256 0.68-0.95, 768
 // 0.62-0.81 (to 192 rows), 1024 0.68-0.87, 1536 0.59-0.81, 2048 0.54-0.86, 3072 0.56-0.88.  Only a K of 512 falls out: there
 // the eight slabs that a CTA of gemm_tc_kernel gets are whole tiles and nothing is exchanged, 0.98-1.22 up to 128 rows,
@@ -1653,16 +1656,18 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
     return ep;
   };
   // Forwards of up to 64 rows (the chain takes no more): with large layers the launches of resident pairs, all SMs instead of the
-  // 132 that clusters of four leave, make up for attention between them.  Measured, ms per 32-row forward, chain against this:
-  // 3.46 -> 3.37 at the 8B shape (436 MB a layer), 2.51 -> 2.40 at d_model 3072 (245 MB), but 1.84 -> 1.88 at 2048 (109 MB) and
-  // 1.38 -> 1.54 at 1024.  33 to 64 rows at the 8B shape: a request whose finished blocks share their forward with the next
-  // block's first step 116.9 -> 116.0, one with windows of 64 and 128 rows 66.0 -> 63.8; at d_model 2048 48 rows gain 10 % and 64
-  // rows lose 3, at 1024 the chain is ahead by 7-27 %.
+  // 132 that clusters of four leave, make up for attention between them.  Measured, us a layer, chain against this, for a block
+  // of 32, 48 and 64 rows and a window of two blocks of 32, prefixes of 350: 8B shape (436 MB a layer) 103.2 -> 101.0, 114.5 -> 103.3,
+  // 117.9 -> 111.0, 116.9 -> 113.6; d_model 3584 (312 MB) 86.2 -> 84.1, 97.4 -> 85.4, 100.0 -> 93.5, 100.3 -> 96.1; 3072 (226 MB) 74.1 ->
+  // 68.0, 81.7 -> 78.2, 84.7 -> 77.9, 84.4 -> 80.5; 2048 (103 MB) 53.3 -> 53.9, 60.3 -> 54.5, 62.7 -> 61.8, 62.7 -> 64.7.  (At 2560 and
+  // 2816, 159 and 193 MB, this is ahead by 5-20 %, at 1024 the chain by 7-27 %: the two cross somewhere below the line.  The sums
+  // of the two are cut at different places: keys and values of such a forward differ by bf16 roundings from one to the other.)
   const bool large_layers = static_cast<double>(nq + 2 * nkv + nq + 3.0 * f) * d * c->esz >= 200e6;
   const bool pairs_first = M <= 64 && large_layers && c->tune_chain < 0 && c->tune_chain_clusters == 0 && sk_forward_usable(c, M);
   const bool chain = !pairs_first && chain_usable(c, bs, rows_per_seq, seg);
   // The LM head is the last matmul of the last layer's launch.  (Behind the chain it stays a launch of its own on 128-row tiles,
-  // whose weights are on their way while the chain drains: 3.79 ms a 64-row forward against 3.83.)
+  // whose weights are on their way while the chain drains: a 64-row forward of the 8B shape, when that ran on the chain, took
+  // 3.79 ms so and 3.83 with the head on the pairs.)
   const bool head_sk = head == 1 && !chain && sk_forward_usable(c, M) && sk_shape_ok(g.vocab, d);
 
   if (chain) {

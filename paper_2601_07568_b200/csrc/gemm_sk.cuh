@@ -11,21 +11,23 @@
 // ranges, a range touches at most two tiles, and the partial accumulators meet in global memory (L2).  What a pair
 // moves per slab is 16 KB of weights and half of X per CTA, where a lone CTA would stage all of X.
 //
-// Reduction.  A CTA leaves its accumulators in global memory (L2) as [row of X][128 columns] fp32, gives the tensor
-// memory back, raises the tile's counter (release), waits until all contributors have, and finishes an equal share of
+// Reduction.  A CTA leaves its accumulators of a cut tile in global memory (L2) as [row of X][128 columns] fp32, gives the
+// tensor memory back, raises the tile's counter (release), waits until all contributors have, and finishes its share of
 // the rows: the partials added in contributor order (fixed order: the same bits on every run).  All CTAs of the launch
 // are resident at once (the host sizes the grid by the occupancy of clusters) and every range ends at about the same
-// time, so the wait is short.  It is bounded like every other one.
+// time, so the wait is short.  It is bounded like every other one.  Cut tiles come first, and the whole ones behind them
+// hide the exchange (SkPlan).
 //
-// Epilogue.  A warp finishes whole rows of X, four columns a lane, three or four rows at a time: all that they need
-// (partials, residual values, cosines) is requested at once, because behind the last MMA of a matmul every trip to L2 is
+// Epilogue.  Whole gate/up tiles are finished from tensor memory (swiglu_tile); whole tiles of the other matmuls go through
+// global memory like a partial.  From there a warp finishes whole rows of X, four columns a lane, three or four rows at a
+// time: all that they need (partials, residual values, cosines) is requested at once, because behind the last MMA of a matmul every trip to L2 is
 // on the critical path and takes one to two microseconds beside the next matmul's weights.  Row factors of the folded
 // RMSNorm are worked out while the MMAs run, everything that needs an integer division before the launch's dependencies
 // are there.  (Forms that were slower, microseconds for O-proj, gate/up, down and QKV of the 8B shape at 128 / 256 rows:
 // an output column a lane and sixteen rows unrolled 148 / 190, with the row factors fetched where they are used 108 /
-// 139; this one 100 / 128.  Their weights alone take 67 at the measured copy bandwidth, and the MMA loops add up to 72;
-// the rest is the exchange at the end of each matmul, 7 to 9 microseconds.  Holding the next matmul's weights back until
-// the exchange is over costs 3 to 6.)
+// 139.  With whole tiles in front 107 / 139, as it is 102 / 128, CUDA events around the launch.  Their weights alone take 67
+// at the measured copy bandwidth; the rest is mostly the exchanges of the cut tiles, where no whole tile follows to hide
+// them (O-proj, down, QKV).  Holding the next matmul's weights back until the exchange is over costs 3 to 6.)
 //
 // Borders.  A launch runs up to four matmuls in order (O-proj, gate/up, down, the next layer's QKV or the LM head); the next one
 // reads what the one before wrote on other SMs, so there is a grid-wide counter between them, as in the chain

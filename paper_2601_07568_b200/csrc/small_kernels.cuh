@@ -908,9 +908,11 @@ __global__ void trajectory_rank_kernel(const int* __restrict__ commit_step, int 
 }
 // The same with four positions a lane and all loads of 512 positions in flight: block sizes that are a power of two from 4
 // to 128, 16-byte aligned rows.  Bound by memory (8 bytes a position); a warp per 32-thread block that waits for every
-// decoding block's load in turn takes 22 us for 16384 x 256 positions, this one 8.
+// decoding block's load in turn takes 18.5 us for 16384 x 240 positions that are in L2 and 26.8 for positions that are not, this
+// one 5.2 and 7.6 for 16384 x 256.  A dependent launch, as the one below: as plain launches 6.3 and 10.3, the two together 14.5 and
+// 20.6 instead of 11.3 and 16.8.
 __global__ void __launch_bounds__(256) trajectory_rank4_kernel(const int* __restrict__ commit_step, int bs, int gen_len, int B, int* __restrict__ rank) {
-  ptx::grid_dep_wait();  // (dependent launches, here and below: the gap between two kernels of 6 us each is a fifth of the pair)
+  ptx::grid_dep_wait();
   ptx::grid_dep_launch();
   const int b = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (b >= bs) return;  // warp-uniform
@@ -966,7 +968,8 @@ __global__ void noisy_sequence_kernel(const int* __restrict__ y, const int* __re
 }
 
 // The same with four positions a thread over the whole batch (n a multiple of 4, 16-byte aligned rows), loading only what
-// the result depends on: 16384 x 256 positions in 8 us, with one position a thread in 16.
+// the result depends on: 16384 x 256 positions in 6.0 us where they are in L2 and 9.7 where they are not (8.3 and 12.1 as a plain
+// launch; one position a thread took 16).
 __global__ void __launch_bounds__(256) noisy_sequence4_kernel(const int4* __restrict__ y, const int4* __restrict__ rank, const int* __restrict__ s_arr,
                                                               const int* __restrict__ k_arr, const int* __restrict__ m_arr, int bs, int n4, int mask_id,
                                                               int4* __restrict__ out) {
