@@ -1659,7 +1659,8 @@ int forward(d3_ctx* c, const int* ids, int bs, int rows_per_seq, int head, float
   // 132 that clusters of four leave, make up for attention between them.  Measured, us a layer, chain against this, for a block
   // of 32, 48 and 64 rows and a window of two blocks of 32, prefixes of 350: 8B shape (436 MB a layer) 103.2 -> 101.0, 114.5 -> 103.3,
   // 117.9 -> 111.0, 116.9 -> 113.6; d_model 3584 (312 MB) 86.2 -> 84.1, 97.4 -> 85.4, 100.0 -> 93.5, 100.3 -> 96.1; 3072 (226 MB) 74.1 ->
-  // 68.0, 81.7 -> 78.2, 84.7 -> 77.9, 84.4 -> 80.5; 2048 (103 MB) 53.3 -> 53.9, 60.3 -> 54.5, 62.7 -> 61.8, 62.7 -> 64.7.  (At 2560 and
+  // 68.0, 81.7 -> 78.2, 84.7 -> 77.9, 84.4 -> 80.5; 2048 (103 MB) 53.3 -> 53.9, 60.3 -> 54.5, 62.7 -> 61.8, 62.7 -> 64.7.
+  // Grouped heads, two blocks of 32 and four of 16: d_model 4096 109.3 -> 106.7 and 106.7 -> 103.5, 3072 83.5 -> 84.0 and 83.6 -> 74.3.  (At 2560 and
   // 2816, 159 and 193 MB, this is ahead by 5-20 %, at 1024 the chain by 7-27 %: the two cross somewhere below the line.  The sums
   // of the two are cut at different places: keys and values of such a forward differ by bf16 roundings from one to the other.)
   const bool large_layers = static_cast<double>(nq + 2 * nkv + nq + 3.0 * f) * d * c->esz >= 200e6;
